@@ -184,47 +184,6 @@ __device__ __forceinline__ bool mbar_wait2_warp(uint64_t* a, uint32_t pa, uint64
   return __all_sync(0xffffffffu, ok);
 }
 
-// One lane of the warp, the same one for every call with all lanes active.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t r;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
-  return r != 0;
-}
-
-// The two 32-bit words of a 128-byte-swizzle shared-memory descriptor: the
-// low word holds start address >> 4 (bits 0..13) and LBO >> 4 (bits
-// 16..29), the high word SBO >> 4, the descriptor version (bit 46) and the
-// swizzle mode (bits 61..63). Shared addresses stay below 2^18 bytes, so
-// adding an offset >> 4 to a low word never carries into the LBO field.
-__host__ __device__ constexpr uint32_t sw128_lo_lbo(uint32_t lbo) { return ((lbo >> 4) & 0x3FFFu) << 16; }
-__host__ __device__ constexpr uint32_t sw128_hi(uint32_t sbo) {
-  return ((sbo >> 4) & 0x3FFFu) | (1u << 14) | (2u << 29);
-}
-
-// tcgen05.mma kind::f16, A and B from shared memory, descriptors given as words
-__device__ __forceinline__ void umma_bf16_w(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
-                                            uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "setp.ne.b32 p, %5, 0;\n\t"
-      "mov.b64 da, {%1, %3};\n\t"
-      "mov.b64 db, {%2, %3};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc)
-      : "memory");
-}
-// the same with A from tensor memory
-__device__ __forceinline__ void umma_bf16_tmem_a_w(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi,
-                                                   uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
-      "setp.ne.b32 p, %5, 0;\n\t"
-      "mov.b64 db, {%2, %3};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc)
-      : "memory");
-}
-
 // The largest of three floats in one instruction (three-input max.f32). A
 // maximum is exact, so grouping the row's values by threes gives the same
 // result as any other order.
@@ -470,7 +429,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
 #pragma unroll
         for (int k = 0; k < HD / 16; ++k) {
           const uint32_t off = static_cast<uint32_t>((k >> 2) * BOX_BYTES + (k & 3) * 32) >> 4;
-          umma_bf16_w(tmem + 128u * i, a + off, b + off, hi, idesc_s, k > 0 ? 1u : 0u);
+          umma_f16_w(tmem + 128u * i, a + off, b + off, hi, idesc_s, k > 0 ? 1u : 0u);
         }
         umma_commit(&s_full[i]);
       }
@@ -484,7 +443,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
         const uint32_t b = v_lo + static_cast<uint32_t>(vst) * TILE16;
 #pragma unroll
         for (int k = 0; k < BKV / 16; ++k)
-          umma_bf16_tmem_a_w(tmem + 256u + 128u * i, tmem + 128u * i + 8u * k, b + ((k * 2048) >> 4), hi, idesc_o,
+          umma_f16_tmem_a_w(tmem + 256u + 128u * i, tmem + 128u * i + 8u * k, b + ((k * 2048) >> 4), hi, idesc_o,
                              (acc || k > 0) ? 1u : 0u);
         if (last) umma_commit(&o_done[i]);
       }

@@ -306,8 +306,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && leader) {
-      // ---------------- MMA issuer (even CTA)
+    if (leader) {
+      // ---------------- MMA issuer (even CTA): the whole warp walks the
+      // schedule and waits, one elected lane issues
+      const bool issuer = elect_one();
+      const uint32_t a_lo = (smem_u32(smem) >> 4) + sw128_lo_lbo(16);
+      constexpr uint32_t hi = sw128_hi(1024);
+      const uint32_t idesc = p.idesc;
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
@@ -316,45 +321,45 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       WorkIter it(sc, cid, ncl, kblocks, split_k);
       Work w;
       while (ok && it.next(w)) {
-        if (!mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 2)) break;
+        if (!mbar_wait_warp(&tempty[acc], acc_phase ^ 1u, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 2)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem + static_cast<uint32_t>(acc * PN);
         for (int kb = w.k0; kb < w.k1; ++kb) {
-          if (!mbar_wait(&full[stage], phase, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 3)) {
+          if (!mbar_wait_warp(&full[stage], phase, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 3)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a_base = smem_u32(smem + stage * STAGE_BYTES);
-          const uint32_t b_base = a_base + HALF_BYTES;
+          if (issuer) {
+            const uint32_t a = a_lo + static_cast<uint32_t>(stage) * (STAGE_BYTES >> 4);
+            const uint32_t b = a + (HALF_BYTES >> 4);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t ad = sw128_desc(a_base + k * 32, 16, 1024);
-            const uint64_t bd = sw128_desc(b_base + k * 32, 16, 1024);
-            if (FP8)
-              umma_f8_pair(d_tmem, ad, bd, p.idesc, (kb > w.k0 || k > 0) ? 1u : 0u);
-            else
-              umma_f16_pair(d_tmem, ad, bd, p.idesc, (kb > w.k0 || k > 0) ? 1u : 0u);
+            for (int k = 0; k < BK / 16; ++k)
+              umma_pair_w<FP8>(d_tmem, a + 2 * k, b + 2 * k, hi, idesc, (kb > w.k0 || k > 0) ? 1u : 0u);
+            umma_commit_pair(&empty[stage], 0x3);
           }
-          umma_commit_pair(&empty[stage], 0x3);
+          __syncwarp();
           if (++stage == STAGES) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!ok) break;
-        umma_commit_pair(&tfull[acc], 0x3);
+        if (issuer) umma_commit_pair(&tfull[acc], 0x3);
+        __syncwarp();
         acc ^= 1;
         if (acc == 0) acc_phase ^= 1u;
       }
-      umma_commit_pair(drain, 0x1);
+      if (issuer) umma_commit_pair(drain, 0x1);
+      __syncwarp();
       const uint64_t t0 = globaltimer_ns();
       while (!mbar_try_wait(smem_u32(drain), 0u)) {
         if (globaltimer_ns() - t0 > HILO_WAIT_LIMIT_NS) {
-          atomicExch(err, DEV_TIMEOUT_GEMM + 256 * 4);
+          if (issuer) atomicExch(err, DEV_TIMEOUT_GEMM + 256 * 4);
           break;
         }
       }
+      __syncwarp();
     }
   } else {
     // ---------------- epilogue (warps 2..5 -> TMEM lane quarters 2,3,0,1), both CTAs

@@ -184,53 +184,58 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
-      const uint32_t idesc = p.idesc;
-      int stage = 0;
-      uint32_t phase = 0;
-      int acc = 0;
-      uint32_t acc_phase = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < sc.total && ok; t += gridDim.x) {
-        if (!mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, err, DEV_TIMEOUT_GEMM)) break;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem + static_cast<uint32_t>(acc * BN);
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&full[stage], phase, abort_flag, err, DEV_TIMEOUT_GEMM)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t a_base = smem_u32(smem + stage * STAGE_BYTES);
-          const uint32_t b_base = a_base + A_STAGE_BYTES;
-#pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t ad = sw128_desc(a_base + k * 32, 16, 1024);
-            const uint64_t bd = sw128_desc(b_base + k * 32, 16, 1024);
-            umma_bf16(d_tmem, ad, bd, idesc, (kb | k) != 0 ? 1u : 0u);
-          }
-          umma_commit(&empty[stage]);
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
-        }
-        if (!ok) break;
-        umma_commit(&tfull[acc]);
-        acc ^= 1;
-        if (acc == 0) acc_phase ^= 1u;
-      }
-      // every MMA this thread issued has completed before TMEM is freed
-      umma_commit(drain);
-      const uint64_t t0 = globaltimer_ns();
-      while (!mbar_try_wait(smem_u32(drain), 0u)) {
-        if (globaltimer_ns() - t0 > HILO_WAIT_LIMIT_NS) {
-          atomicExch(err, DEV_TIMEOUT_GEMM);
+    // ---------------- MMA issuer: the whole warp walks the schedule and
+    // waits, one elected lane issues
+    const bool issuer = elect_one();
+    const uint32_t a_lo = (smem_u32(smem) >> 4) + sw128_lo_lbo(16);
+    constexpr uint32_t hi = sw128_hi(1024);
+    const uint32_t idesc = p.idesc;
+    int stage = 0;
+    uint32_t phase = 0;
+    int acc = 0;
+    uint32_t acc_phase = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < sc.total && ok; t += gridDim.x) {
+      if (!mbar_wait_warp(&tempty[acc], acc_phase ^ 1u, abort_flag, err, DEV_TIMEOUT_GEMM)) break;
+      tc_fence_after();
+      const uint32_t d_tmem = tmem + static_cast<uint32_t>(acc * BN);
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (!mbar_wait_warp(&full[stage], phase, abort_flag, err, DEV_TIMEOUT_GEMM)) {
+          ok = false;
           break;
         }
+        tc_fence_after();
+        if (issuer) {
+          const uint32_t a = a_lo + static_cast<uint32_t>(stage) * (STAGE_BYTES >> 4);
+          const uint32_t b = a + (A_STAGE_BYTES >> 4);
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k)
+            umma_f16_w(d_tmem, a + 2 * k, b + 2 * k, hi, idesc, (kb | k) != 0 ? 1u : 0u);
+          umma_commit(&empty[stage]);
+        }
+        __syncwarp();
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+      if (!ok) break;
+      if (issuer) umma_commit(&tfull[acc]);
+      __syncwarp();
+      acc ^= 1;
+      if (acc == 0) acc_phase ^= 1u;
+    }
+    // every MMA this warp issued has completed before TMEM is freed
+    if (issuer) umma_commit(drain);
+    __syncwarp();
+    const uint64_t t0 = globaltimer_ns();
+    while (!mbar_try_wait(smem_u32(drain), 0u)) {
+      if (globaltimer_ns() - t0 > HILO_WAIT_LIMIT_NS) {
+        if (issuer) atomicExch(err, DEV_TIMEOUT_GEMM);
+        break;
       }
     }
+    __syncwarp();
   } else {
     // ---------------- epilogue (warps 2..5 -> TMEM lane quarters 2,3,0,1)
     const int q = warp & 3;
