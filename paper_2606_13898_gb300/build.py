@@ -38,7 +38,7 @@ LIB_ASAN = os.path.join(BUILD_ASAN, "libhilo.so")
 SANITIZED = ("api.cu", "noalloc.cu")  # the C ABI's host code
 SAN_FLAGS = ["-Xcompiler", "-fsanitize=address", "-Xcompiler", "-fsanitize=undefined",
              "-Xcompiler", "-fno-omit-frame-pointer"]
-SOURCES = ["api.cu", "bw_kernels.cu", "gemm_tc.cu", "gemm2_tc.cu", "attn_tc.cu", "noalloc.cu", "select.cu"]
+SOURCES = ["api.cu", "bw_kernels.cu", "gemm2_tc.cu", "attn_tc.cu", "noalloc.cu", "select.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fno-strict-aliasing",
          "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]

@@ -177,11 +177,6 @@ bool encode_tmap_2d(CUtensorMap* map, TmapType type, const void* base, uint64_t 
   if (!fn) return false;
   CUtensorMapDataType dt = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   uint64_t esize = 2;
-  if (type == TMAP_F16) dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-  if (type == TMAP_F32) {
-    dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-    esize = 4;
-  }
   if (type == TMAP_U8) {
     dt = CU_TENSOR_MAP_DATA_TYPE_UINT8;
     esize = 1;
@@ -243,15 +238,13 @@ int hilo_sync_status(void* stream) {
   cudaError_t e = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "hilo_sync_status: stream");
   const int g = hilo::gemm_take_device_error();
-  const int g2 = hilo::gemm2_take_device_error();
   const int a = hilo::attn_take_device_error();
   const int pr = hilo::probe_take_device_error();
   const int dc = hilo::dcheck_take_bw();
-  if (g < 0 || g2 < 0 || a < 0 || pr < 0 || dc < 0)
+  if (g < 0 || a < 0 || pr < 0 || dc < 0)
     return fail(HILO_ERR_CUDA, "hilo_sync_status: reading the device error word failed");
-  if (g || g2 || a || pr)
-    return fail(HILO_ERR_TIMEOUT, "device-side wait ran out (gemm=%d, gemm pair=%d, attention=%d, probe=%d)", g,
-                g2, a, pr);
+  if (g || a || pr)
+    return fail(HILO_ERR_TIMEOUT, "device-side wait ran out (gemm=%d, attention=%d, probe=%d)", g, a, pr);
   if (dc) return fail(HILO_ERR_CHECK, "device-side index check %d failed (checks build)", dc);
   return HILO_OK;
 }

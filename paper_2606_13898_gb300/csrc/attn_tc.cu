@@ -193,29 +193,37 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return y;
 }
 
+// The images' packed-row offsets within the capacity: from shared memory, where
+// the kernel puts them when they fit (CU_SMEM), else from global memory.
+constexpr int CU_SMEM = 128;
+struct Offsets {
+  const int* s;
+  const AttnParams& p;
+  __device__ __forceinline__ int operator()(int b) const {
+    return s ? s[b] : min(ld_l2(p.cu_img + b), p.cap);
+  }
+  // packed rows of image b
+  __device__ __forceinline__ int len(int b) const { return (*this)(b + 1) - (*this)(b); }
+};
+
 // Row range of tile j of image b (text tiles first, then image tiles); used
 // for both query and key/value tiles.
-__device__ __forceinline__ void seq_tile(const AttnParams& p, int b, int L, int j, int& row0,
+__device__ __forceinline__ void seq_tile(const AttnParams& p, const Offsets& cu, int b, int L, int j, int& row0,
                                          int& valid) {
   if (j < p.qt_txt) {
     row0 = b * p.T + j * BKV;
     valid = min(BKV, p.T - j * BKV);
   } else {
     const int k = j - p.qt_txt;
-    row0 = p.B * p.T + min(p.cu_img[b], p.cap) + k * BKV;
+    row0 = p.B * p.T + cu(b) + k * BKV;
     valid = min(BKV, L - k * BKV);
   }
 }
 
-// Packed image rows of image b within the capacity.
-__device__ __forceinline__ int img_len(const AttnParams& p, int b) {
-  return min(p.cu_img[b + 1], p.cap) - min(p.cu_img[b], p.cap);
-}
-
 // Query tiles of all (image, head) groups.
-__device__ long long total_qtiles(const AttnParams& p) {
+__device__ long long total_qtiles(const AttnParams& p, const Offsets& cu) {
   long long q = 0;
-  for (int b = 0; b < p.B; ++b) q += p.qt_txt + (img_len(p, b) + BQ - 1) / BQ;
+  for (int b = 0; b < p.B; ++b) q += p.qt_txt + (cu.len(b) + BQ - 1) / BQ;
   return q * p.heads;
 }
 
@@ -231,22 +239,22 @@ struct Job {
 // The next job of the flat query-tile range [g, end) (tiles ordered by image,
 // head, tile): two tiles of one group form a pair, a lone tile at the edge of
 // the range or of its group is a split job.
-__device__ bool next_job(const AttnParams& p, long long& g, long long end, Job& jb) {
+__device__ bool next_job(const AttnParams& p, const Offsets& cu, long long& g, long long end, Job& jb) {
   if (g >= end) return false;
   long long base = 0;
   int b = 0, nq = 0, L = 0;
   for (; b < p.B; ++b) {
-    L = img_len(p, b);
+    L = cu.len(b);
     nq = p.qt_txt + (L + BQ - 1) / BQ;
     const long long cnt = static_cast<long long>(nq) * p.heads;
     if (g < base + cnt) break;
     base += cnt;
   }
   if (b >= p.B) return false;
-  const long long r = g - base;
+  const uint32_t r = static_cast<uint32_t>(g - base);  // < nq * heads: row indices are int32
   jb.b = b;
-  jb.h = static_cast<int>(r / nq);
-  jb.j0 = static_cast<int>(r % nq);
+  jb.h = static_cast<int>(r / static_cast<uint32_t>(nq));
+  jb.j0 = static_cast<int>(r % static_cast<uint32_t>(nq));
   jb.nkv = nq;
   jb.L = L;
   const long long grp_end = base + static_cast<long long>(jb.h + 1) * nq;
@@ -265,15 +273,28 @@ template <int HD, bool PROP>
 __global__ void __launch_bounds__(ATTN_THREADS, 1)
     attn_kernel(const __grid_constant__ CUtensorMap tm, const __grid_constant__ AttnParams p) {
   using C = Cfg<HD, PROP>;
-  pdl_trigger();
-  pdl_wait();  // cu_img and q/k/v are written by the previous kernels
+  // The row offsets were written before the previous kernel started: the
+  // schedule, the barriers and tensor memory are ready when it ends.
+  __shared__ int cu_s[CU_SMEM + 1];
+  const bool in_smem = p.B <= CU_SMEM;
+  if (in_smem) {
+    for (int b = threadIdx.x; b <= p.B; b += ATTN_THREADS) cu_s[b] = min(ld_l2(p.cu_img + b), p.cap);
+    __syncthreads();
+  }
+  const Offsets cu{in_smem ? cu_s : nullptr, p};
   // ---- this CTA's share: a contiguous range of the query tiles of all
   // (image, head) groups, ceil(total / grid) tiles per CTA
-  const long long qtiles = total_qtiles(p);
+  const long long qtiles = total_qtiles(p, cu);
   const long long per = (qtiles + gridDim.x - 1) / gridDim.x;
   const long long g_begin = static_cast<long long>(blockIdx.x) * per;
   const long long g_end = min(qtiles, g_begin + per);
-  if (g_begin >= g_end) return;  // uniform across the CTA: nothing allocated yet
+  long long g = g_begin;
+  Job jb;
+  bool more = next_job(p, cu, g, g_end, jb);
+  if (!more) {  // uniform across the CTA: nothing allocated yet
+    pdl_wait();
+    return;
+  }
 
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -324,6 +345,8 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();  // q, k and v are written by the previous kernel
+  pdl_trigger();
   // key tile t of a job whose first tile is the CTA's running tile kt0: its
   // stage and the parity of that stage's use
   auto kv_stage = [](uint32_t kt0, int t) { return static_cast<int>((kt0 + t) & 1u); };
@@ -344,11 +367,9 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
       uint32_t q_par = 0;
       bool ok = true;
       uint32_t kt = 0;
-      long long g = g_begin;
-      Job jb;
       uint64_t* full = kq ? k_full : v_full;
       uint64_t* empty = kq ? k_empty : v_empty;
-      for (uint32_t jn = 0; ok && next_job(p, g, g_end, jb); ++jn) {
+      for (uint32_t jn = 0; ok && more; ++jn, more = next_job(p, cu, g, g_end, jb)) {
         if (kq) {
           // Q of this job once the previous job's MMAs are done with Q
           if (jn > 0 && !mbar_wait(q_empty, (jn - 1) & 1u, abort_flag, err, DEV_TIMEOUT_ATTN + 256 * 16)) {
@@ -356,8 +377,8 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
             break;
           }
           int qr0, qv, qr1 = 0, qv1;
-          seq_tile(p, jb.b, jb.L, jb.j0, qr0, qv);
-          if (jb.pair) seq_tile(p, jb.b, jb.L, jb.j0 + 1, qr1, qv1);
+          seq_tile(p, cu, jb.b, jb.L, jb.j0, qr0, qv);
+          if (jb.pair) seq_tile(p, cu, jb.b, jb.L, jb.j0 + 1, qr1, qv1);
           mbar_arrive_expect_tx(q_full, (jb.pair ? 2 : 1) * C::TILE_BYTES);
 #pragma unroll
           for (int j = 0; j < C::NBOX; ++j) {
@@ -378,7 +399,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
           const int st = kv_stage(kt, t);
           const uint32_t ph = kv_phase(kt, t);
           int row0, valid;
-          seq_tile(p, jb.b, jb.L, t, row0, valid);
+          seq_tile(p, cu, jb.b, jb.L, t, row0, valid);
           if (!mbar_wait(&empty[st], ph ^ 1u, abort_flag, err, DEV_TIMEOUT_ATTN + 256 * (kq ? 1 : 2))) {
             ok = false;
             break;
@@ -455,9 +476,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
     };
     bool ok = true;
     uint32_t kt = 0, sc0 = 0, sc1 = 0;
-    long long g = g_begin;
-    Job jb;
-    for (uint32_t jn = 0; ok && next_job(p, g, g_end, jb); ++jn) {
+    for (uint32_t jn = 0; ok && more; ++jn, more = next_job(p, cu, g, g_end, jb)) {
       const int n0 = job_steps(jb, 0), n1 = job_steps(jb, 1);
       const int qb1 = jb.pair ? 1 : 0;  // the Q buffer of warpgroup 1
       auto wait_k = [&](int t) {
@@ -577,8 +596,8 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
           for (int u = 0; u < 4; ++u) wb[lane + 32 * u] = 1.0f;
         } else {
           int r0, v;
-          seq_tile(p, jb.b, jb.L, tt, r0, v);
-          const float* src = p.n_img + (min(p.cu_img[jb.b], p.cap) + (tt - p.qt_txt) * BKV);
+          seq_tile(p, cu, jb.b, jb.L, tt, r0, v);
+          const float* src = p.n_img + (cu(jb.b) + (tt - p.qt_txt) * BKV);
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             const int col = lane + 32 * u;
@@ -592,9 +611,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
     // sc*: S phases so far (one per step); oc*: o_done phases so far (one
     // per job in which the warpgroup has steps)
     uint32_t kt = 0, sc0 = 0, sc1 = 0, oc0 = 0, oc1 = 0;
-    long long g = g_begin;
-    Job jb;
-    for (uint32_t jn = 0; ok && next_job(p, g, g_end, jb); ++jn) {
+    for (uint32_t jn = 0; ok && more; ++jn, more = next_job(p, cu, g, g_end, jb)) {
       const int n0 = job_steps(jb, 0), n1 = job_steps(jb, 1);
       const int n = i ? n1 : n0;
       const uint32_t sc = i ? sc1 : sc0;
@@ -644,7 +661,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
       for (int s = 0; s < n && ok; ++s) {
         const int t = job_tile(jb, i, s);
         int row0, valid;
-        seq_tile(p, jb.b, jb.L, t, row0, valid);
+        seq_tile(p, cu, jb.b, jb.L, t, row0, valid);
         if (PROP) {
           // every lane is done with slot (s + 1) & 1 (read for step s - 1)
           // before the next step's weights are fetched into it
@@ -809,7 +826,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
           }
           inv = 1.0f / lt;
           int qr0, qv;
-          seq_tile(p, jb.b, jb.L, jb.j0 + (jb.pair ? i : 0), qr0, qv);
+          seq_tile(p, cu, jb.b, jb.L, jb.j0 + (jb.pair ? i : 0), qr0, qv);
           // normalised O rows to bf16, staged through shared memory so that
           // the global stores leave as whole 128-byte lines (one row per
           // lane would write 16 bytes into 32 different rows per

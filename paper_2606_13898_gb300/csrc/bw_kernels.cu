@@ -39,8 +39,8 @@ constexpr int SCORE_MAX_ITERS = 4;  // d <= 4096: at most 4 groups of 8 per thre
 __global__ void __launch_bounds__(SCORE_THREADS) score_kernel(const __nv_bfloat16* __restrict__ x,
                                                               float* __restrict__ s, int B, int H,
                                                               int W, int d) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float part[4][SCORE_THREADS];
   const int j = threadIdx.x;
   const int lane = j & 31;
@@ -411,8 +411,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_select_kernel(
   // their code (this CTA has 1024 threads and at most 64 registers each)
   constexpr bool granular = GRANULAR;
   const int lf = LFMODE ? lf_arg : 0;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ SelectShared sh;
   const int N = H * W;
@@ -569,8 +569,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_select_kernel(
 __global__ void __launch_bounds__(SPLIT_THREADS) split_compact_kernel(
     const uint8_t* __restrict__ labels, const int32_t* __restrict__ counts, int32_t* cu_img,
     int32_t* row_src, int32_t* tok_row, int H, int W, int levels, int lf) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int warp_tot[32];
   const int N = H * W;
@@ -641,8 +641,8 @@ __global__ void __launch_bounds__(256) pack_kernel(const __nv_bfloat16* __restri
                                                    const int32_t* __restrict__ cu_img,
                                                    __nv_bfloat16* __restrict__ packed, int B,
                                                    int H, int W, int d, int cap) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int N = H * W;
   const int G = d >> 3;
@@ -731,8 +731,8 @@ __global__ void __launch_bounds__(256) pack_lf_kernel(const __nv_bfloat16* __res
                                                       const int32_t* __restrict__ cu_img,
                                                       __nv_bfloat16* __restrict__ packed, int B, int H, int W,
                                                       int d, int cap) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int N = H * W;
   const int G = d >> 3;
@@ -771,8 +771,8 @@ __global__ void __launch_bounds__(256) row_sizes_kernel(const uint8_t* __restric
                                                         const int32_t* __restrict__ cu_img,
                                                         float* __restrict__ n_img, int B, int H, int W,
                                                         int cap, int lf) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int N = H * W;
   const int total = min(cu_img[B], cap);
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < total; r += gridDim.x * blockDim.x) {
@@ -803,8 +803,8 @@ __global__ void __launch_bounds__(256) unpack_kernel(const float* __restrict__ o
                                                      const int32_t* __restrict__ tok_row,
                                                      float* __restrict__ y, long long ntok,
                                                      int d, long long rows_max) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const long long wstep = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
   for (long long t = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -827,8 +827,8 @@ __global__ void __launch_bounds__(256) unpack_delta_kernel(const float* __restri
                                                            const int32_t* __restrict__ tok_row,
                                                            float* __restrict__ y, long long ntok, int d,
                                                            long long rows_max) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const long long wstep = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
   for (long long t = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -863,8 +863,8 @@ __global__ void __launch_bounds__(256) unpack_update_kernel(const float* __restr
                                                             __nv_bfloat16* __restrict__ x,
                                                             long long ntok, int d, float alpha,
                                                             long long rows_max) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const long long wstep = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
   for (long long t = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -939,8 +939,8 @@ __global__ void __launch_bounds__(LN_THREADS) layernorm_kernel(const void* __res
                                                                float* __restrict__ ln_scale,
                                                                const int32_t* __restrict__ cu_img,
                                                                int B, int n_txt, int cap, int d) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float red[LN_THREADS / 32];
   const int rows = n_txt + min(cu_img[B], cap);
   const float inv_d = 1.0f / static_cast<float>(d);
@@ -1063,8 +1063,8 @@ __global__ void __launch_bounds__(QR_THREADS) quant_rows_kernel(const void* __re
                                                                 const int32_t* __restrict__ cu_img, int B,
                                                                 int n_txt, int cap, uint8_t* __restrict__ dst,
                                                                 float* __restrict__ scale) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ float red[QR_THREADS / 32];
   const int rows = cu_img ? n_txt + min(cu_img[B], cap) : rows_static;
   const int g8 = cols >> 3;
@@ -1106,8 +1106,8 @@ __global__ void __launch_bounds__(QR_THREADS) quant_rows_kernel(const void* __re
 
 __global__ void __launch_bounds__(256) bf16_to_f16_kernel(const uint4* __restrict__ src,
                                                           uint4* __restrict__ dst, long long n8) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n8;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
     float f[8];

@@ -132,39 +132,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
-// Bulk tensor store of a shared-memory box to global memory (tile mode),
-// tracked by the issuing thread's bulk async-group.
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* src, int x, int y) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(smem_u32(src)), "r"(x), "r"(y)
-               : "memory");
-}
-
-// Same, but the box is added element-wise to what global memory holds (the
-// addition is done by the memory system; the element type is the map's).
-__device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* map, const void* src, int x, int y) {
-  asm volatile(
-      "cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
-          reinterpret_cast<uint64_t>(map)),
-      "r"(smem_u32(src)), "r"(x), "r"(y)
-      : "memory");
-}
-
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-
-// Wait until at most N of this thread's bulk groups still read shared memory.
-template <int N>
-__device__ __forceinline__ void bulk_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
-}
-
-// Wait until at most N of this thread's bulk groups are still incomplete.
-template <int N>
-__device__ __forceinline__ void bulk_wait() {
-  asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // Bulk tensor prefetch of a box into L2 (no shared memory, no completion).
 __device__ __forceinline__ void tma_prefetch_l2_2d(const CUtensorMap* map, int x, int y) {
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
@@ -440,11 +407,16 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int a_mn_major, 
 
 // ---------------------------------------------- programmatic dependent launch --
 // Every libhilo kernel is launched with programmatic stream serialization: it
-// may start while the previous kernel on the stream is finishing. It signals
-// at once that its own successor may launch (pdl_trigger) and waits for its
-// predecessor's completion and memory (pdl_wait) before its first global
-// memory access; only the prologue (barrier init, TMEM allocation, tensor-map
-// prefetch) runs before that. Both are no-ops without a predecessor.
+// may start while the previous kernel on the stream is finishing. It waits for
+// its predecessor's completion and memory (pdl_wait) before it touches anything
+// the predecessor may write or still read, and only then signals that its own
+// successor may launch (pdl_trigger). So when a kernel starts, everything up to
+// the kernel before its predecessor is complete: a kernel that always has
+// another one of the same call before it (the block's GEMMs and its attention)
+// may read the row counts and the weights before its own wait, through L2
+// (ld_l2, TMA), and have its schedule, barriers, tensor memory and first weight
+// tiles ready when the wait ends. Every CTA executes the wait, also one that
+// has no work, or this would not carry over from kernel to kernel.
 // Per-warpgroup register budget (all 128 threads of the warpgroup execute
 // it). inc waits until enough registers were released by dec elsewhere in
 // the CTA, so the shares must add up to the launch's allocation.
@@ -455,6 +427,14 @@ __device__ __forceinline__ void setmaxnreg_inc() {
 template <uint32_t R>
 __device__ __forceinline__ void setmaxnreg_dec() {
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R));
+}
+
+// A value written two or more kernels ago, from L2 (this SM's L1 may hold an
+// older one).
+__device__ __forceinline__ int ld_l2(const int32_t* p) {
+  int v;
+  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
 }
 
 __device__ __forceinline__ void pdl_trigger() {

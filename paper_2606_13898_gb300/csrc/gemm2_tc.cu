@@ -1,26 +1,37 @@
-// Grouped GEMM on CTA pairs (tcgen05 cta_group::2): same computation and
-// epilogues as gemm_tc.cu, with 256x256 output tiles per pair of SMs.
+// Grouped GEMM of the MMDiT block's linear layers (paper Sec. 2.1, the DiT's
+// QKV, output and MLP projections) on the 5th-generation tensor cores:
+//   C[r, n] = sum_k X[r, k] * W_g[n, k] + b_g[n]
+// with the text rows (group 0) and the packed image rows (group 1) of the row
+// space using their own weights. The image row count is read on the device,
+// so no host synchronisation is needed between split and block.
 //
-// Each CTA of a pair loads 128 rows of A and 128 rows of W (half of the
-// tile's 256 output columns) into its own shared memory at identical offsets;
-// the even CTA issues tcgen05.mma.cta_group::2 with M = 256, N = 256, which
-// reads both CTAs' halves. Compared with one SM computing a 128x256 tile,
-// each SM stages and feeds half the W bytes per MAC, so the shared-memory
-// traffic per MAC drops by a third and the ring can be 6 stages deep.
+// CTA pairs (tcgen05 cta_group::2), transposed tiles: the MMA's 256 rows (M)
+// are output features and its columns (N) are rows of the row space, 32 to 256
+// of them in steps of 32. Features come in multiples of 128, so M wastes
+// little, while the row counts are whatever the selection left: with the rows
+// on N a group is cut into tiles of nearly equal height, and the tiles of the
+// last, partial round are cut again, so that they reach every pair (Plan).
 //
-// Per CTA, 192 threads:
-//   warp 0     TMA producer: A and W halves; the completion of both CTAs'
-//              copies is counted on the even CTA's "full" barrier
-//   warp 1     TMEM allocation (both CTAs); MMA issue (even CTA only)
-//   warps 2-5  epilogue over this CTA's 128 rows x 256 columns
+// Each CTA of a pair stages 128 rows of W (half of the tile's features) and
+// half of the tile's X rows at identical shared-memory offsets; the even CTA
+// issues the MMAs, which read both CTAs' halves.
+//
+// Per CTA, 320 threads:
+//   warp 0     TMA producer: W half, X half (as up to three boxes of 128, 64,
+//              32 and 16 rows); the completion of both CTAs' copies is counted
+//              on the even CTA's "full" barrier
+//   warp 1     TMEM allocation (both CTAs); MMA issue (even CTA only): the
+//              whole warp walks the schedule and waits, one elected lane issues
+//   warps 2-9  epilogue over this CTA's 128 features x the tile's rows, two
+//              warps per TMEM lane quarter, 32-row chunks alternating
 // "empty" and "accumulator ready" barriers are signalled in both CTAs by a
-// multicast commit; "accumulator free" collects 8 arrivals (4 epilogue warps
+// multicast commit; "accumulator free" collects 16 arrivals (8 epilogue warps
 // x 2 CTAs) in the even CTA. Every wait is bounded.
 //
-// FP8 (e4m3 A and W, kind::f8f6f4): a k-block is the same 128-byte swizzled
+// FP8 (e4m3 X and W, kind::f8f6f4): a k-block is the same 128-byte swizzled
 // row of shared memory holding 128 elements instead of 64, and each MMA
 // consumes 32 of them; the epilogue multiplies each accumulator by its row's
-// A scale and its column's W scale before the bias.
+// X scale and its feature's W scale before the bias.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -30,28 +41,38 @@
 
 namespace hilo {
 
-__device__ int g_gemm2_err;
+__device__ int g_gemm_err;
 
 namespace {
 
-constexpr int PM = 256;   // rows per pair tile (128 per CTA)
-constexpr int PN = 256;   // columns per pair tile (128 of W rows staged per CTA)
+constexpr int PF = 256;   // features per pair tile (128 of W staged per CTA)
+constexpr int UNIT = 32;  // rows of a tile come in units of 32 ...
+constexpr int MAXU = 8;   // ... at most 256
 constexpr int BK = 64;
-constexpr int STAGES = 6;
-constexpr int HALF_BYTES = 128 * BK * 2;    // 16 KB: one CTA's A or W slice
-constexpr int STAGE_BYTES = 2 * HALF_BYTES; // A + W slices of this CTA
-constexpr int THREADS = 192;
+constexpr int STAGES = 7;
+constexpr int HALF_BYTES = 128 * BK * 2;    // 16 KB: one CTA's W slice, or its largest X slice
+constexpr int STAGE_BYTES = 2 * HALF_BYTES; // W + X slices of this CTA
+constexpr int EPI_WARPS = 8;
+constexpr int THREADS = 32 * (2 + EPI_WARPS);
 constexpr uint32_t TMEM_COLS = 512;         // two 128 x 256 fp32 accumulators
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_SMEM_BYTES + 1024 + 256;
-constexpr int SPLIT_MIN_KB = 32;            // shortest piece of a tile cut into equal K pieces
-constexpr int SPLIT_MAX = 8;                // most equal pieces per tile
-constexpr int STREAM_MIN_KB = 16;           // shortest stream-K range
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr int SPLIT_MIN_KB = 16;            // shortest piece of a tile cut along K
+constexpr int SPLIT_MAX = 8;                // most pieces per tile
+// the plan's costs in SM cycles beside those of the k-blocks
+constexpr float TILE_CYC = 400.f;           // going from one tile to the next
+constexpr float EPI_CYC = 800.f;            // the last epilogue, per 32 rows
+constexpr float PIECE_CYC = 300.f;          // a K piece's reductions, per 32 rows
+
+struct Maps {
+  CUtensorMap x[4];  // boxes of 128, 64, 32, 16 rows
+  CUtensorMap w[2];
+};
 
 struct Params {
   int N, K;
-  uint32_t idesc;
-  const float* a_scale;     // FP8: dequantisation scale per row of A (row space)
-  const float* b_scale[2];  // FP8: per output column, per weight group
+  uint32_t idesc;           // without the N field
+  const float* a_scale;     // FP8: dequantisation scale per row of X (row space)
+  const float* b_scale[2];  // FP8: per output feature, per weight group
   int row_base[2];
   int rows_static[2];
   const int32_t* rows_dev[2];
@@ -62,151 +83,188 @@ struct Params {
   int resid_f32;
 };
 
-struct Tile {
-  int g, m0, n0, rows, row_base;
+// One unit of a pair's work: k-blocks [k0, k1) of piece `part` of `parts` (cut by
+// rows) of tile t.
+struct Work {
+  int t, k0, k1, part, parts;
 };
 
-struct Sched {
-  // two row groups, kept in scalars (no runtime-indexed arrays, which would
-  // live in local memory)
-  int mt0, mt1, rows0, rows1, nt, total;
-  __device__ void init(const Params& p) {
-    nt = (p.N + PN - 1) / PN;
+// Rows [r0, r0 + 32 units) of group g (of `rows` valid ones), feature block f.
+struct Tile {
+  int g, f, r0, units, rows, row_base;
+};
+
+// How the rows are cut and the tiles dealt; every role of every CTA computes
+// the same plan from the same row counts.
+struct Plan {
+  int rows0, rows1, U0, U1;  // rows and 32-row units per group
+  int t0, t1;                // row tiles per group
+  int total;                 // tiles
+  int whole;                 // tiles dealt whole; the rest are cut
+  int nsplit;                // pieces per cut tile
+  int kcut;                  // cut along K (else by rows)
+
+  // Cycles of one k-block of a tile of x units. The MMAs take 64 x, but every
+  // byte of W and X is written to shared memory once and read once, at 128 bytes
+  // a cycle: 2 (16 KB + 2 KB x) / 128 = 256 + 32 x, plus 6% as measured (520,
+  // 511, 480 and 427 cycles at x = 8, 7, 6 and 4). So a tile of 256 rows runs at
+  // the MMA rate and a lower one loses what it saves in columns.
+  __device__ static float kblock(float x) { return 272.0f + 34.0f * x; }
+
+  // Chosen by cost: lane l tries image tiles of at most u1 = 8 - l % 8 units,
+  // text tiles of at most u1 + l / 8, and cuts of the tiles left over after the
+  // last full round into 2 to 8 pieces, by rows or, with `split`, along K; the
+  // cheapest wins, the higher tile and the fewer pieces among equals. The cost is
+  // that of pair 0, which has the most tiles: its rounds of whole tiles, its
+  // pieces, and the epilogue that nothing hides. Called by whole warps.
+  __device__ void init(const Params& p, int dev0, int dev1, int ncl, int kb, bool split) {
     // a device row count is bounded by the group's capacity (rows_static)
-    rows0 = p.rows_dev[0] ? min(*p.rows_dev[0], p.rows_static[0]) : p.rows_static[0];
-    rows1 = p.rows_dev[1] ? min(*p.rows_dev[1], p.rows_static[1]) : p.rows_static[1];
-    mt0 = (rows0 + PM - 1) / PM;
-    mt1 = (rows1 + PM - 1) / PM;
-    total = (mt0 + mt1) * nt;
+    rows0 = max(0, p.rows_dev[0] ? min(dev0, p.rows_static[0]) : p.rows_static[0]);
+    rows1 = max(0, p.rows_dev[1] ? min(dev1, p.rows_static[1]) : p.rows_static[1]);
+    U0 = (rows0 + UNIT - 1) / UNIT;
+    U1 = (rows1 + UNIT - 1) / UNIT;
+    const int F = (p.N + PF - 1) / PF;
+    const int lane = lane_id();
+    const int u1 = MAXU - (lane & 7), u0 = min(MAXU, u1 + (lane >> 3));
+    const int a0 = (U0 + u0 - 1) / u0, a1 = (U1 + u1 - 1) / u1;
+    const int T0 = F * a0, T = F * (a0 + a1), rem = T % ncl;
+    const float x0 = a0 ? static_cast<float>(U0) / a0 : 0.f, x1 = a1 ? static_cast<float>(U1) / a1 : 0.f;
+    const float xm = fmaxf(x0, x1);
+    const int least = a0 && a1 ? min(U0 / a0, U1 / a1) : (a0 ? U0 / a0 : (a1 ? U1 / a1 : 0));
+    const float kbf = static_cast<float>(kb);
+    const float c0 = kbf * kblock(x0) + TILE_CYC, c1 = kbf * kblock(x1) + TILE_CYC;
+    // ceil(n / ncl) for the small counts here (n + 0.5 keeps the product away
+    // from the whole numbers)
+    const float inv = 1.0f / static_cast<float>(ncl);
+    auto rounds_of = [&](int n) { return static_cast<int>((static_cast<float>(n + ncl - 1) + 0.5f) * inv); };
+    const int g_max = rounds_of(T0);
+    auto rounds_cost = [&](int tiles) {
+      const int rounds = rounds_of(tiles), g0 = min(rounds, g_max);
+      return g0 * c0 + (rounds - g0) * c1;
+    };
+    float best = rounds_cost(T) + EPI_CYC * xm;
+    int best_s = 1, best_k = 0;
+    if (rem > 0) {
+      const float c_full = rounds_cost(T - rem);
+#pragma unroll
+      for (int s = 2; s <= SPLIT_MAX; ++s) {
+        const float n = static_cast<float>(rounds_of(rem * s));
+        const float xs = ceilf(xm * (1.0f / s) - 1e-3f);
+        const float cr = c_full + n * (kbf * kblock(xs) + TILE_CYC) + EPI_CYC * xs;
+        if (s <= least && cr < best) best = cr, best_s = s, best_k = 0;
+        const float ck =
+            c_full + n * (((kb + s - 1) / s) * kblock(xm) + TILE_CYC + PIECE_CYC * xm) + EPI_CYC * xm;
+        if (split && kb >= s * SPLIT_MIN_KB && ck < best) best = ck, best_s = s, best_k = 1;
+      }
+    }
+    // costs are positive, so their bit patterns order like the values
+    const uint32_t key = __float_as_uint(best);
+    const uint32_t lo = __reduce_min_sync(0xffffffffu, key);
+    const int win = __ffs(__ballot_sync(0xffffffffu, key == lo)) - 1;
+    t0 = __shfl_sync(0xffffffffu, a0, win);
+    t1 = __shfl_sync(0xffffffffu, a1, win);
+    nsplit = __shfl_sync(0xffffffffu, best_s, win);
+    kcut = __shfl_sync(0xffffffffu, best_k, win);
+    total = F * (t0 + t1);
+    whole = nsplit > 1 ? total - total % ncl : total;
   }
-  __device__ Tile get(const Params& p, int t) const {
+
+  // (i U + o) / n, the first unit of row tile i of n
+  __device__ static int cut(int i, int U, int n, int o) {
+    const int base = U / n, more = U - base * n;
+    return i * base + (n <= 32768 ? (i * more + o) / n
+                                  : static_cast<int>((static_cast<long long>(i) * more + o) / n));
+  }
+
+  // Row tiles vary fastest, so that the pairs running at one time share W. A
+  // group's units are dealt to its row tiles as evenly as they go; which tiles
+  // get the odd unit turns with the feature block, so that no pair collects
+  // only the higher ones.
+  __device__ Tile get(const Params& p, const Work& w) const {
+    int t = w.t;
+    const int T0 = total / (t0 + t1) * t0;
     Tile r;
-    r.g = t < mt0 * nt ? 0 : 1;
-    if (r.g) t -= mt0 * nt;
-    const int mtg = r.g ? mt1 : mt0;
-    r.row_base = r.g ? p.row_base[1] : p.row_base[0];
-    r.m0 = r.row_base + (t % mtg) * PM;
-    r.n0 = (t / mtg) * PN;
+    r.g = t < T0 ? 0 : 1;
+    if (r.g) t -= T0;
+    const int n = r.g ? t1 : t0, U = r.g ? U1 : U0;
+    r.f = t / n;
+    const int i = t - r.f * n;
+    int b0 = cut(i, U, n, r.f % n), b1 = cut(i + 1, U, n, r.f % n);
+    if (w.parts > 1) {
+      const int x = b1 - b0;
+      b1 = b0 + (w.part + 1) * x / w.parts;
+      b0 += w.part * x / w.parts;
+    }
+    r.r0 = b0 * UNIT;
+    r.units = b1 - b0;
     r.rows = r.g ? rows1 : rows0;
+    r.row_base = r.g ? p.row_base[1] : p.row_base[0];
     return r;
   }
 };
 
-// One unit of a pair's work: k-blocks [k0, k1) of tile t.
-struct Work {
-  int t, k0, k1;
-};
-
-// Pieces per tile of the partial round: the count that makes the longest
-// pair's share of the round (rounds of pieces x piece length, in k-blocks)
-// shortest, with pieces of at least SPLIT_MIN_KB k-blocks, so that a piece's
-// main loop still hides the reduce-add epilogue of the piece before it. Ties
-// go to fewer pieces.
-__device__ __forceinline__ int tail_splits(int rem, int ncl, int kb) {
-  if (rem == 0) return 1;
-  int best = 1, cost = kb;  // rem < ncl: one round of whole tiles
-  for (int s = 2; s <= SPLIT_MAX && kb / s >= SPLIT_MIN_KB; ++s) {
-    const int c = ((rem * s + ncl - 1) / ncl) * ((kb + s - 1) / s);
-    if (c < cost) {
-      best = s;
-      cost = c;
-    }
-  }
-  return best;
-}
-
-// The work of pair `cid` of `ncl`. Tiles are dealt round-robin, whole, while
-// a full round remains. When the output is accumulated in place (fp32 +=,
-// written by TMA reduce-add) the tiles of the last, partial round are cut
-// along K instead; each piece adds its partial sum to the output, and only
-// the piece that starts at k = 0 adds the bias. Two cuts:
-//  * equal pieces (tail_splits of them per tile, when that shortens the
-//    round), dealt round-robin piece-major: the pieces that run at the same
-//    time cover one or two K ranges, so the pairs share those slices of A
-//    and W in L2 even when A and W together exceed it;
-//  * otherwise stream-K: the round's k-blocks in equal contiguous ranges of
-//    at least STREAM_MIN_KB, one per pair, each spanning one or two tiles
-//    (shorter than whole pieces, but every pair at its own K offset).
-// Other epilogues deal every tile whole. All roles of the pair walk the same
-// sequence.
+// The work of pair `cid` of `ncl`: whole tiles round-robin, then the pieces of
+// the remaining ones, dealt piece-major: K pieces that run at the same time
+// cover one or two K ranges, so the pairs share those slices of X and W in L2
+// even when X and W together exceed it. Each K piece adds its partial sum to
+// the output (fp32 += only); the one that starts at k = 0 adds the bias.
 struct WorkIter {
-  int t, t_end, ncl, kb, rem, nsplit, u, u_end;
-  long long lo, hi;  // stream-K: this pair's k-block range, over the whole tile sequence
-  __device__ WorkIter(const Sched& sc, int cid, int ncl_, int kblocks, bool split) {
-    ncl = ncl_;
-    kb = kblocks;
-    rem = split && sc.total > ncl ? sc.total % ncl : 0;
-    t_end = sc.total - rem;
-    t = cid;
-    nsplit = tail_splits(rem, ncl, kblocks);
-    u = cid;
-    u_end = nsplit > 1 ? rem * nsplit : 0;
-    lo = hi = 0;
-    if (rem > 0 && nsplit == 1) {
-      const long long w = static_cast<long long>(rem) * kblocks;
-      const int np = static_cast<int>(max(1LL, min(static_cast<long long>(ncl), w / STREAM_MIN_KB)));
-      if (cid < np) {
-        lo = w * cid / np;
-        hi = w * (cid + 1) / np;
-      }
-      lo += static_cast<long long>(t_end) * kblocks;
-      hi += static_cast<long long>(t_end) * kblocks;
-    }
-  }
+  int t, whole, rem, nsplit, kcut, ncl, kb, u;
+  __device__ WorkIter(const Plan& pl, int cid, int ncl_, int kblocks)
+      : t(cid), whole(pl.whole), rem(pl.total - pl.whole), nsplit(pl.nsplit), kcut(pl.kcut), ncl(ncl_), kb(kblocks),
+        u(cid) {}
   __device__ bool next(Work& w) {
-    if (t < t_end) {
+    w.k0 = 0;
+    w.k1 = kb;
+    w.part = 0;
+    w.parts = 1;
+    if (t < whole) {
       w.t = t;
-      w.k0 = 0;
-      w.k1 = kb;
       t += ncl;
       return true;
     }
-    if (u < u_end) {
-      const int s = u / rem;  // piece index: u_end > 0 implies rem > 0
-      w.t = t_end + (u - s * rem);
+    if (u >= rem * nsplit) return false;
+    const int s = u / rem;  // piece index
+    w.t = whole + (u - s * rem);
+    if (kcut) {
       w.k0 = s * kb / nsplit;
       w.k1 = (s + 1) * kb / nsplit;
-      u += ncl;
-      return true;
+    } else {
+      w.part = s;
+      w.parts = nsplit;
     }
-    if (lo >= hi) return false;
-    w.t = static_cast<int>(lo / kb);
-    w.k0 = static_cast<int>(lo % kb);
-    const long long end = min(hi, static_cast<long long>(w.t + 1) * kb);
-    w.k1 = w.k0 + static_cast<int>(end - lo);
-    lo = end;
+    u += ncl;
     return true;
   }
 };
 
 template <bool FP8>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
-    gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
-                 const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmOut,
-                 const __grid_constant__ Params p) {
-  // elements per k-block: one 128-byte swizzled row of A / W
+    gemm2_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Params p) {
+  // elements per k-block: one 128-byte swizzled row of X / W
   constexpr int BKE = FP8 ? 128 : BK;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  unsigned char* epi_stage = smem + STAGES * STAGE_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(epi_stage + EPI_SMEM_BYTES);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
   uint64_t* empty = full + STAGES;
   uint64_t* tfull = empty + STAGES;
   uint64_t* tempty = tfull + 2;
   uint64_t* drain = tempty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  int* err = &g_gemm2_err;
+  int* err = &g_gemm_err;
 
   const int warp = warp_id(), lane = lane_id();
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   const int cid = blockIdx.x >> 1;
   const int ncl = gridDim.x >> 1;
-  pdl_trigger();
-  Sched sc;
 
+  // The row counts and the weights were there before the previous kernel
+  // started: the plan is made, and this pair's first W slices are on their way,
+  // while that kernel finishes. Only X, the residual and the outputs wait for it.
+  const int dev0 = p.rows_dev[0] ? ld_l2(p.rows_dev[0]) : 0, dev1 = p.rows_dev[1] ? ld_l2(p.rows_dev[1]) : 0;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
@@ -214,116 +272,125 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&tfull[a], 1);
-      mbar_init(&tempty[a], 8);  // 4 epilogue warps x 2 CTAs
+      mbar_init(&tempty[a], 2 * EPI_WARPS);
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
-  if (warp == 0 && lane == 0) {
-    tma_prefetch_desc(&tmA);
-    tma_prefetch_desc(&tmB0);
-    tma_prefetch_desc(&tmB1);
-  }
+  if (warp == 0 && lane < 6) tma_prefetch_desc(lane < 4 ? &tm.x[lane] : &tm.w[lane - 4]);
   if (warp == 1) {
     tmem_alloc_pair(tmem_slot, TMEM_COLS);
     tmem_relinquish_pair();
   }
+  const int kblocks = p.K / BKE;
+  Plan pl;
+  pl.init(p, dev0, dev1, ncl, kblocks, p.epilogue == EPI_BIAS_RESID_F32);
+  WorkIter it(pl, cid, ncl, kblocks);
+  Work w;
   tc_fence_before();
   __syncthreads();
   cluster_sync();  // both CTAs' barriers are initialised before any remote use
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int kblocks = p.K / BKE;
-  // The weights do not depend on the previous kernel: while it finishes,
-  // pull the first k-blocks of this pair's first weight tile into L2. The
-  // tile is exact when it lies in a group whose row count is static (the
-  // text rows); in the image rows, whose count is read only after the wait,
-  // the column block is a guess, and a wrong one costs only the prefetch.
-  if (warp == 0 && lane == 0) {
-    const int nt = p.N / PN;
-    const int mt0 = p.rows_dev[0] ? 0 : (p.rows_static[0] + PM - 1) / PM;
-    const CUtensorMap* tb;
-    int n;
-    if (cid < mt0 * nt) {
-      tb = &tmB0;
-      n = cid / mt0;
-    } else {
-      tb = &tmB1;
-      n = (cid - mt0 * nt) % nt;
-    }
-    const int y = n * PN + 128 * static_cast<int>(rank);
-    for (int kb = 0; kb < min(kblocks, STAGES); ++kb) tma_prefetch_l2_2d(tb, kb * BKE, y);
-  }
-  pdl_wait();  // the row counts and A are written by the previous kernel
-  sc.init(p);
-  const bool split_k = p.epilogue == EPI_BIAS_RESID_F32;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer (both CTAs)
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t armed = 0, armed_par = 0;  // per stage: armed at least once, parity of the last arming
-      bool ok = true;
-      WorkIter it(sc, cid, ncl, kblocks, split_k);
-      Work w;
-      while (ok && it.next(w)) {
-        const Tile tl = sc.get(p, w.t);
-        const CUtensorMap* tb = tl.g ? &tmB1 : &tmB0;
-        for (int kb = w.k0; kb < w.k1; ++kb) {
-          if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 1)) {
-            ok = false;
-            break;
+    // ---------------- TMA producer (both CTAs): the whole warp walks the
+    // schedule, one elected lane issues
+    const bool issuer = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    uint32_t armed = 0, armed_par = 0;  // per stage: armed at least once, parity of the last arming
+    bool ok = true;
+    const uint32_t full0 = mapa_shared(smem_u32(full), 0);
+    bool first = true;
+    while (ok && it.next(w)) {
+      const Tile tl = pl.get(p, w);
+      const CUtensorMap* mw = tl.g ? &tm.w[1] : &tm.w[0];
+      const int yw = tl.f * PF + 128 * static_cast<int>(rank);
+      const int yx = tl.row_base + tl.r0 + static_cast<int>(rank) * tl.units * 16;
+      const uint32_t bytes = 2u * (HALF_BYTES + static_cast<uint32_t>(tl.units) * 16 * 128);
+      auto load_w = [&](int st, int kb) {
+        if (leader) mbar_arrive_expect_tx(&full[st], bytes);
+        tma_load_2d_pair(smem + st * STAGE_BYTES, mw, full0 + 8u * static_cast<uint32_t>(st), kb * BKE, yw);
+      };
+      auto load_x = [&](int st, int kb) {
+        unsigned char* dst = smem + st * STAGE_BYTES + HALF_BYTES;
+        int y = yx;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (tl.units & (8 >> i)) {
+            tma_load_2d_pair(dst, &tm.x[i], full0 + 8u * static_cast<uint32_t>(st), kb * BKE, y);
+            dst += (128 >> i) * 128;
+            y += 128 >> i;
           }
-          unsigned char* sa = smem + stage * STAGE_BYTES;
-          const uint32_t full_cl = mapa_shared(smem_u32(&full[stage]), 0);
-          if (leader) mbar_arrive_expect_tx(&full[stage], 2 * STAGE_BYTES);
-          tma_load_2d_pair(sa, &tmA, full_cl, kb * BKE, tl.m0 + 128 * static_cast<int>(rank));
-          tma_load_2d_pair(sa + HALF_BYTES, tb, full_cl, kb * BKE, tl.n0 + 128 * static_cast<int>(rank));
-          armed |= 1u << stage;
-          armed_par = (armed_par & ~(1u << stage)) | (phase << stage);
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
-        }
+      };
+      int kb = w.k0;
+      if (first) {
+        // the ring is empty: W of its first stages before the wait, X after it
+        first = false;
+        const int n = min(STAGES, w.k1 - w.k0);
+        if (issuer)
+          for (int i = 0; i < n; ++i) load_w(i, w.k0 + i);
+        pdl_wait();
+        if (issuer)
+          for (int i = 0; i < n; ++i) load_x(i, w.k0 + i);
+        __syncwarp();
+        armed = (1u << n) - 1u;  // every parity is still 0
+        kb += n;
+        stage = n == STAGES ? 0 : n;
+        phase = n == STAGES ? 1u : 0u;
       }
-      if (!ok) {
-        // let the bulk copies already issued land before the CTA can exit
-        const uint64_t t0 = globaltimer_ns();
-        if (leader) {
-          for (int s = 0; s < STAGES; ++s) {
-            if (!((armed >> s) & 1u)) continue;
-            while (!mbar_try_wait(smem_u32(&full[s]), (armed_par >> s) & 1u) &&
-                   globaltimer_ns() - t0 < HILO_WAIT_LIMIT_NS / 4) {
-            }
-          }
-        } else {
-          while (globaltimer_ns() - t0 < 50000ull) {
-          }
+      for (; kb < w.k1; ++kb) {
+        if (!mbar_wait_warp(&empty[stage], phase ^ 1u, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 1)) {
+          ok = false;
+          break;
+        }
+        if (issuer) {
+          load_w(stage, kb);
+          load_x(stage, kb);
+        }
+        __syncwarp();
+        armed |= 1u << stage;
+        armed_par = (armed_par & ~(1u << stage)) | (phase << stage);
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
     }
+    if (!ok) {
+      // let the bulk copies already issued land before the CTA can exit
+      const uint64_t tw = globaltimer_ns();
+      if (leader) {
+        for (int s = 0; s < STAGES; ++s) {
+          if (!((armed >> s) & 1u)) continue;
+          while (!mbar_try_wait(smem_u32(&full[s]), (armed_par >> s) & 1u) &&
+                 globaltimer_ns() - tw < HILO_WAIT_LIMIT_NS / 4) {
+          }
+        }
+      } else {
+        while (globaltimer_ns() - tw < 50000ull) {
+        }
+      }
+    }
+    __syncwarp();
   } else if (warp == 1) {
     if (leader) {
-      // ---------------- MMA issuer (even CTA): the whole warp walks the
-      // schedule and waits, one elected lane issues
+      // ---------------- MMA issuer (even CTA)
       const bool issuer = elect_one();
-      const uint32_t a_lo = (smem_u32(smem) >> 4) + sw128_lo_lbo(16);
+      const uint32_t w_lo = (smem_u32(smem) >> 4) + sw128_lo_lbo(16);
       constexpr uint32_t hi = sw128_hi(1024);
-      const uint32_t idesc = p.idesc;
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
-      WorkIter it(sc, cid, ncl, kblocks, split_k);
-      Work w;
       while (ok && it.next(w)) {
+        const uint32_t idesc = p.idesc | (static_cast<uint32_t>(pl.get(p, w).units * (UNIT / 8)) << 17);
         if (!mbar_wait_warp(&tempty[acc], acc_phase ^ 1u, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 2)) break;
         tc_fence_after();
-        const uint32_t d_tmem = tmem + static_cast<uint32_t>(acc * PN);
+        const uint32_t d_tmem = tmem + static_cast<uint32_t>(acc * UNIT * MAXU);
         for (int kb = w.k0; kb < w.k1; ++kb) {
           if (!mbar_wait_warp(&full[stage], phase, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 3)) {
             ok = false;
@@ -331,7 +398,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
           }
           tc_fence_after();
           if (issuer) {
-            const uint32_t a = a_lo + static_cast<uint32_t>(stage) * (STAGE_BYTES >> 4);
+            const uint32_t a = w_lo + static_cast<uint32_t>(stage) * (STAGE_BYTES >> 4);
             const uint32_t b = a + (HALF_BYTES >> 4);
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k)
@@ -352,9 +419,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       }
       if (issuer) umma_commit_pair(drain, 0x1);
       __syncwarp();
-      const uint64_t t0 = globaltimer_ns();
+      const uint64_t tw = globaltimer_ns();
       while (!mbar_try_wait(smem_u32(drain), 0u)) {
-        if (globaltimer_ns() - t0 > HILO_WAIT_LIMIT_NS) {
+        if (globaltimer_ns() - tw > HILO_WAIT_LIMIT_NS) {
           if (issuer) atomicExch(err, DEV_TIMEOUT_GEMM + 256 * 4);
           break;
         }
@@ -362,56 +429,90 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       __syncwarp();
     }
   } else {
-    // ---------------- epilogue (warps 2..5 -> TMEM lane quarters 2,3,0,1), both CTAs
-    const int q = warp & 3;
-    unsigned char* stage = epi_stage + q * EPI_WARP_BYTES;
-    int buf = 0;
+    // ---------------- epilogue, both CTAs: TMEM lane quarter warp % 4, the
+    // even or the odd 32-row chunks
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const int N = p.N, epi = p.epilogue;
+    const bool resid_f32 = p.resid_f32 != 0;
     int acc = 0;
     uint32_t acc_phase = 0;
-    if (warp == 2 && lane == 0) tma_prefetch_desc(&tmOut);
-    WorkIter it(sc, cid, ncl, kblocks, split_k);
-    Work w;
+    pdl_wait();
+    pdl_trigger();
     while (it.next(w)) {
-      const Tile tl = sc.get(p, w.t);
+      const Tile tl = pl.get(p, w);
+      EpiChunk ch;
+      ch.feat = tl.f * PF + 128 * static_cast<int>(rank) + q * 32 + lane;
+      const bool on = ch.feat < N;  // N is a multiple of 128: the same for the whole warp
       // the bias is added once per tile, by the piece that starts at k = 0
-      const uint4 bpre = w.k0 == 0 ? epi_bias_preload<PN>(tl.g ? p.bias[1] : p.bias[0], tl.n0, p.N)
-                                   : make_uint4(0u, 0u, 0u, 0u);
-      EpiScale escale;
-      if (FP8) escale = epi_scale_preload<PN>(p.a_scale, tl.g ? p.b_scale[1] : p.b_scale[0],
-                                              tl.m0 + 128 * static_cast<int>(rank) + q * 32,
-                                              min(32, max(0, tl.rows - (tl.m0 - tl.row_base) -
-                                                                 (128 * static_cast<int>(rank) + q * 32))),
-                                              tl.n0, p.N);
-      const int off = 128 * static_cast<int>(rank) + q * 32;  // slab offset in the pair tile
-      const int nvalid = min(32, max(0, tl.rows - (tl.m0 - tl.row_base) - off));
-      if (p.epilogue == EPI_BIAS_RESIDIN_F32 && lane < nvalid && tl.n0 < p.N) {
-        // this lane's residual row into L2 while the accumulator is still
-        // being computed, so that the epilogue's chunk loads do not each
-        // wait for DRAM
-        const int esz = p.resid_f32 ? 4 : 2;
-        const char* r = static_cast<const char*>(tl.g ? p.resid_src[1] : p.resid_src[0]) +
-                        (static_cast<long long>(tl.m0 + off + lane - tl.row_base) * p.N + tl.n0) * esz;
-        for (int j = 0; j < PN * esz / 128; ++j) prefetch_l2(r + 128 * j);
+      const float bias = on && w.k0 == 0 ? __bfloat162float(__ldg((tl.g ? p.bias[1] : p.bias[0]) + ch.feat)) : 0.f;
+      const float wscale = FP8 && on ? __ldg((tl.g ? p.b_scale[1] : p.b_scale[0]) + ch.feat) : 1.f;
+      const void* resid = tl.g ? p.resid_src[1] : p.resid_src[0];
+      uint32_t rn[32];
+      const bool with_resid = epi == EPI_BIAS_RESIDIN_F32 && on;
+      if (with_resid) {
+        // this warp's residual rows into L2 while the accumulator is still
+        // being computed, and the first chunk of them into registers
+        const int esz = resid_f32 ? 4 : 2;
+        for (int c = half + 2; c < tl.units; c += 2) {
+          const int r = tl.r0 + c * UNIT + lane;
+          if (r < tl.rows)
+            prefetch_l2(static_cast<const char*>(resid) + (static_cast<long long>(r) * N + (ch.feat - lane)) * esz);
+        }
+        const int r = tl.r0 + half * UNIT;
+        epi_load_resid(resid, resid_f32, r, half < tl.units ? tl.rows - r : 0, ch.feat, N, rn);
       }
       if (!mbar_wait_warp(&tfull[acc], acc_phase, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 5)) break;
       tc_fence_after();
-      EpiSlab sl;
-      sl.g = tl.g;
-      sl.row0 = tl.m0 + off;
-      sl.nvalid = nvalid;
-      sl.row_base = tl.row_base;
-      sl.n0 = tl.n0;
-      const uint32_t taddr = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * PN);
-      const int a = acc;
-      epilogue_warp<PN>(p, &tmOut, taddr, sl, bpre, escale, stage, buf, [&] {
+      const uint32_t taddr =
+          tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * UNIT * MAXU);
+#pragma unroll 1
+      for (int c = half; c < tl.units; c += 2) {
+        float v[32];
+        tmem_ld32(taddr + c * UNIT, v);
+        const int r = tl.r0 + c * UNIT;
+        uint32_t rc[32];
+        if (with_resid) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) rc[j] = rn[j];
+          if (c + 2 < tl.units)
+            epi_load_resid(resid, resid_f32, r + 2 * UNIT, tl.rows - (r + 2 * UNIT), ch.feat, N, rn);
+        }
+        ch.nvalid = min(UNIT, tl.rows - r);
+        ch.row = tl.row_base + r;
+        float rscale = 0.f;
+        if (FP8 && lane < ch.nvalid) rscale = __ldg(p.a_scale + ch.row + lane);
+        tmem_ld_wait_regs(v);
+        if (c + 2 >= tl.units) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(&tempty[acc]), 0));
+        }
+        if (!on) continue;
+        if (FP8) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] *= __shfl_sync(0xffffffffu, rscale, j) * wscale;
+        }
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] += bias;
+        if (epi == EPI_BIAS_GELU_F16) {
+          epi_store16<true>(p.out, N, ch, v);
+        } else if (epi == EPI_BIAS_BF16) {
+          epi_store16<false>(p.out, N, ch, v);
+        } else if (epi == EPI_BIAS_RESID_F32) {
+          epi_store32<true>(p.out, N, ch, v);
+        } else {
+          epi_add_resid(resid_f32, rc, v);
+          epi_store32<false>(p.out, N, ch, v);
+        }
+      }
+      if (half >= tl.units) {  // a one-unit tile has no chunk for this warp
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(&tempty[a]), 0));
-      });
+        if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(&tempty[acc]), 0));
+      }
       acc ^= 1;
       if (acc == 0) acc_phase ^= 1u;
     }
-    epilogue_drain();
   }
 
   tc_fence_before();
@@ -425,44 +526,38 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 
 }  // namespace
 
-bool gemm_pair_supported(const GemmArgs& a) { return a.K % (a.fp8 ? 128 : BK) == 0 && a.N % PN == 0; }
-
-cudaError_t launch_gemm_pair(const GemmArgs& a, int num_sms, cudaStream_t st) {
-  if (!gemm_pair_supported(a)) return cudaErrorInvalidValue;
-  CUtensorMap tA, tB0, tB1;
-  // FP8: bytes are the elements, 128 per swizzled row (box 128 x 128)
+cudaError_t launch_gemm(const GemmArgs& a, int num_sms, cudaStream_t st) {
+  // FP8: bytes are the elements, 128 per swizzled row
   const TmapType tt = a.fp8 ? TMAP_U8 : TMAP_BF16;
   const uint32_t bk = a.fp8 ? 128 : BK;
-  if (!encode_tmap_2d(&tA, tt, a.A, a.K, a.R, a.K, bk, 128)) return cudaErrorInvalidValue;
-  if (!encode_tmap_2d(&tB0, tt, a.g[0].weight ? a.g[0].weight : a.g[1].weight, a.K, a.N, a.K, bk, 128))
-    return cudaErrorInvalidValue;
-  if (!encode_tmap_2d(&tB1, tt, a.g[1].weight ? a.g[1].weight : a.g[0].weight, a.K, a.N, a.K, bk, 128))
-    return cudaErrorInvalidValue;
-  CUtensorMap tOut;
-  if (!encode_epilogue_map(&tOut, a)) return cudaErrorInvalidValue;
+  if (a.K % bk != 0 || a.N % 128 != 0) return cudaErrorInvalidValue;
+  Maps m;
+  for (int i = 0; i < 4; ++i)
+    if (!encode_tmap_2d(&m.x[i], tt, a.A, a.K, a.R, a.K, bk, 128u >> i)) return cudaErrorInvalidValue;
+  for (int g = 0; g < 2; ++g) {
+    const void* wg = a.g[g].weight ? a.g[g].weight : a.g[1 - g].weight;
+    if (!encode_tmap_2d(&m.w[g], tt, wg, a.K, a.N, a.K, bk, 128)) return cudaErrorInvalidValue;
+  }
   Params p;
   p.N = a.N;
   p.K = a.K;
-  // format code 0: fp16 for kind::f16, E4M3 for kind::f8f6f4
-  p.idesc = idesc_kind_f16(PM, PN, 0, 0, (a.op_f16 || a.fp8) ? 0 : 1);
+  // format code 0: fp16 for kind::f16, E4M3 for kind::f8f6f4; the N field is set per tile
+  p.idesc = idesc_kind_f16(PF, 0, 0, 0, (a.op_f16 || a.fp8) ? 0 : 1);
   p.a_scale = a.a_scale;
-  p.b_scale[0] = a.g[0].w_scale;
-  p.b_scale[1] = a.g[1].w_scale;
-  long long upper = 0;
+  long long units = 0;
   for (int g = 0; g < 2; ++g) {
+    p.b_scale[g] = a.g[g].w_scale;
     p.row_base[g] = a.g[g].row_base;
     p.rows_static[g] = a.g[g].rows_dev ? a.g[g].rows_cap : a.g[g].rows_static;
     p.rows_dev[g] = a.g[g].rows_dev;
     p.bias[g] = static_cast<const __nv_bfloat16*>(a.g[g].bias);
-    upper += (a.g[g].rows_cap + PM - 1) / PM;
+    p.resid_src[g] = a.resid_src[g];
+    units += (a.g[g].rows_cap + UNIT - 1) / UNIT;
   }
-  upper *= a.N / PN;
   p.epilogue = a.epilogue;
   p.out = a.out;
-  p.resid_src[0] = a.resid_src[0];
-  p.resid_src[1] = a.resid_src[1];
   p.resid_f32 = a.resid_f32;
-  if (upper <= 0) return cudaSuccess;
+  if (units <= 0) return cudaSuccess;
   auto* kern = a.fp8 ? gemm2_kernel<true> : gemm2_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
   if (e != cudaSuccess) return e;
@@ -487,15 +582,13 @@ cudaError_t launch_gemm_pair(const GemmArgs& a, int num_sms, cudaStream_t st) {
     }
     max_pairs = n;
   }
-  const long long pairs = upper < max_pairs ? upper : max_pairs;
-  return launch_pdl(kern, dim3(static_cast<int>(2 * pairs)), dim3(THREADS), SMEM_BYTES, st, tA, tB0, tB1, tOut,
-                    p);
+  return launch_pdl(kern, dim3(2 * max_pairs), dim3(THREADS), SMEM_BYTES, st, m, p);
 }
 
-int gemm2_take_device_error() {
+int gemm_take_device_error() {
   int v = 0, z = 0;
-  if (cudaMemcpyFromSymbol(&v, g_gemm2_err, sizeof(int)) != cudaSuccess) return -1;
-  if (v) cudaMemcpyToSymbol(g_gemm2_err, &z, sizeof(int));
+  if (cudaMemcpyFromSymbol(&v, g_gemm_err, sizeof(int)) != cudaSuccess) return -1;
+  if (v) cudaMemcpyToSymbol(g_gemm_err, &z, sizeof(int));
   return v;
 }
 

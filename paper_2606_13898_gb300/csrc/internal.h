@@ -55,7 +55,7 @@ cudaError_t launch_sobel_select(const float* img, int B, int H, int W, int C, in
                                 const uint8_t* mask, int radius, float threshold, uint8_t* keep, void* ws,
                                 int num_sms, cudaStream_t st);
 
-// ---- tcgen05 grouped GEMM (gemm_tc.cu)
+// ---- tcgen05 grouped GEMM on CTA pairs (gemm2_tc.cu)
 enum GemmEpilogue : int {
   EPI_BIAS_BF16 = 0,      // out_bf16 = acc + bias
   EPI_BIAS_GELU_F16 = 1,  // out_f16 = gelu_tanh(acc + bias)   (saturating)
@@ -79,9 +79,9 @@ struct GemmGroupArgs {
 
 struct GemmArgs {
   const void* A;  // [R, K] row space, bf16 (op_f16 = 0) or fp16 (op_f16 = 1); W_g the same type
-  int R, N, K;
+  int R, N, K;    // N a multiple of 128, K of 64 (128 with fp8)
   int op_f16;
-  int fp8 = 0;                     // A and W_g e4m3 (kind::f8f6f4), pair kernel only
+  int fp8 = 0;                     // A and W_g e4m3 (kind::f8f6f4)
   const float* a_scale = nullptr;  // fp8: dequantisation scale per row of A
   GemmGroupArgs g[2];
   int epilogue;
@@ -94,11 +94,6 @@ struct GemmArgs {
 
 cudaError_t launch_gemm(const GemmArgs& a, int num_sms, cudaStream_t st);
 int gemm_take_device_error();
-
-// ---- tcgen05 grouped GEMM on CTA pairs, 256x256 tiles (gemm2_tc.cu)
-bool gemm_pair_supported(const GemmArgs& a);
-cudaError_t launch_gemm_pair(const GemmArgs& a, int num_sms, cudaStream_t st);
-int gemm2_take_device_error();
 
 // ---- tcgen05 joint varlen attention (attn_tc.cu)
 struct AttnArgs {
@@ -124,7 +119,7 @@ int set_error(int status, const char* msg);
 int check_block_shape(const hilo_shape* shape);
 
 // ---- tensor maps (api.cu): 2-D, row-major, 128-byte swizzled boxes
-enum TmapType : int { TMAP_BF16 = 0, TMAP_F16 = 1, TMAP_F32 = 2, TMAP_U8 = 3 };
+enum TmapType : int { TMAP_BF16 = 0, TMAP_U8 = 1 };  // 16-bit elements (bf16 and fp16 alike), bytes
 bool encode_tmap_2d(CUtensorMap* map, TmapType type, const void* base, uint64_t inner, uint64_t outer,
                     uint64_t row_stride_elems, uint32_t box_inner, uint32_t box_outer);
 bool encode_tmap_bf16_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer,

@@ -60,8 +60,8 @@ __global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float
                                                                      float* __restrict__ tokmax,
                                                                      uint32_t* __restrict__ tilemax, int H,
                                                                      int W, int vec_ok) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   constexpr int TOK_Y = TILE_Y / P, TOK_X = TILE_X / P;
   static_assert(TOK_Y * TOK_X <= 32, "token maxima of a tile fit one warp");
   __shared__ float tile[C][TILE_Y + 2][TILE_X + 2];
@@ -221,8 +221,8 @@ __global__ void __launch_bounds__(KEEP_T * KEEP_T) sobel_keep_kernel(const float
                                                                    int ntiles, const uint8_t* __restrict__ mask,
                                                                    uint8_t* __restrict__ keep, int H, int W,
                                                                    int radius, float threshold) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __shared__ uint8_t mt[KEEP_T + 2 * MAX_RADIUS][KEEP_T + 2 * MAX_RADIUS];
   __shared__ uint32_t wred[KEEP_T * KEEP_T / 32];
   const int b = blockIdx.z;
