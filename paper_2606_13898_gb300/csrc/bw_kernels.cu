@@ -158,6 +158,7 @@ struct SelectShared {
   int warp_tot3[3][32];
   int sel_digit;
   int sel_k;
+  int sel_all;
 };
 
 // Exclusive scans of three ints per thread at once (one pass of barriers).
@@ -196,35 +197,38 @@ __device__ __forceinline__ void block_excl_scan3(int& a, int& b, int& c, int (*w
   __syncthreads();
 }
 
-// MSB-first radix select over the candidates (cand[i] != 0, or every key when
-// cand is null): the key of the k-th largest candidate (1 <= k <=
-// #candidates) and how many candidates with exactly that key belong to the
-// top k (those with the lowest token ids). The passes alternate between two
-// histograms, so clearing the next one needs no barrier of its own.
-__device__ void radix_select(const uint32_t* keys, const uint8_t* cand, int N, int k,
-                             SelectShared& sh, uint32_t& thr, int& take) {
+// MSB-first radix select over the candidates (bit i of cand: key[i] of this
+// thread): the key of the k-th largest candidate of the block (1 <= k <=
+// #candidates) and how many candidates with exactly that key belong to the top k
+// (those with the lowest token ids). The passes alternate between two
+// histograms, so clearing the next one needs no barrier of its own. A pass whose
+// digit is taken whole ends the search: every candidate with the prefix so far
+// ranks in the top k, so the prefix is the threshold, with all its equals.
+template <int CH>
+__device__ __forceinline__ void radix_select(const uint32_t (&key)[CH], uint32_t cand, int k, SelectShared& sh,
+                                             uint32_t& thr, int& take) {
   uint32_t prefix = 0, pmask = 0;
   int kk = k;
   if (threadIdx.x < 256) sh.hist[0][threadIdx.x] = 0;
   __syncthreads();
   int h = 0;
+#pragma unroll 1
   for (int shift = 24; shift >= 0; shift -= 8, h ^= 1) {
     int* hist = sh.hist[h];
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const uint32_t key = keys[i];
-      if ((!cand || cand[i]) && (key & pmask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
-    }
+#pragma unroll
+    for (int i = 0; i < CH; ++i)
+      if (((cand >> i) & 1u) && (key[i] & pmask) == prefix) atomicAdd(&hist[(key[i] >> shift) & 255u], 1);
     if (threadIdx.x >= blockDim.x - 256) sh.hist[h ^ 1][threadIdx.x - (blockDim.x - 256)] = 0;
     __syncthreads();
     if (threadIdx.x < 32) {
       const int lane = threadIdx.x;
       // lane L covers digits 255-8L .. 248-8L (descending)
-      int cnt[8], lsum = 0;
+      const int4 lo = *reinterpret_cast<const int4*>(hist + 248 - 8 * lane);
+      const int4 hi = *reinterpret_cast<const int4*>(hist + 252 - 8 * lane);
+      const int cnt[8] = {hi.w, hi.z, hi.y, hi.x, lo.w, lo.z, lo.y, lo.x};
+      int lsum = 0;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        cnt[j] = hist[255 - 8 * lane - j];
-        lsum += cnt[j];
-      }
+      for (int j = 0; j < 8; ++j) lsum += cnt[j];
       int incl = lsum;
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
@@ -232,74 +236,62 @@ __device__ void radix_select(const uint32_t* keys, const uint8_t* cand, int N, i
         if (lane >= off) incl += n;
       }
       const int excl = incl - lsum;
-      const bool here = excl < kk && kk <= incl;
-      if (here) {
-        int c = excl;
+      if (excl < kk && kk <= incl) {
+        int c = excl, dig = 0, left = 0, all = 0;
+        bool found = false;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          if (c + cnt[j] >= kk) {
-            sh.sel_digit = 255 - 8 * lane - j;
-            sh.sel_k = kk - c;
-            break;
+          if (!found && c + cnt[j] >= kk) {
+            found = true;
+            dig = 255 - 8 * lane - j;
+            left = kk - c;
+            all = left == cnt[j];
           }
           c += cnt[j];
         }
+        sh.sel_digit = dig;
+        sh.sel_k = left;
+        sh.sel_all = all;
       }
     }
     __syncthreads();
-    // sel_digit / sel_k are rewritten only after the next pass's barrier,
-    // which every thread reaches after these reads
+    // sel_* are rewritten only after the next pass's barrier, which every
+    // thread reaches after these reads
     prefix |= static_cast<uint32_t>(sh.sel_digit) << shift;
     pmask |= 255u << shift;
     kk = sh.sel_k;
+    if (sh.sel_all) break;
   }
   thr = prefix;
   take = kk;
 }
 
-// Marks sel[i] = 1 for the top-k candidates under (key desc, index asc).
-__device__ void mark_topk(const uint32_t* keys, const uint8_t* cand, uint8_t* sel, int N, int k,
-                          SelectShared& sh) {
-  int ncand = N;  // cand == nullptr: every key is a candidate
-  if (cand) {
-    int c = 0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) c += cand[i] ? 1 : 0;
-    ncand = block_sum(c, sh.warp_tot);
-  }
-  if (k <= 0) {
-    for (int i = threadIdx.x; i < N; i += blockDim.x) sel[i] = 0;
-    __syncthreads();
-    return;
-  }
-  if (k >= ncand) {
-    for (int i = threadIdx.x; i < N; i += blockDim.x) sel[i] = (!cand || cand[i]) ? 1 : 0;
-    __syncthreads();
-    return;
-  }
+// Bits of this thread's top-k candidates under (key desc, index asc); thread t
+// holds the tokens t CH .. t CH + CH - 1.
+template <int CH>
+__device__ __forceinline__ uint32_t topk_bits(const uint32_t (&key)[CH], uint32_t cand, int ncand, int k,
+                                              SelectShared& sh) {
+  if (k <= 0) return 0u;
+  if (k >= ncand) return cand;
   uint32_t thr;
   int take;
-  radix_select(keys, cand, N, k, sh, thr, take);
-  // rank of equal-key candidates in index order: contiguous chunk per thread
-  const int chunk = (N + blockDim.x - 1) / blockDim.x;
-  const int i0 = threadIdx.x * chunk;
-  const int i1 = min(N, i0 + chunk);
-  int eq = 0;
-  for (int i = i0; i < i1; ++i) eq += ((!cand || cand[i]) && keys[i] == thr) ? 1 : 0;
-  int rank = block_excl_scan(eq, sh.warp_tot, nullptr);
-  for (int i = i0; i < i1; ++i) {
-    uint8_t v = 0;
-    if (!cand || cand[i]) {
-      const uint32_t key = keys[i];
-      if (key > thr) {
-        v = 1;
-      } else if (key == thr) {
-        v = rank < take ? 1 : 0;
-        ++rank;
-      }
-    }
-    sel[i] = v;
+  radix_select<CH>(key, cand, k, sh, thr, take);
+  uint32_t gt = 0, eq = 0;
+#pragma unroll
+  for (int i = 0; i < CH; ++i) {
+    gt |= (key[i] > thr ? 1u : 0u) << i;
+    eq |= (key[i] == thr ? 1u : 0u) << i;
   }
-  __syncthreads();
+  gt &= cand;
+  eq &= cand;
+  int rank = block_excl_scan(__popc(eq), sh.warp_tot, nullptr);
+  // the equals of lowest index, as many as are left to take
+  while (eq && rank < take) {
+    gt |= eq & (0u - eq);
+    eq &= eq - 1;
+    ++rank;
+  }
+  return gt;
 }
 
 // Packed rows of one image from its labels (in shared memory): row_src and
@@ -394,124 +386,182 @@ __device__ void compact_image(const uint8_t* lab, int b, int H, int W, int level
   }
 }
 
-// Labels and per-image counts. One CTA per image. With a single image
-// (fused != 0) the same CTA also writes cu_img and the packed rows, as
-// nothing depends on other images. granular != 0 is the window-granular
-// split: every pooling window takes the finest class of its members (an
-// aligned 2x2 window with a kept member is kept whole; with two levels an
-// aligned 4x4 block is pooled 4x4 only when all its members rank below the
-// k_mid cut, else its non-kept members are pooled 2x2).
-template <bool GRANULAR, bool LFMODE>
+// Labels and per-image counts. One CTA per image; thread t owns the tokens
+// t CH .. t CH + CH - 1, whose scores stay in its registers (CH is the smallest of
+// 4, 8, 16, 32 for which 1024 threads cover the image, and no more threads are
+// launched than own tokens, but at least 256). With a single image (fused != 0)
+// the same CTA also writes cu_img and the packed rows, as nothing depends on
+// other images. granular != 0 is the window-granular split: every pooling window
+// takes the finest class of its members (an aligned 2x2 window with a kept member
+// is kept whole; with two levels an aligned 4x4 block is pooled 4x4 only when all
+// its members rank below the k_mid cut, else its non-kept members are pooled 2x2).
+// Bound by one SM's latency: barriers, shared atomics and dependent loads. With
+// the keys in shared memory and re-read by each pass (contiguous chunks per
+// thread, up to 16-way bank conflicts) two levels on 128x128 took 66 us.
+template <int CH, bool GRANULAR, bool LFMODE>
 __global__ void __launch_bounds__(SPLIT_THREADS) split_select_kernel(
     const float* __restrict__ score, const uint8_t* __restrict__ mask,
     const int32_t* __restrict__ k_keep, const int32_t* __restrict__ k_mid, uint8_t* labels_out,
     int32_t* counts, int H, int W, int levels, int lf_arg, int fused, int32_t* cu_img,
     int32_t* row_src, int32_t* tok_row) {
   // the modes are template parameters, so the plain split carries none of
-  // their code (this CTA has 1024 threads and at most 64 registers each)
+  // their code (this CTA has up to 1024 threads and at most 64 registers each)
   constexpr bool granular = GRANULAR;
   const int lf = LFMODE ? lf_arg : 0;
   pdl_wait();
   pdl_trigger();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ SelectShared sh;
+  __shared__ __align__(16) SelectShared sh;
   const int N = H * W;
   const int b = blockIdx.x;
-  uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);
-  uint8_t* lab = reinterpret_cast<uint8_t*>(keys + N);
-  uint8_t* cand = lab + N;
-  uint8_t* sel = cand + N;
+  uint8_t* lab = smem_raw;  // the labels, padded to the threads' tokens
+  const long long base = static_cast<long long>(b) * N;
   const int k = min(max(k_keep[b], 0), N);
   const int km = levels == 2 ? min(max(k_mid[b], 0), N) : 0;
-  // the first selection has every token as a candidate, so `cand` holds the
-  // mask until the keep labels are formed
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+  const int i0 = static_cast<int>(threadIdx.x) * CH;
+  // N is a multiple of 4 (H and W are even), so four tokens at a time are all
+  // inside or all outside the image; wide loads only where the arrays allow them
+  const bool wide = ((reinterpret_cast<uintptr_t>(score + base) & 15) == 0) &&
+                    ((reinterpret_cast<uintptr_t>(mask + base) & 3) == 0);
+  uint32_t key[CH];
+  uint32_t keep = 0, every = 0;  // bit i: token i0 + i is masked (then: kept) / exists
+#pragma unroll
+  for (int q = 0; q < CH / 4; ++q) {
+    const int i = i0 + 4 * q;
+    uint32_t m = 0;
+    float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < N) {
+      every |= 15u << (4 * q);
+      if (wide) {
+        f = __ldg(reinterpret_cast<const float4*>(score + base + i));
+        m = __ldg(reinterpret_cast<const uint32_t*>(mask + base + i));
+      } else {
+        f = make_float4(score[base + i], score[base + i + 1], score[base + i + 2], score[base + i + 3]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) m |= static_cast<uint32_t>(mask[base + i + j]) << (8 * j);
+      }
+    }
     // scores are >= +0, so their IEEE bit patterns order like the values
-    keys[i] = __float_as_uint(score[static_cast<long long>(b) * N + i]);
-    cand[i] = mask[static_cast<long long>(b) * N + i];
+    key[4 * q] = __float_as_uint(f.x);
+    key[4 * q + 1] = __float_as_uint(f.y);
+    key[4 * q + 2] = __float_as_uint(f.z);
+    key[4 * q + 3] = __float_as_uint(f.w);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) keep |= ((m >> (8 * j)) & 255u ? 1u : 0u) << (4 * q + j);
   }
-  __syncthreads();
-  mark_topk(keys, nullptr, sel, N, k, sh);
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    const bool keep = sel[i] || cand[i];
-    lab[i] = keep ? HILO_LABEL_KEEP : (lf ? HILO_LABEL_LF : HILO_LABEL_POOL2);
-    cand[i] = keep ? 0 : 1;
-  }
-  __syncthreads();
+  keep |= topk_bits<CH>(key, every, N, k, sh);
+  // labels of this thread's tokens: a byte each, low = the tokens of `coarse`
+  auto put_labels = [&](uint32_t kept, uint32_t coarse) {
+#pragma unroll
+    for (int q = 0; q < CH / 4; ++q) {
+      uint32_t v = 0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int i = 4 * q + j;
+        const uint32_t l = (kept >> i) & 1u ? HILO_LABEL_KEEP
+                                            : (lf ? HILO_LABEL_LF
+                                                  : ((coarse >> i) & 1u ? HILO_LABEL_POOL4 : HILO_LABEL_POOL2));
+        v |= l << (8 * j);
+      }
+      if (i0 + 4 * q < N) *reinterpret_cast<uint32_t*>(lab + i0 + 4 * q) = v;
+    }
+  };
   if (granular) {
     // one thread per 2x2 window: a window with a kept member is kept whole
+    put_labels(keep, 0u);
+    __syncthreads();
     const int W2 = W >> 1, nw = (H >> 1) * W2;
     for (int w = threadIdx.x; w < nw; w += blockDim.x) {
       const int t = (2 * (w / W2)) * W + 2 * (w % W2);
-      if (lab[t] == HILO_LABEL_KEEP || lab[t + 1] == HILO_LABEL_KEEP || lab[t + W] == HILO_LABEL_KEEP ||
-          lab[t + W + 1] == HILO_LABEL_KEEP) {
-        lab[t] = lab[t + 1] = lab[t + W] = lab[t + W + 1] = HILO_LABEL_KEEP;
-        cand[t] = cand[t + 1] = cand[t + W] = cand[t + W + 1] = 0;
-      }
+      uint16_t* l0 = reinterpret_cast<uint16_t*>(lab + t);
+      uint16_t* l1 = reinterpret_cast<uint16_t*>(lab + t + W);
+      // labels are 0 (kept) or 1 here, so a window is all pooled or has a kept member
+      if ((*l0 & *l1) != 0x0101u) *l0 = *l1 = 0;
     }
     __syncthreads();
+    keep = 0;
+#pragma unroll
+    for (int i = 0; i < CH; ++i)
+      if (i0 + i < N && lab[i0 + i] == HILO_LABEL_KEEP) keep |= 1u << i;
   }
+  uint32_t coarse = 0;
   if (levels == 2) {
-    mark_topk(keys, cand, sel, N, km, sh);
-    for (int i = threadIdx.x; i < N; i += blockDim.x)
-      if (cand[i]) lab[i] = sel[i] ? HILO_LABEL_POOL2 : HILO_LABEL_POOL4;
+    const uint32_t cand = every & ~keep;
+    const int ncand = block_sum(__popc(cand), sh.warp_tot);
+    coarse = cand & ~topk_bits<CH>(key, cand, ncand, km, sh);
+  }
+  if (!granular || levels == 2) put_labels(keep, coarse);
+  __syncthreads();
+  if (granular && levels == 2) {
+    // one thread per 4x4 block: pooled 4x4 only when every member is
+    const int W4 = W >> 2, nb = (H >> 2) * W4;
+    for (int v = threadIdx.x; v < nb; v += blockDim.x) {
+      const int t = (4 * (v / W4)) * W + 4 * (v % W4);
+      bool all4 = true;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) all4 &= *reinterpret_cast<const uint32_t*>(lab + t + i * W) == 0x02020202u;
+      if (all4) continue;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (lab[t + i * W + j] == HILO_LABEL_POOL4) lab[t + i * W + j] = HILO_LABEL_POOL2;
+    }
     __syncthreads();
-    if (granular) {
-      // one thread per 4x4 block: pooled 4x4 only when every member is
-      const int W4 = W >> 2, nb = (H >> 2) * W4;
-      for (int v = threadIdx.x; v < nb; v += blockDim.x) {
-        const int t = (4 * (v / W4)) * W + 4 * (v % W4);
-        bool all4 = true;
+  }
+  // labels out
+  const bool wide_out = (reinterpret_cast<uintptr_t>(labels_out + base) & 3) == 0;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+  for (int q = 0; q < CH / 4; ++q) {
+    const int i = i0 + 4 * q;
+    if (i >= N) continue;
+    const uint32_t v = *reinterpret_cast<const uint32_t*>(lab + i);
+    if (wide_out) {
+      *reinterpret_cast<uint32_t*>(labels_out + base + i) = v;
+    } else {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) all4 &= lab[t + i * W + j] == HILO_LABEL_POOL4;
-        if (all4) continue;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (lab[t + i * W + j] == HILO_LABEL_POOL4) lab[t + i * W + j] = HILO_LABEL_POOL2;
-      }
-      __syncthreads();
+      for (int j = 0; j < 4; ++j) labels_out[base + i + j] = static_cast<uint8_t>(v >> (8 * j));
     }
   }
-  // Per thread, a contiguous chunk of tokens, of 2x2 windows and of 4x4
+  // Per thread, its tokens and a contiguous chunk of 2x2 windows and of 4x4
   // windows: kept tokens, and windows holding at least one member of their
   // class, are counted, and one three-way block scan gives both the image's
   // counts and each thread's first packed row.
-  const int tch = (N + blockDim.x - 1) / blockDim.x;
-  const int i0 = min(N, static_cast<int>(threadIdx.x) * tch), i1 = min(N, i0 + tch);
   // (low-frequency mode: the "2x2 windows" below are the lf x lf windows,
   // every one of which has a row)
   const int W2 = lf ? W / lf : W >> 1, nw2 = (lf ? H / lf : H >> 1) * W2;
-  const int wch = (nw2 + blockDim.x - 1) / blockDim.x;
+  const int wch = (nw2 + blockDim.x - 1) / blockDim.x;  // at most 32
   const int w0 = min(nw2, static_cast<int>(threadIdx.x) * wch), w1 = min(nw2, w0 + wch);
   const int W4 = W >> 2, nw4 = levels == 2 ? (H >> 2) * W4 : 0;
   const int vch = (nw4 + blockDim.x - 1) / blockDim.x;
   const int v0 = min(nw4, static_cast<int>(threadIdx.x) * vch), v1 = min(nw4, v0 + vch);
-  auto has2 = [&](int w) {
-    if (lf) return true;
-    const int t = (2 * (w / W2)) * W + 2 * (w % W2);
-    return lab[t] == HILO_LABEL_POOL2 || lab[t + 1] == HILO_LABEL_POOL2 || lab[t + W] == HILO_LABEL_POOL2 ||
-           lab[t + W + 1] == HILO_LABEL_POOL2;
+  // bit j of a label pair / quad: the member has the class
+  auto any2 = [&](int t) {  // a 2x2 window's POOL2 members, bits 0..3 in raster order
+    const uint32_t a = *reinterpret_cast<const uint16_t*>(lab + t), c = *reinterpret_cast<const uint16_t*>(lab + t + W);
+    return ((a & 255u) == HILO_LABEL_POOL2 ? 1u : 0u) | ((a >> 8) == HILO_LABEL_POOL2 ? 2u : 0u) |
+           ((c & 255u) == HILO_LABEL_POOL2 ? 4u : 0u) | ((c >> 8) == HILO_LABEL_POOL2 ? 8u : 0u);
   };
-  auto has4 = [&](int v) {
-    const int t = (4 * (v / W4)) * W + 4 * (v % W4);
-    bool any = false;
+  auto any4 = [&](int t) {  // any POOL4 member (label 2: bit 1 of a byte, and not 3 in this mode)
+    uint32_t o = 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) any |= lab[t + i * W + j] == HILO_LABEL_POOL4;
-    return any;
+    for (int i = 0; i < 4; ++i) o |= *reinterpret_cast<const uint32_t*>(lab + t + i * W);
+    return (o & 0x02020202u) != 0;
   };
-  int rk = 0, r2 = 0, r4 = 0;
-  for (int i = i0; i < i1; ++i) {
-    labels_out[static_cast<long long>(b) * N + i] = lab[i];
-    rk += lab[i] == HILO_LABEL_KEEP ? 1 : 0;
+  int rk = __popc(keep), r2 = 0, r4 = 0;
+  uint32_t has2 = 0, has4 = 0;
+  if (lf) {
+    r2 = w1 - w0;
+  } else {
+    int row = w0 / W2, col = w0 - row * W2;
+    for (int w = w0; w < w1; ++w) {
+      if (any2(2 * row * W + 2 * col)) has2 |= 1u << (w - w0);
+      if (++col == W2) col = 0, ++row;
+    }
+    r2 = __popc(has2);
   }
-  for (int w = w0; w < w1; ++w) r2 += has2(w) ? 1 : 0;
-  for (int v = v0; v < v1; ++v) r4 += has4(v) ? 1 : 0;
+  for (int v = v0; v < v1; ++v)
+    if (any4((4 * (v / W4)) * W + 4 * (v % W4))) has4 |= 1u << (v - v0);
+  r4 = __popc(has4);
   int nk, n2, n4;
   block_excl_scan3(rk, r2, r4, sh.warp_tot3, nk, n2, n4);
   if (threadIdx.x == 0) {
@@ -525,35 +575,38 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_select_kernel(
   }
   if (!fused) return;
   // packed rows: kept tokens (raster order), then 2x2, then 4x4 windows
-  int32_t* trow = tok_row + static_cast<long long>(b) * N;
-  for (int i = i0; i < i1; ++i)
-    if (lab[i] == HILO_LABEL_KEEP) {
-      row_src[rk] = i;
-      trow[i] = rk;
-      ++rk;
-    }
+  int32_t* trow = tok_row + base;
+  for (uint32_t m = keep; m; m &= m - 1) {
+    const int i = i0 + __ffs(m) - 1;
+    row_src[rk] = i;
+    trow[i] = rk;
+    ++rk;
+  }
   r2 += nk;
-  for (int w = w0; w < w1; ++w) {
-    if (!has2(w)) continue;
-    row_src[r2] = w;
-    if (lf) {
+  if (lf) {
+    for (int w = w0; w < w1; ++w, ++r2) {
+      row_src[r2] = w;
       const int t0 = (lf * (w / W2)) * W + lf * (w % W2);
       for (int i = 0; i < lf; ++i)
         for (int j = 0; j < lf; ++j)
           if (lab[t0 + i * W + j] != HILO_LABEL_KEEP) trow[t0 + i * W + j] = r2;
-      ++r2;
-      continue;
     }
-    const int t = (2 * (w / W2)) * W + 2 * (w % W2);
-    const int mem[4] = {t, t + 1, t + W, t + W + 1};
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (lab[mem[j]] == HILO_LABEL_POOL2) trow[mem[j]] = r2;
-    ++r2;
+  } else {
+    for (uint32_t m = has2; m; m &= m - 1) {
+      const int w = w0 + __ffs(m) - 1;
+      const int t = (2 * (w / W2)) * W + 2 * (w % W2);
+      const uint32_t mem = any2(t);
+      row_src[r2] = w;
+      if (mem & 1u) trow[t] = r2;
+      if (mem & 2u) trow[t + 1] = r2;
+      if (mem & 4u) trow[t + W] = r2;
+      if (mem & 8u) trow[t + W + 1] = r2;
+      ++r2;
+    }
   }
   r4 += nk + n2;
-  for (int v = v0; v < v1; ++v) {
-    if (!has4(v)) continue;
+  for (uint32_t m = has4; m; m &= m - 1) {
+    const int v = v0 + __ffs(m) - 1;
     const int t = (4 * (v / W4)) * W + 4 * (v % W4);
     row_src[r4] = v;
 #pragma unroll
@@ -576,7 +629,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_compact_kernel(
   const int N = H * W;
   const int b = blockIdx.x;
   uint8_t* lab = smem_raw;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) lab[i] = labels[static_cast<long long>(b) * N + i];
+  const uint8_t* src = labels + static_cast<long long>(b) * N;
+  if ((reinterpret_cast<uintptr_t>(src) & 3) == 0) {  // N is a multiple of 4
+    for (int i = threadIdx.x; i < N / 4; i += blockDim.x)
+      reinterpret_cast<uint32_t*>(lab)[i] = __ldg(reinterpret_cast<const uint32_t*>(src) + i);
+  } else {
+    for (int i = threadIdx.x; i < N; i += blockDim.x) lab[i] = src[i];
+  }
   int base = 0;
   for (int j = 0; j < b; ++j) base += counts[3 * j] + counts[3 * j + 1] + counts[3 * j + 2];
   const int nk = counts[3 * b], n2 = counts[3 * b + 1], n4 = counts[3 * b + 2];
@@ -1138,27 +1197,33 @@ cudaError_t launch_score(const void* x, float* s, int B, int H, int W, int d, in
                     static_cast<const __nv_bfloat16*>(x), s, B, H, W, d);
 }
 
-size_t split_select_smem(int N) { return static_cast<size_t>(N) * 7; }
-size_t split_compact_smem(int N) { return static_cast<size_t>(N); }
+template <bool GRANULAR, bool LFMODE>
+static auto split_kernel_for(int ch) {
+  switch (ch) {
+    case 4: return split_select_kernel<4, GRANULAR, LFMODE>;
+    case 8: return split_select_kernel<8, GRANULAR, LFMODE>;
+    case 16: return split_select_kernel<16, GRANULAR, LFMODE>;
+    default: return split_select_kernel<32, GRANULAR, LFMODE>;
+  }
+}
 
 cudaError_t launch_split(const float* score, const uint8_t* mask, const int32_t* k_keep,
                          const int32_t* k_mid, uint8_t* labels, int32_t* row_src, int32_t* counts,
                          int32_t* cu_img, int32_t* tok_row, int B, int H, int W, int levels,
                          int granular, int lf, cudaStream_t st) {
   const int N = H * W;
-  const size_t sm1 = split_select_smem(N), sm2 = split_compact_smem(N);
-  auto* kern = lf ? split_select_kernel<false, true>
-                  : (granular ? split_select_kernel<true, false> : split_select_kernel<false, false>);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm1));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(split_compact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(sm2));
-  if (e != cudaSuccess) return e;
+  int ch = 4;  // tokens per thread
+  while (ch < 32 && N > ch * SPLIT_THREADS) ch *= 2;
+  int threads = (((N + ch - 1) / ch + 31) / 32) * 32;
+  threads = threads < 256 ? 256 : threads;
+  auto* kern = lf ? split_kernel_for<false, true>(ch)
+                  : (granular ? split_kernel_for<true, false>(ch) : split_kernel_for<false, false>(ch));
   const int fused = B == 1 ? 1 : 0;
-  e = launch_pdl(kern, dim3(B), dim3(SPLIT_THREADS), sm1, st, score, mask, k_keep, k_mid, labels, counts, H, W,
-                 levels, lf, fused, cu_img, row_src, tok_row);
+  // at most 32 KB of labels: no larger shared-memory limit to ask for
+  const cudaError_t e = launch_pdl(kern, dim3(B), dim3(threads), N, st, score, mask, k_keep, k_mid, labels, counts,
+                                   H, W, levels, lf, fused, cu_img, row_src, tok_row);
   if (e != cudaSuccess || fused) return e;
-  return launch_pdl(split_compact_kernel, dim3(B), dim3(SPLIT_THREADS), sm2, st,
+  return launch_pdl(split_compact_kernel, dim3(B), dim3(SPLIT_THREADS), N, st,
                     static_cast<const uint8_t*>(labels), static_cast<const int32_t*>(counts), cu_img,
                     row_src, tok_row, H, W, levels, lf);
 }
@@ -1173,10 +1238,7 @@ cudaError_t launch_pack(const void* x, const uint8_t* labels, const int32_t* row
   if (lf == 4) return launch_pdl(pack_lf_kernel<4>, grid, dim3(256), 0, st, xs, row_src, counts, cu_img, ps, B, H, W, d, cap);
   if (lf == 8) return launch_pdl(pack_lf_kernel<8>, grid, dim3(256), 0, st, xs, row_src, counts, cu_img, ps, B, H, W, d, cap);
   if (lf) return cudaErrorInvalidValue;
-  return launch_pdl(pack_kernel, dim3(grid_for(static_cast<long long>(cap) * PACK_WARPS_PER_ROW, 8, num_sms, 8)),
-                    dim3(256), 0, st,
-                    static_cast<const __nv_bfloat16*>(x), labels, row_src, counts, cu_img,
-                    static_cast<__nv_bfloat16*>(packed), B, H, W, d, cap);
+  return launch_pdl(pack_kernel, grid, dim3(256), 0, st, xs, labels, row_src, counts, cu_img, ps, B, H, W, d, cap);
 }
 
 cudaError_t launch_unpack(const float* out_img, const int32_t* tok_row, float* y, long long ntok,

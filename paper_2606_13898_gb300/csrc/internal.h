@@ -18,8 +18,6 @@ namespace hilo {
 // ---- bandwidth kernels (bw_kernels.cu)
 cudaError_t launch_score(const void* x, float* s, int B, int H, int W, int d, int num_sms,
                          cudaStream_t st);
-size_t split_select_smem(int N);
-size_t split_compact_smem(int N);
 cudaError_t launch_split(const float* score, const uint8_t* mask, const int32_t* k_keep,
                          const int32_t* k_mid, uint8_t* labels, int32_t* row_src, int32_t* counts,
                          int32_t* cu_img, int32_t* tok_row, int B, int H, int W, int levels,
