@@ -408,7 +408,7 @@ static int block_forward_impl(const hilo_shape* shape, const hilo_block_weights*
   stage_mark(0, s);
   // the residual is read from the input by the out-projection epilogue (no
   // fp32 copy of it is made) unless the input already is the output buffer
-  cudaError_t e = hilo::launch_layernorm(in_txt, in_img, in_f32, nullptr, ln, 0, nullptr, cu_img, B, BT, cap, d,
+  cudaError_t e = hilo::launch_layernorm(in_txt, in_img, in_f32, ln, 0, nullptr, cu_img, B, BT, cap, d,
                                          dev->num_sms, s);
   if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward: layernorm 1");
   count(1);
@@ -459,7 +459,7 @@ static int block_forward_impl(const hilo_shape* shape, const hilo_block_weights*
   if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward: out-projection gemm");
   stage_mark(4, s);
   if (shape->mlp) {
-    e = hilo::launch_layernorm(out, out + static_cast<size_t>(BT) * d, 1, nullptr, ln, 1, nullptr, cu_img, B, BT,
+    e = hilo::launch_layernorm(out, out + static_cast<size_t>(BT) * d, 1, ln, 1, nullptr, cu_img, B, BT,
                                cap, d, dev->num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward: layernorm 2");
     count(1);
@@ -568,7 +568,7 @@ static int block_forward_fp8_impl(const hilo_shape* shape, const hilo_block_weig
   const bool in_place_img = in_f32 && BT == 0 && in_img == out;
 
   stage_mark(0, s);
-  cudaError_t e = hilo::launch_layernorm(in_txt, in_img, in_f32, nullptr, q8, 2, qs, cu_img, B, BT, cap, d,
+  cudaError_t e = hilo::launch_layernorm(in_txt, in_img, in_f32, q8, 2, qs, cu_img, B, BT, cap, d,
                                          dev->num_sms, s);
   if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward_fp8: layernorm 1");
   count(1);
@@ -623,7 +623,7 @@ static int block_forward_fp8_impl(const hilo_shape* shape, const hilo_block_weig
   if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward_fp8: out-projection gemm");
   stage_mark(4, s);
   if (shape->mlp) {
-    e = hilo::launch_layernorm(out, out + static_cast<size_t>(BT) * d, 1, nullptr, q8, 2, qs, cu_img, B, BT, cap,
+    e = hilo::launch_layernorm(out, out + static_cast<size_t>(BT) * d, 1, q8, 2, qs, cu_img, B, BT, cap,
                                d, dev->num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward_fp8: layernorm 2");
     count(1);

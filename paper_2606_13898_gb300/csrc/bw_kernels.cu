@@ -952,32 +952,39 @@ __global__ void __launch_bounds__(256) unpack_update_kernel(const float* __restr
 
 // ========================================================== layernorm =====
 //
-// One 128-thread CTA per row of the row space. Rows [0, n_txt) come from
-// in_txt, rows [n_txt, n_txt + cu_img[B]) from in_img (bf16 or fp32). Thread
-// t holds elements 4t + 512k. Writes the normalised row (no affine, eps 1e-6,
-// biased variance) as bf16 or fp16 and, when `resid` is not null, the fp32
-// copy of the input row (the residual stream).
+// A row of the row space per group of 128 threads, three groups per CTA, two
+// CTAs per SM looping over the rows. Rows [0, n_txt) come from in_txt, rows
+// [n_txt, n_txt + cu_img[B]) from in_img (bf16 or fp32). Thread t of a group holds
+// elements 4t + 512k. Writes the normalised row (no affine, eps 1e-6, biased
+// variance) as bf16, fp16 or e4m3.
+// Bound by memory latency: a row is one load round trip, two dependent
+// reductions and a store, so each group loads its next row before it reduces the
+// present one, and every row of a 2400-row block is asked for within two trips.
 
-constexpr int LN_THREADS = 128;
+constexpr int LN_GROUP = 128;
+constexpr int LN_GROUPS = 3;
+constexpr int LN_THREADS = LN_GROUP * LN_GROUPS;
 
-__device__ __forceinline__ float ln_block_sum(float v, float* red) {
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  const float t = (red[0] + red[1]) + (red[2] + red[3]);
-  __syncthreads();
-  return t;
+// Over one group: `red` is 4 floats of its own, used by no other reduction
+// until the group has met at two further barriers or ends its row.
+__device__ __forceinline__ void ln_group_sync() {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + static_cast<int>(threadIdx.x) / LN_GROUP), "n"(LN_GROUP) : "memory");
 }
 
-__device__ __forceinline__ float ln_block_max(float v, float* red) {
+__device__ __forceinline__ float ln_group_sum(float v, float* red) {
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if ((threadIdx.x & 31) == 0) red[(threadIdx.x >> 5) & 3] = v;
+  ln_group_sync();
+  return (red[0] + red[1]) + (red[2] + red[3]);
+}
+
+__device__ __forceinline__ float ln_group_max(float v, float* red) {
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  const float t = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
-  __syncthreads();
-  return t;
+  if ((threadIdx.x & 31) == 0) red[(threadIdx.x >> 5) & 3] = v;
+  ln_group_sync();
+  return fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
 }
 
 // e4m3 row quantisation constants from the row's largest magnitude: inv =
@@ -990,49 +997,67 @@ __device__ __forceinline__ void e4m3_row_scale(float amax, float& inv, float& sc
 
 // ln_mode: 0 bf16, 1 fp16 (saturating), 2 e4m3 per row (ln_scale[r] = the
 // row's dequantisation scale)
-template <int NCH>
-__global__ void __launch_bounds__(LN_THREADS) layernorm_kernel(const void* __restrict__ in_txt,
-                                                               const void* __restrict__ in_img,
-                                                               int in_f32, float* resid,
-                                                               void* __restrict__ ln, int ln_mode,
-                                                               float* __restrict__ ln_scale,
-                                                               const int32_t* __restrict__ cu_img,
-                                                               int B, int n_txt, int cap, int d) {
+template <int NCH, bool F32>
+__global__ void __launch_bounds__(LN_THREADS, 2) layernorm_kernel(const void* __restrict__ in_txt,
+                                                                  const void* __restrict__ in_img,
+                                                                  void* __restrict__ ln, int ln_mode,
+                                                                  float* __restrict__ ln_scale,
+                                                                  const int32_t* __restrict__ cu_img, int B,
+                                                                  int n_txt, int cap, int d) {
   pdl_wait();
   pdl_trigger();
-  __shared__ float red[LN_THREADS / 32];
+  __shared__ float red_s[LN_GROUPS][3][4];
+  const int group = threadIdx.x / LN_GROUP, tid = threadIdx.x % LN_GROUP;
+  float(*red)[4] = red_s[group];
   const int rows = n_txt + min(cu_img[B], cap);
+  const int step = gridDim.x * LN_GROUPS;
   const float inv_d = 1.0f / static_cast<float>(d);
-  for (int r = blockIdx.x; r < rows; r += gridDim.x) {
+  uint4 raw[NCH];  // the next row as it is in memory (bf16: .x and .y)
+  auto load = [&](int r) {
     const long long off = static_cast<long long>(r < n_txt ? r : r - n_txt) * d;
     const void* base = r < n_txt ? in_txt : in_img;
+#pragma unroll
+    for (int t = 0; t < NCH; ++t) {
+      const int c = 512 * t + 4 * tid;
+      raw[t] = make_uint4(0u, 0u, 0u, 0u);
+      if (c < d) {
+        if (F32) {
+          raw[t] = __ldg(reinterpret_cast<const uint4*>(static_cast<const float*>(base) + off + c));
+        } else {
+          const uint2 u = __ldg(reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(base) + off + c));
+          raw[t].x = u.x;
+          raw[t].y = u.y;
+        }
+      }
+    }
+  };
+  int r = blockIdx.x + gridDim.x * group;
+  if (r < rows) load(r);
+  for (; r < rows; r += step) {
     float v[NCH * 4];
 #pragma unroll
     for (int t = 0; t < NCH; ++t) {
-      const int c = 512 * t + 4 * threadIdx.x;
-      if (c < d) {
-        if (in_f32) {
-          const float4 f = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(base) + off + c));
-          v[4 * t] = f.x; v[4 * t + 1] = f.y; v[4 * t + 2] = f.z; v[4 * t + 3] = f.w;
-        } else {
-          const uint2 u = __ldg(reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(base) + off + c));
-          v[4 * t] = __uint_as_float(u.x << 16);
-          v[4 * t + 1] = __uint_as_float(u.x & 0xFFFF0000u);
-          v[4 * t + 2] = __uint_as_float(u.y << 16);
-          v[4 * t + 3] = __uint_as_float(u.y & 0xFFFF0000u);
-        }
+      if (F32) {
+        v[4 * t] = __uint_as_float(raw[t].x);
+        v[4 * t + 1] = __uint_as_float(raw[t].y);
+        v[4 * t + 2] = __uint_as_float(raw[t].z);
+        v[4 * t + 3] = __uint_as_float(raw[t].w);
       } else {
-        v[4 * t] = v[4 * t + 1] = v[4 * t + 2] = v[4 * t + 3] = 0.f;
+        v[4 * t] = __uint_as_float(raw[t].x << 16);
+        v[4 * t + 1] = __uint_as_float(raw[t].x & 0xFFFF0000u);
+        v[4 * t + 2] = __uint_as_float(raw[t].y << 16);
+        v[4 * t + 3] = __uint_as_float(raw[t].y & 0xFFFF0000u);
       }
     }
+    if (r + step < rows) load(r + step);
     float sum = 0.f;
 #pragma unroll
     for (int i = 0; i < NCH * 4; ++i) sum += v[i];
-    const float mean = ln_block_sum(sum, red) * inv_d;
+    const float mean = ln_group_sum(sum, red[0]) * inv_d;
     float sq = 0.f;
 #pragma unroll
     for (int t = 0; t < NCH; ++t) {
-      if (512 * t + 4 * static_cast<int>(threadIdx.x) < d) {
+      if (512 * t + 4 * tid < d) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float e = v[4 * t + i] - mean;
@@ -1040,37 +1065,34 @@ __global__ void __launch_bounds__(LN_THREADS) layernorm_kernel(const void* __res
         }
       }
     }
-    const float rstd = rsqrtf(ln_block_sum(sq, red) * inv_d + 1e-6f);
-    float* rr = resid ? resid + static_cast<long long>(r) * d : nullptr;
+    const float rstd = rsqrtf(ln_group_sum(sq, red[1]) * inv_d + 1e-6f);
     if (ln_mode == 2) {
       float am = 0.f;
 #pragma unroll
       for (int t = 0; t < NCH; ++t)
-        if (512 * t + 4 * static_cast<int>(threadIdx.x) < d) {
+        if (512 * t + 4 * tid < d) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) am = fmaxf(am, fabsf((v[4 * t + i] - mean) * rstd));
         }
       float inv, scale;
-      e4m3_row_scale(ln_block_max(am, red), inv, scale);
+      e4m3_row_scale(ln_group_max(am, red[2]), inv, scale);
       uint8_t* q = static_cast<uint8_t*>(ln) + static_cast<long long>(r) * d;
 #pragma unroll
       for (int t = 0; t < NCH; ++t) {
-        const int c = 512 * t + 4 * threadIdx.x;
+        const int c = 512 * t + 4 * tid;
         if (c >= d) continue;
-        if (rr) *reinterpret_cast<float4*>(rr + c) = make_float4(v[4 * t], v[4 * t + 1], v[4 * t + 2], v[4 * t + 3]);
         *reinterpret_cast<uint32_t*>(q + c) =
             pack_e4m3x4(__fmul_rn((v[4 * t] - mean) * rstd, inv), __fmul_rn((v[4 * t + 1] - mean) * rstd, inv),
                         __fmul_rn((v[4 * t + 2] - mean) * rstd, inv), __fmul_rn((v[4 * t + 3] - mean) * rstd, inv));
       }
-      if (threadIdx.x == 0) ln_scale[r] = scale;
+      if (tid == 0) ln_scale[r] = scale;
       continue;
     }
     uint16_t* lo = static_cast<uint16_t*>(ln) + static_cast<long long>(r) * d;
 #pragma unroll
     for (int t = 0; t < NCH; ++t) {
-      const int c = 512 * t + 4 * threadIdx.x;
+      const int c = 512 * t + 4 * tid;
       if (c >= d) continue;
-      if (rr) *reinterpret_cast<float4*>(rr + c) = make_float4(v[4 * t], v[4 * t + 1], v[4 * t + 2], v[4 * t + 3]);
       const float y0 = (v[4 * t] - mean) * rstd, y1 = (v[4 * t + 1] - mean) * rstd;
       const float y2 = (v[4 * t + 2] - mean) * rstd, y3 = (v[4 * t + 3] - mean) * rstd;
       uint2 o;
@@ -1287,16 +1309,17 @@ cudaError_t launch_bf16_to_f16(const void* src, void* dst, long long n, int num_
                     static_cast<const uint4*>(src), static_cast<uint4*>(dst), n8);
 }
 
-cudaError_t launch_layernorm(const void* in_txt, const void* in_img, int in_f32, float* resid,
-                             void* ln, int ln_mode, float* ln_scale, const int32_t* cu_img, int B, int n_txt,
-                             int cap, int d, int num_sms, cudaStream_t st) {
-  const dim3 grid(grid_for(static_cast<long long>(n_txt) + cap, 1, num_sms, 16));
-  void* lo = ln;
+cudaError_t launch_layernorm(const void* in_txt, const void* in_img, int in_f32, void* ln, int ln_mode,
+                             float* ln_scale, const int32_t* cu_img, int B, int n_txt, int cap, int d, int num_sms,
+                             cudaStream_t st) {
+  const dim3 grid(grid_for(static_cast<long long>(n_txt) + cap, LN_GROUPS, num_sms, 2));
   switch ((d + 511) / 512) {
-#define HILO_LN_CASE(NC)                                                                      \
-  case NC:                                                                                    \
-    return launch_pdl(layernorm_kernel<NC>, grid, dim3(LN_THREADS), 0, st, in_txt, in_img, in_f32, \
-                      resid, lo, ln_mode, ln_scale, cu_img, B, n_txt, cap, d);
+#define HILO_LN_CASE(NC)                                                                                     \
+  case NC:                                                                                                   \
+    return in_f32 ? launch_pdl(layernorm_kernel<NC, true>, grid, dim3(LN_THREADS), 0, st, in_txt, in_img, ln, \
+                               ln_mode, ln_scale, cu_img, B, n_txt, cap, d)                                  \
+                  : launch_pdl(layernorm_kernel<NC, false>, grid, dim3(LN_THREADS), 0, st, in_txt, in_img, ln, \
+                               ln_mode, ln_scale, cu_img, B, n_txt, cap, d);
     HILO_LN_CASE(1)
     HILO_LN_CASE(2)
     HILO_LN_CASE(3)

@@ -38,9 +38,9 @@ cudaError_t launch_unpack_delta(const float* out_img, const void* packed, const 
 cudaError_t launch_unpack_update(const float* out_img, const int32_t* tok_row, void* x,
                                  long long ntok, int d, float alpha, long long rows_max, int num_sms,
                                  cudaStream_t st);
-cudaError_t launch_layernorm(const void* in_txt, const void* in_img, int in_f32, float* resid,
-                             void* ln, int ln_mode, float* ln_scale, const int32_t* cu_img, int B, int n_txt,
-                             int cap, int d, int num_sms, cudaStream_t st);
+cudaError_t launch_layernorm(const void* in_txt, const void* in_img, int in_f32, void* ln, int ln_mode,
+                             float* ln_scale, const int32_t* cu_img, int B, int n_txt, int cap, int d, int num_sms,
+                             cudaStream_t st);
 cudaError_t launch_quant_rows(const void* src, int type, int cols, int rows_static, const int32_t* cu_img,
                               int B, int n_txt, int cap, uint8_t* dst, float* scale, int num_sms,
                               cudaStream_t st);
