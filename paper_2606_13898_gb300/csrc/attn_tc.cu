@@ -11,7 +11,7 @@
 //
 // A persistent grid, one CTA per SM. The query tiles of all (image, head)
 // groups, in image, head, tile order, are cut into one contiguous range per
-// CTA (ceil(tiles / CTAs) each), so every CTA has the same work, whatever the
+// CTA of about equal cost, so every CTA has the same work, whatever the
 // count of tiles, which only the device knows. A CTA walks its range as jobs:
 // two tiles of one group form a pair (one query tile per softmax warpgroup,
 // sharing every K/V tile); a lone tile at the edge of the range or of its
@@ -35,7 +35,8 @@
 //                lane issues. (With one lane alone, each MMA's descriptor
 //                arithmetic sat on that lane's dependent chain and the issue
 //                fell behind the tensor pipe.)
-//   warp 11      idle (the third warpgroup gives its registers away)
+//   warp 11      the softmax warps' job list (the third warpgroup gives its
+//                registers away)
 // Tensor memory holds S_0 | S_1 | O_0 | O_1 (128 columns each). A softmax
 // warpgroup reads S_i once into registers and writes the probabilities P_i
 // back over the first 64 columns of S_i as packed bf16; the PV product takes
@@ -73,10 +74,11 @@ namespace {
 
 constexpr int BQ = 128;
 constexpr int BKV = 128;
-// Three warpgroups: two softmax warpgroups and one for TMA, MMA and two idle
-// warps. The control warpgroup gives registers to the softmax warpgroups
+// Three warpgroups: two softmax warpgroups and one for TMA, MMA and the job
+// list. The control warpgroup gives registers to the softmax warpgroups
 // (setmaxnreg); launch_hd checks that the shares fit the launch allocation.
 constexpr int ATTN_THREADS = 384;
+constexpr int JOB_BAR_THREADS = 256 + 32;  // softmax, and the warp that prepares the next job
 constexpr int PRODUCER_WARP = 8;    // Q and K copies
 constexpr int V_PRODUCER_WARP = 10; // V copies
 constexpr int MMA_WARP = 9;
@@ -85,6 +87,24 @@ constexpr uint32_t CONTROL_REGS = 72;
 constexpr uint32_t ATTN_TMEM_COLS = 512;  // S0 | S1 | O0 | O1
 constexpr int BOX_BYTES = 128 * 128;       // 128 rows x 64 16-bit elements
 constexpr float RESCALE_LOG2 = 8.0f;
+
+// A CTA's unit of work: two query tiles of one (image, head) over all key
+// tiles (pair), or one query tile whose key tiles are split between the two
+// softmax warpgroups -- even tiles to the first, odd tiles to the second --
+// and merged at the end (split).
+struct Job {
+  bool pair;
+  int b, h, j0, nkv, L;
+};
+
+// The row maxima and sums that a split job's second warpgroup hands over, and the
+// current and the next job (more: there is one), which the softmax warps read from
+// here: they have no registers to keep a job in.
+struct Shared {
+  float m1[BQ], l1[BQ];
+  Job job[2];
+  int more[2];
+};
 
 template <int HD, bool PROP>
 struct Cfg {
@@ -96,10 +116,10 @@ struct Cfg {
   static constexpr int OFF_V = 4 * TILE_BYTES;
   static constexpr int DATA_BYTES = 6 * TILE_BYTES;
   // barriers (256 B); with PROP, 8 softmax warps x 2 slots x 128 weights;
-  // the row maxima and sums a split job's second warpgroup hands over
+  // what the softmax warps read and hand over (Shared)
   static constexpr int OFF_W = DATA_BYTES + 256;
-  static constexpr int OFF_ML = OFF_W + (PROP ? 8 * 2 * BKV * 4 : 0);
-  static constexpr int SMEM_BYTES = OFF_ML + 2 * BQ * 4 + 1024;  // + alignment of the base
+  static constexpr int OFF_X = OFF_W + (PROP ? 8 * 2 * BKV * 4 : 0);
+  static constexpr int SMEM_BYTES = OFF_X + static_cast<int>(sizeof(Shared)) + 1024;  // + alignment of the base
 };
 
 struct AttnParams {
@@ -220,21 +240,35 @@ __device__ __forceinline__ void seq_tile(const AttnParams& p, const Offsets& cu,
   }
 }
 
-// Query tiles of all (image, head) groups.
-__device__ long long total_qtiles(const AttnParams& p, const Offsets& cu) {
-  long long q = 0;
-  for (int b = 0; b < p.B; ++b) q += p.qt_txt + (cu.len(b) + BQ - 1) / BQ;
-  return q * p.heads;
+// The flat query tiles (ordered by image, head, tile) are cut into one contiguous
+// range per CTA: first tile of CTA x of G, x in [0, G]. Where all images have the
+// same number of tiles, or there are no more tiles than CTAs, the ranges are
+// ceil(tiles / G) tiles long. Else they are of equal cost: a tile costs as many steps
+// as its image has key tiles, plus JOB_STEPS for its prologue and epilogue. (Cut by
+// count, the CTAs of the longest of four images of 18 to 25 tiles had 24% more steps
+// than the mean, and attention took 344 us instead of 303.)
+constexpr int JOB_STEPS = 2;
+__device__ long long range_start(const AttnParams& p, const Offsets& cu, long long x, long long G) {
+  auto image_tiles = [&](int b) -> long long { return p.qt_txt + (cu.len(b) + BQ - 1) / BQ; };
+  long long cost = 0, tiles = 0;
+  bool same = true;
+  const long long first = image_tiles(0);
+  for (int b = 0; b < p.B; ++b) {
+    const long long nq = image_tiles(b);
+    same = same && nq == first;
+    tiles += nq * p.heads;
+    cost += nq * p.heads * (nq + JOB_STEPS);
+  }
+  if (same || tiles <= G) return min(tiles, x * ((tiles + G - 1) / G));
+  long long want = (x * cost + G - 1) / G, g = 0;
+  for (int b = 0; b < p.B; ++b) {
+    const long long nq = image_tiles(b), c = nq + JOB_STEPS, all = nq * p.heads * c;
+    if (want < all) return g + (want + c - 1) / c;
+    want -= all;
+    g += nq * p.heads;
+  }
+  return g;
 }
-
-// A CTA's unit of work: two query tiles of one (image, head) over all key
-// tiles (pair), or one query tile whose key tiles are split between the two
-// softmax warpgroups -- even tiles to the first, odd tiles to the second --
-// and merged at the end (split).
-struct Job {
-  bool pair;
-  int b, h, j0, nkv, L;
-};
 
 // The next job of the flat query-tile range [g, end) (tiles ordered by image,
 // head, tile): two tiles of one group form a pair, a lone tile at the edge of
@@ -282,12 +316,9 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
     __syncthreads();
   }
   const Offsets cu{in_smem ? cu_s : nullptr, p};
-  // ---- this CTA's share: a contiguous range of the query tiles of all
-  // (image, head) groups, ceil(total / grid) tiles per CTA
-  const long long qtiles = total_qtiles(p, cu);
-  const long long per = (qtiles + gridDim.x - 1) / gridDim.x;
-  const long long g_begin = static_cast<long long>(blockIdx.x) * per;
-  const long long g_end = min(qtiles, g_begin + per);
+  // ---- this CTA's share of the query tiles of all (image, head) groups
+  const long long g_begin = range_start(p, cu, blockIdx.x, gridDim.x);
+  const long long g_end = range_start(p, cu, blockIdx.x + 1LL, gridDim.x);
   long long g = g_begin;
   Job jb;
   bool more = next_job(p, cu, g, g_end, jb);
@@ -297,8 +328,8 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
   }
 
   extern __shared__ unsigned char smem_raw[];
-  unsigned char* smem = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  // (an offset from smem_raw, so that accesses stay 32-bit shared-memory ones)
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::DATA_BYTES);
   uint64_t* q_full = bars + 0;
   uint64_t* k_full = bars + 1;    // [2]
@@ -313,7 +344,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
   uint64_t* epi_done = bars + 17; // a job's output rows are out: K stages free
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 18);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* ml_slot = reinterpret_cast<float*>(smem + C::OFF_ML);  // split merge: m | l of warpgroup 1
+  Shared& shr = *reinterpret_cast<Shared*>(smem + C::OFF_X);
   int* err = &g_attn_err;
   auto sQ = [&](int i) { return smem + C::OFF_Q + i * C::TILE_BYTES; };
   auto sK = [&](int st) { return smem + C::OFF_K + st * C::TILE_BYTES; };
@@ -336,6 +367,8 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
     mbar_init(epi_done, 1);
     *abort_flag = 0;
     fence_mbar_init();
+    shr.job[0] = jb;
+    shr.more[0] = 1;
   }
   if (warp == MMA_WARP) {
     tmem_alloc(tmem_slot, ATTN_TMEM_COLS);
@@ -352,7 +385,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
   auto kv_stage = [](uint32_t kt0, int t) { return static_cast<int>((kt0 + t) & 1u); };
   auto kv_phase = [](uint32_t kt0, int t) { return ((kt0 + static_cast<uint32_t>(t)) >> 1) & 1u; };
   if (warp >= 8) {
-    // control warpgroup: two TMA producers, the MMA issuer, one idle warp
+    // control warpgroup: two TMA producers, the MMA issuer, the job list
     setmaxnreg_dec<CONTROL_REGS>();
     if (warp == PRODUCER_WARP || warp == V_PRODUCER_WARP) {
     if (lane == 0) {
@@ -575,6 +608,17 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
       }
     }
     __syncwarp();
+    } else {
+      // ---------------- warp 11, the softmax's job list: the next job is ready
+      // when the present one's last barrier is met
+      for (uint32_t jn = 1; more; ++jn) {
+        more = next_job(p, cu, g, g_end, jb);
+        if (lane == 0) {
+          shr.job[jn & 1u] = jb;
+          shr.more[jn & 1u] = more;
+        }
+        if (bar_red_or(2, JOB_BAR_THREADS, false)) break;
+      }
     }
   } else {
     setmaxnreg_inc<SOFTMAX_REGS>();
@@ -585,44 +629,49 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
     const uint32_t tS = tmem + 128u * i + lane_off;
     const uint32_t tO = tmem + 256u + 128u * i + lane_off;
     const uint32_t tO1 = tmem + 384u + lane_off;  // warpgroup 1's accumulator (split merge)
-    // PROP: key weights of tile tt into the warp's slot `slot` (text tiles
-    // weigh 1; columns past the ragged end 0), one commit group per call
+    // PROP: key weights of tile tt (v valid keys; nsrc: the image's weights) into
+    // the warp's slot `slot` (text tiles weigh 1; columns past the ragged end 0),
+    // one commit group per call
     float* wslots = reinterpret_cast<float*>(smem + C::OFF_W) + warp * 2 * BKV;
-    auto fetch_weights = [&](const Job& jb, int tt, int slot) {
-      if (tt < jb.nkv) {
-        float* wb = wslots + slot * BKV;
-        if (tt < p.qt_txt) {
+    auto fetch_weights = [&](const float* nsrc, int tt, int v, int slot) {
+      float* wb = wslots + slot * BKV;
+      if (tt < p.qt_txt) {
 #pragma unroll
-          for (int u = 0; u < 4; ++u) wb[lane + 32 * u] = 1.0f;
-        } else {
-          int r0, v;
-          seq_tile(p, cu, jb.b, jb.L, tt, r0, v);
-          const float* src = p.n_img + (cu(jb.b) + (tt - p.qt_txt) * BKV);
+        for (int u = 0; u < 4; ++u) wb[lane + 32 * u] = 1.0f;
+      } else {
+        const float* src = nsrc + (tt - p.qt_txt) * BKV;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int col = lane + 32 * u;
-            cp_async4(smem_u32(wb + col), col < v ? src + col : p.n_img, col < v ? 4u : 0u);
-          }
+        for (int u = 0; u < 4; ++u) {
+          const int col = lane + 32 * u;
+          cp_async4(smem_u32(wb + col), col < v ? src + col : p.n_img, col < v ? 4u : 0u);
         }
       }
       cp_async_commit();
     };
     bool ok = true;
-    // sc*: S phases so far (one per step); oc*: o_done phases so far (one
-    // per job in which the warpgroup has steps)
-    uint32_t kt = 0, sc0 = 0, sc1 = 0, oc0 = 0, oc1 = 0;
-    for (uint32_t jn = 0; ok && more; ++jn, more = next_job(p, cu, g, g_end, jb)) {
-      const int n0 = job_steps(jb, 0), n1 = job_steps(jb, 1);
-      const int n = i ? n1 : n0;
-      const uint32_t sc = i ? sc1 : sc0;
-      const uint32_t oc = i ? oc1 : oc0;
+    // sc: S phases of this warpgroup so far (one per step); oc*: o_done phases so
+    // far (one per job in which a warpgroup has steps); kt: the running key tile
+    uint32_t kt = 0, sc = 0, oc0 = 0, oc1 = 0;
+    for (uint32_t jn = 0;; ++jn) {
+      const Job& jb = shr.job[jn & 1u];
+      const bool pair = jb.pair;
+      const int nkv = jb.nkv;
+      const int n1 = pair ? nkv : nkv / 2;  // steps of the second warpgroup
+      const int n = i ? n1 : nkv - (pair ? 0 : n1);
+      const int tail = jb.L - (nkv - p.qt_txt - 1) * BKV;  // rows of the last image tile
+      // rows of key tile t: only the last of the text and of the image are ragged
+      auto valid_rows = [&](int t) {
+        if (t == p.qt_txt - 1) return p.T - t * BKV;
+        return t == nkv - 1 ? tail : BKV;
+      };
+      auto step_tile = [&](int s) { return pair ? s : 2 * s + i; };
       float m = -INFINITY, l = 0.f;
       // ragged key tile: rows past `valid` hold other tokens (or stale data);
       // the warpgroup that owns V tile t (the first one in a pair) zeroes
       // them so that the zero-probability columns add exactly 0. Returns
       // false when the wait for V gave up.
       auto zero_v_tail = [&](int t, int valid) -> bool {
-        if ((jb.pair ? i == 0 : true) && valid < BKV) {
+        if ((pair ? i == 0 : true) && valid < BKV) {
           if (!mbar_wait_warp(&v_full[kv_stage(kt, t)], kv_phase(kt, t), abort_flag, err,
                               DEV_TIMEOUT_ATTN + 256 * 11))
             return false;
@@ -657,16 +706,15 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
           l *= alpha;
         }
       };
-      if (PROP && n > 0) fetch_weights(jb, job_tile(jb, i, 0), 0);
+      const float* nsrc = PROP ? p.n_img + cu(jb.b) : nullptr;
+      if (PROP && n > 0) fetch_weights(nsrc, step_tile(0), valid_rows(step_tile(0)), 0);
       for (int s = 0; s < n && ok; ++s) {
-        const int t = job_tile(jb, i, s);
-        int row0, valid;
-        seq_tile(p, cu, jb.b, jb.L, t, row0, valid);
+        const int t = step_tile(s), valid = valid_rows(t);
         if (PROP) {
           // every lane is done with slot (s + 1) & 1 (read for step s - 1)
           // before the next step's weights are fetched into it
           __syncwarp();
-          if (s + 1 < n) fetch_weights(jb, job_tile(jb, i, s + 1), (s + 1) & 1);
+          if (s + 1 < n) fetch_weights(nsrc, step_tile(s + 1), valid_rows(step_tile(s + 1)), (s + 1) & 1);
           else cp_async_commit();
         }
         if (!mbar_wait_warp(&s_full[i], (sc + s) & 1u, abort_flag, err, DEV_TIMEOUT_ATTN + 256 * 10)) {
@@ -791,7 +839,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
         // V rows zeroed above (ragged tile, owning warpgroup) are read by the
         // tensor core: make them visible to the async proxy before P_i is
         // handed over; other steps wrote no shared memory
-        if ((jb.pair ? i == 0 : true) && valid < BKV) fence_proxy_async_smem();
+        if ((pair ? i == 0 : true) && valid < BKV) fence_proxy_async_smem();
         tc_fence_before();
         mbar_arrive(&p_full[i]);
       }
@@ -800,25 +848,25 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
       // split job: warpgroup 1 hands its row maximum and sum to warpgroup 0,
       // which merges the two accumulators (each relative to its own maximum)
       // and writes query tile j0.
-      const bool writer = jb.pair || i == 0;
-      if (!jb.pair) {
+      const bool writer = pair || i == 0;
+      if (!pair) {
         if (i == 1) {
-          ml_slot[row] = m;
-          ml_slot[BQ + row] = l;
+          shr.m1[row] = m;
+          shr.l1[row] = l;
         }
         named_bar_sync(1, 256);
       }
       float a0 = 1.f, a1 = 0.f, inv = 1.f;
       if (ok && writer) {
-        bool done = mbar_wait_warp(&o_done[i], oc & 1u, abort_flag, err, DEV_TIMEOUT_ATTN + 256 * 14);
-        if (!jb.pair && n1 > 0)
+        bool done = mbar_wait_warp(&o_done[i], (i ? oc1 : oc0) & 1u, abort_flag, err, DEV_TIMEOUT_ATTN + 256 * 14);
+        if (!pair && n1 > 0)
           done = done && mbar_wait_warp(&o_done[1], oc1 & 1u, abort_flag, err, DEV_TIMEOUT_ATTN + 256 * 15);
         ok = done;
         if (ok) {
           tc_fence_after();
           float lt = l;
-          if (!jb.pair && n1 > 0) {
-            const float m1 = ml_slot[row], l1 = ml_slot[BQ + row];
+          if (!pair && n1 > 0) {
+            const float m1 = shr.m1[row], l1 = shr.l1[row];
             const float mm = fmaxf(m, m1);
             a0 = ex2(m - mm);
             a1 = ex2(m1 - mm);
@@ -826,7 +874,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
           }
           inv = 1.0f / lt;
           int qr0, qv;
-          seq_tile(p, cu, jb.b, jb.L, jb.j0 + (jb.pair ? i : 0), qr0, qv);
+          seq_tile(p, cu, jb.b, jb.L, jb.j0 + (pair ? i : 0), qr0, qv);
           // normalised O rows to bf16, staged through shared memory so that
           // the global stores leave as whole 128-byte lines (one row per
           // lane would write 16 bytes into 32 different rows per
@@ -839,7 +887,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
           constexpr int UNITS = HD / 8;    // 16-byte units per row
           constexpr int RPI = 32 / UNITS;  // rows per store instruction
           uint4* stage = reinterpret_cast<uint4*>(smem + C::OFF_K) + warp * 32 * UNITS;
-          const bool merge = !jb.pair && n1 > 0;
+          const bool merge = !pair && n1 > 0;
           auto stage_chunk = [&](int c, const float* o) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -892,14 +940,13 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
       // next PV may overwrite it
       fence_proxy_async_smem();
       tc_fence_before();
-      ok = bar_red_or(2, 256, !ok) ? false : ok;
-      if (!ok) break;
+      if (bar_red_or(2, JOB_BAR_THREADS, !ok)) break;
       if (threadIdx.x == 0) mbar_arrive(epi_done);
-      sc0 += static_cast<uint32_t>(n0);
-      sc1 += static_cast<uint32_t>(n1);
-      oc0 += n0 > 0 ? 1u : 0u;
+      sc += static_cast<uint32_t>(n);
+      oc0 += nkv > (pair ? 0 : n1) ? 1u : 0u;
       oc1 += n1 > 0 ? 1u : 0u;
-      kt += static_cast<uint32_t>(jb.nkv);
+      kt += static_cast<uint32_t>(nkv);
+      if (!shr.more[(jn + 1) & 1u]) break;
     }
     if (PROP) cp_async_wait<0>();
   }
