@@ -1109,22 +1109,17 @@ __global__ void __launch_bounds__(LN_THREADS, 2) layernorm_kernel(const void* __
 }
 
 // ==================================================== e4m3 rows =====
-// Per-row e4m3 quantisation: one 256-thread CTA per row. The row's largest
+// Per-row e4m3 quantisation by persistent 256-thread CTAs. The row's largest
 // magnitude, then each element times 448 / amax (fp32) rounded to e4m3; the
-// dequantisation scale amax / 448 per row. src_type 0 bf16, 1 fp16, 2 fp32;
-// cols a multiple of 8. Rows: rows_static, or n_txt + min(cu_img[B], cap)
-// when cu_img is given (the row space of the block).
+// dequantisation scale amax / 448 per row. TYPE 0 bf16, 1 fp16, 2 fp32; cols a
+// multiple of 8. Rows: rows_static, or n_txt + min(cu_img[B], cap) when cu_img is
+// given (the row space of the block). Bound by memory: 16-bit rows of up to 2048 NP
+// elements (NP > 0) are read once and stay in registers while the next row is on its
+// way; longer or fp32 rows (NP = 0) are read a second time, from L1 / L2.
 
 constexpr int QR_THREADS = 256;
 
-__device__ __forceinline__ void load8(const void* src, int type, long long i8, float* f) {
-  if (type == 2) {
-    const float4* p = static_cast<const float4*>(src) + 2 * i8;
-    const float4 a = __ldg(p), b = __ldg(p + 1);
-    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
-    return;
-  }
-  const uint4 u = __ldg(static_cast<const uint4*>(src) + i8);
+__device__ __forceinline__ void widen8(const uint4& u, int type, float* f) {
   if (type == 0) {
     bf16x8_to_f32(u, f);
     return;
@@ -1139,43 +1134,93 @@ __device__ __forceinline__ void load8(const void* src, int type, long long i8, f
   }
 }
 
-__global__ void __launch_bounds__(QR_THREADS) quant_rows_kernel(const void* __restrict__ src, int type,
-                                                                int cols, int rows_static,
-                                                                const int32_t* __restrict__ cu_img, int B,
-                                                                int n_txt, int cap, uint8_t* __restrict__ dst,
-                                                                float* __restrict__ scale) {
+__device__ __forceinline__ void load8(const void* src, int type, long long i8, float* f) {
+  if (type == 2) {
+    const float4* p = static_cast<const float4*>(src) + 2 * i8;
+    const float4 a = __ldg(p), b = __ldg(p + 1);
+    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+    return;
+  }
+  widen8(__ldg(static_cast<const uint4*>(src) + i8), type, f);
+}
+
+__device__ __forceinline__ uint2 quant8(const float* f, float inv) {
+  uint2 o;
+  o.x = pack_e4m3x4(__fmul_rn(f[0], inv), __fmul_rn(f[1], inv), __fmul_rn(f[2], inv), __fmul_rn(f[3], inv));
+  o.y = pack_e4m3x4(__fmul_rn(f[4], inv), __fmul_rn(f[5], inv), __fmul_rn(f[6], inv), __fmul_rn(f[7], inv));
+  return o;
+}
+
+// The row's largest magnitude over the CTA; `red` is rewritten only after the
+// CTA has met again.
+__device__ __forceinline__ float quant_amax(float am, float* red) {
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, off));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = am;
+  __syncthreads();
+  am = red[0];
+#pragma unroll
+  for (int w = 1; w < QR_THREADS / 32; ++w) am = fmaxf(am, red[w]);
+  return am;
+}
+
+template <int TYPE, int NP>
+__global__ void __launch_bounds__(QR_THREADS, NP == 6 ? 3 : 6)
+    quant_rows_kernel(const void* __restrict__ src, int cols, int rows_static, const int32_t* __restrict__ cu_img,
+                      int B, int n_txt, int cap, uint8_t* __restrict__ dst, float* __restrict__ scale) {
+  constexpr bool REG = NP > 0;
   pdl_wait();
   pdl_trigger();
-  __shared__ float red[QR_THREADS / 32];
+  __shared__ float red[2][QR_THREADS / 32];  // rows alternate
   const int rows = cu_img ? n_txt + min(cu_img[B], cap) : rows_static;
   const int g8 = cols >> 3;
-  for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-    const long long base8 = static_cast<long long>(r) * g8;
-    float am = 0.f;
-    for (int g = threadIdx.x; g < g8; g += QR_THREADS) {
-      float f[8];
-      load8(src, type, base8 + g, f);
+  uint4 raw[REG ? NP : 1];
+  auto load = [&](int r) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) am = fmaxf(am, fabsf(f[i]));
+    for (int k = 0; k < NP; ++k) {
+      const int g = threadIdx.x + k * QR_THREADS;
+      raw[k] = make_uint4(0u, 0u, 0u, 0u);
+      if (g < g8) raw[k] = __ldg(static_cast<const uint4*>(src) + static_cast<long long>(r) * g8 + g);
     }
+  };
+  if (REG && blockIdx.x < rows) load(blockIdx.x);
+  int h = 0;
+  for (int r = blockIdx.x; r < rows; r += gridDim.x, h ^= 1) {
+    const long long base8 = static_cast<long long>(r) * g8;
+    float am = 0.f, inv, sc;
+    if constexpr (REG) {
+      uint4 cur[NP];
 #pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, off));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = am;
-    __syncthreads();
-    am = red[0];
+      for (int k = 0; k < NP; ++k) {
+        cur[k] = raw[k];
+        float f[8];
+        widen8(cur[k], TYPE, f);
 #pragma unroll
-    for (int w = 1; w < QR_THREADS / 32; ++w) am = fmaxf(am, red[w]);
-    __syncthreads();
-    float inv, sc;
-    e4m3_row_scale(am, inv, sc);
-    // second pass: the row is in L1 / L2 from the first
-    for (int g = threadIdx.x; g < g8; g += QR_THREADS) {
-      float f[8];
-      load8(src, type, base8 + g, f);
-      uint2 o;
-      o.x = pack_e4m3x4(__fmul_rn(f[0], inv), __fmul_rn(f[1], inv), __fmul_rn(f[2], inv), __fmul_rn(f[3], inv));
-      o.y = pack_e4m3x4(__fmul_rn(f[4], inv), __fmul_rn(f[5], inv), __fmul_rn(f[6], inv), __fmul_rn(f[7], inv));
-      reinterpret_cast<uint2*>(dst)[base8 + g] = o;
+        for (int i = 0; i < 8; ++i) am = fmaxf(am, fabsf(f[i]));
+      }
+      if (r + static_cast<long long>(gridDim.x) < rows) load(r + gridDim.x);
+      e4m3_row_scale(quant_amax(am, red[h]), inv, sc);
+#pragma unroll
+      for (int k = 0; k < NP; ++k) {
+        const int g = threadIdx.x + k * QR_THREADS;
+        float f[8];
+        widen8(cur[k], TYPE, f);
+        if (g < g8) reinterpret_cast<uint2*>(dst)[base8 + g] = quant8(f, inv);
+      }
+    } else {
+      for (int g = threadIdx.x; g < g8; g += QR_THREADS) {
+        float f[8];
+        load8(src, TYPE, base8 + g, f);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) am = fmaxf(am, fabsf(f[i]));
+      }
+      e4m3_row_scale(quant_amax(am, red[h]), inv, sc);
+      // second pass: the row is in L1 / L2 from the first
+      for (int g = threadIdx.x; g < g8; g += QR_THREADS) {
+        float f[8];
+        load8(src, TYPE, base8 + g, f);
+        reinterpret_cast<uint2*>(dst)[base8 + g] = quant8(f, inv);
+      }
     }
     if (threadIdx.x == 0) scale[r] = sc;
   }
@@ -1297,8 +1342,13 @@ cudaError_t launch_quant_rows(const void* src, int type, int cols, int rows_stat
                               cudaStream_t st) {
   const long long rmax = cu_img ? static_cast<long long>(n_txt) + cap : rows_static;
   if (rmax <= 0) return cudaSuccess;
-  return launch_pdl(quant_rows_kernel, dim3(grid_for(rmax, 1, num_sms, 8)), dim3(QR_THREADS), 0, st, src, type,
-                    cols, rows_static, cu_img, B, n_txt, cap, dst, scale);
+  const int np = type == 2 || cols > 6 * 2048 ? 0 : (cols > 2 * 2048 ? 6 : 2);
+  auto* kern = type == 2 ? quant_rows_kernel<2, 0>
+               : type == 0
+                   ? (np == 2 ? quant_rows_kernel<0, 2> : np == 6 ? quant_rows_kernel<0, 6> : quant_rows_kernel<0, 0>)
+                   : (np == 2 ? quant_rows_kernel<1, 2> : np == 6 ? quant_rows_kernel<1, 6> : quant_rows_kernel<1, 0>);
+  return launch_pdl(kern, dim3(grid_for(rmax, 1, num_sms, np == 6 ? 3 : np == 2 ? 6 : 8)), dim3(QR_THREADS), 0, st,
+                    src, cols, rows_static, cu_img, B, n_txt, cap, dst, scale);
 }
 
 cudaError_t launch_bf16_to_f16(const void* src, void* dst, long long n, int num_sms,
