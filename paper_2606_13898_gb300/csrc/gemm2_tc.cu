@@ -60,7 +60,8 @@ constexpr int SPLIT_MIN_KB = 16;            // shortest piece of a tile cut alon
 constexpr int SPLIT_MAX = 8;                // most pieces per tile
 // the plan's costs in SM cycles beside those of the k-blocks
 constexpr float TILE_CYC = 400.f;           // going from one tile to the next
-constexpr float EPI_CYC = 800.f;            // the last epilogue, per 32 rows
+constexpr float EPI_CYC = 700.f;            // the last epilogue, per 32 rows
+constexpr float EPI_RESID_CYC = 1200.f;     // the same with a residual to load
 constexpr float PIECE_CYC = 300.f;          // a K piece's reductions, per 32 rows
 
 struct Maps {
@@ -113,11 +114,13 @@ struct Plan {
 
   // Chosen by cost: lane l tries image tiles of at most u1 = 8 - l % 8 units,
   // text tiles of at most u1 + l / 8, and cuts of the tiles left over after the
-  // last full round into 2 to 8 pieces, by rows or, with `split`, along K; the
+  // last full round into 2 to 8 pieces, by rows or (fp32 += only) along K; the
   // cheapest wins, the higher tile and the fewer pieces among equals. The cost is
   // that of pair 0, which has the most tiles: its rounds of whole tiles, its
   // pieces, and the epilogue that nothing hides. Called by whole warps.
-  __device__ void init(const Params& p, int dev0, int dev1, int ncl, int kb, bool split) {
+  __device__ void init(const Params& p, int dev0, int dev1, int ncl, int kb) {
+    const bool split = p.epilogue == EPI_BIAS_RESID_F32;
+    const float EPI = p.epilogue == EPI_BIAS_RESIDIN_F32 ? EPI_RESID_CYC : EPI_CYC;
     // a device row count is bounded by the group's capacity (rows_static)
     rows0 = max(0, p.rows_dev[0] ? min(dev0, p.rows_static[0]) : p.rows_static[0]);
     rows1 = max(0, p.rows_dev[1] ? min(dev1, p.rows_static[1]) : p.rows_static[1]);
@@ -142,7 +145,7 @@ struct Plan {
       const int rounds = rounds_of(tiles), g0 = min(rounds, g_max);
       return g0 * c0 + (rounds - g0) * c1;
     };
-    float best = rounds_cost(T) + EPI_CYC * xm;
+    float best = rounds_cost(T) + EPI * xm;
     int best_s = 1, best_k = 0;
     if (rem > 0) {
       const float c_full = rounds_cost(T - rem);
@@ -150,10 +153,10 @@ struct Plan {
       for (int s = 2; s <= SPLIT_MAX; ++s) {
         const float n = static_cast<float>(rounds_of(rem * s));
         const float xs = ceilf(xm * (1.0f / s) - 1e-3f);
-        const float cr = c_full + n * (kbf * kblock(xs) + TILE_CYC) + EPI_CYC * xs;
+        const float cr = c_full + n * (kbf * kblock(xs) + TILE_CYC) + EPI * xs;
         if (s <= least && cr < best) best = cr, best_s = s, best_k = 0;
         const float ck =
-            c_full + n * (((kb + s - 1) / s) * kblock(xm) + TILE_CYC + PIECE_CYC * xm) + EPI_CYC * xm;
+            c_full + n * (((kb + s - 1) / s) * kblock(xm) + TILE_CYC + PIECE_CYC * xm) + EPI * xm;
         if (split && kb >= s * SPLIT_MIN_KB && ck < best) best = ck, best_s = s, best_k = 1;
       }
     }
@@ -244,8 +247,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   // elements per k-block: one 128-byte swizzled row of X / W
   constexpr int BKE = FP8 ? 128 : BK;
   extern __shared__ unsigned char smem_raw[];
-  unsigned char* smem = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  // (an offset from smem_raw, so that accesses stay 32-bit shared-memory ones)
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
   uint64_t* empty = full + STAGES;
   uint64_t* tfull = empty + STAGES;
@@ -285,7 +288,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   }
   const int kblocks = p.K / BKE;
   Plan pl;
-  pl.init(p, dev0, dev1, ncl, kblocks, p.epilogue == EPI_BIAS_RESID_F32);
+  pl.init(p, dev0, dev1, ncl, kblocks);
   WorkIter it(pl, cid, ncl, kblocks);
   Work w;
   tc_fence_before();
@@ -461,6 +464,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
         const int r = tl.r0 + half * UNIT;
         epi_load_resid(resid, resid_f32, r, half < tl.units ? tl.rows - r : 0, ch.feat, N, rn);
       }
+      // FP8: lane r's row scale of each of this warp's chunks
+      float rscale[MAXU / 2];
+      if (FP8) {
+#pragma unroll
+        for (int k = 0; k < MAXU / 2; ++k) {
+          const int r = tl.r0 + (half + 2 * k) * UNIT + lane;
+          rscale[k] = half + 2 * k < tl.units && r < tl.rows ? __ldg(p.a_scale + tl.row_base + r) : 0.f;
+        }
+      }
       if (!mbar_wait_warp(&tfull[acc], acc_phase, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 5)) break;
       tc_fence_after();
       const uint32_t taddr =
@@ -479,8 +491,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
         }
         ch.nvalid = min(UNIT, tl.rows - r);
         ch.row = tl.row_base + r;
-        float rscale = 0.f;
-        if (FP8 && lane < ch.nvalid) rscale = __ldg(p.a_scale + ch.row + lane);
         tmem_ld_wait_regs(v);
         if (c + 2 >= tl.units) {
           tc_fence_before();
@@ -489,8 +499,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
         }
         if (!on) continue;
         if (FP8) {
+          float rs = rscale[0];  // of this chunk (selected: no runtime-indexed array)
 #pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] *= __shfl_sync(0xffffffffu, rscale, j) * wscale;
+          for (int k = 1; k < MAXU / 2; ++k) rs = c == half + 2 * k ? rscale[k] : rs;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] *= __shfl_sync(0xffffffffu, rs, j) * wscale;
         }
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] += bias;
