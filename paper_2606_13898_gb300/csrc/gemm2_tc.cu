@@ -112,12 +112,14 @@ struct Plan {
   // the MMA rate and a lower one loses what it saves in columns.
   __device__ static float kblock(float x) { return 272.0f + 34.0f * x; }
 
-  // Chosen by cost: lane l tries image tiles of at most u1 = 8 - l % 8 units,
-  // text tiles of at most u1 + l / 8, and cuts of the tiles left over after the
-  // last full round into 2 to 8 pieces, by rows or (fp32 += only) along K; the
-  // cheapest wins, the higher tile and the fewer pieces among equals. The cost is
-  // that of pair 0, which has the most tiles: its rounds of whole tiles, its
-  // pieces, and the epilogue that nothing hides. Called by whole warps.
+  // Chosen by cost: lane l tries image tiles of at most u1 = 8 - l % 8 units (and
+  // text tiles of at most two more), whole or with the tiles left over after the last
+  // full round cut into 2 to 8 pieces, by rows or (fp32 += only) along K, of which
+  // lane l takes the counts 1 + l / 8 and 5 + l / 8; the cheapest wins, the higher
+  // tile and the fewer pieces among equals. The cost is that of pair 0, which has the
+  // most tiles: its rounds of whole tiles, its pieces, and the epilogue that nothing
+  // hides. Called by whole warps. Every cycle here is one before the first product
+  // wherever the previous kernel held the SM to its end.
   __device__ void init(const Params& p, int dev0, int dev1, int ncl, int kb) {
     const bool split = p.epilogue == EPI_BIAS_RESID_F32;
     const float EPI = p.epilogue == EPI_BIAS_RESIDIN_F32 ? EPI_RESID_CYC : EPI_CYC;
@@ -128,37 +130,43 @@ struct Plan {
     U1 = (rows1 + UNIT - 1) / UNIT;
     const int F = (p.N + PF - 1) / PF;
     const int lane = lane_id();
-    const int u1 = MAXU - (lane & 7), u0 = min(MAXU, u1 + (lane >> 3));
+    const int u1 = MAXU - (lane & 7), u0 = min(MAXU, u1 + 2);
     const int a0 = (U0 + u0 - 1) / u0, a1 = (U1 + u1 - 1) / u1;
-    const int T0 = F * a0, T = F * (a0 + a1), rem = T % ncl;
-    const float x0 = a0 ? static_cast<float>(U0) / a0 : 0.f, x1 = a1 ? static_cast<float>(U1) / a1 : 0.f;
+    const int T0 = F * a0, T = F * (a0 + a1);
+    const float x0 = a0 ? __fdividef(U0, a0) : 0.f, x1 = a1 ? __fdividef(U1, a1) : 0.f;
     const float xm = fmaxf(x0, x1);
-    const int least = a0 && a1 ? min(U0 / a0, U1 / a1) : (a0 ? U0 / a0 : (a1 ? U1 / a1 : 0));
+    // no tile has fewer units than its group's floor(U / a), so it can be cut into as
+    // many pieces (the quotient is checked: a piece must not be empty)
+    auto least_of = [](int U, int a, float x) {
+      const int q = static_cast<int>(x + 1e-3f);
+      return a == 0 ? MAXU : (q * a <= U ? q : q - 1);
+    };
+    const int least = min(least_of(U0, a0, x0), least_of(U1, a1, x1));
     const float kbf = static_cast<float>(kb);
     const float c0 = kbf * kblock(x0) + TILE_CYC, c1 = kbf * kblock(x1) + TILE_CYC;
     // ceil(n / ncl) for the small counts here (n + 0.5 keeps the product away
     // from the whole numbers)
-    const float inv = 1.0f / static_cast<float>(ncl);
+    const float inv = __fdividef(1.0f, static_cast<float>(ncl));
     auto rounds_of = [&](int n) { return static_cast<int>((static_cast<float>(n + ncl - 1) + 0.5f) * inv); };
-    const int g_max = rounds_of(T0);
-    auto rounds_cost = [&](int tiles) {
-      const int rounds = rounds_of(tiles), g0 = min(rounds, g_max);
-      return g0 * c0 + (rounds - g0) * c1;
+    const int g_max = rounds_of(T0), rounds = rounds_of(T);
+    auto rounds_cost = [&](int n) {
+      const int g0 = min(n, g_max);
+      return g0 * c0 + (n - g0) * c1;
     };
-    float best = rounds_cost(T) + EPI * xm;
+    const int rem = T > 0 && rounds * ncl != T ? T - (rounds - 1) * ncl : 0;  // of a partial last round
+    float best = rounds_cost(rounds) + EPI * xm;
     int best_s = 1, best_k = 0;
-    if (rem > 0) {
-      const float c_full = rounds_cost(T - rem);
+    const float c_full = rounds_cost(rounds - 1);
 #pragma unroll
-      for (int s = 2; s <= SPLIT_MAX; ++s) {
-        const float n = static_cast<float>(rounds_of(rem * s));
-        const float xs = ceilf(xm * (1.0f / s) - 1e-3f);
-        const float cr = c_full + n * (kbf * kblock(xs) + TILE_CYC) + EPI * xs;
-        if (s <= least && cr < best) best = cr, best_s = s, best_k = 0;
-        const float ck =
-            c_full + n * (((kb + s - 1) / s) * kblock(xm) + TILE_CYC + PIECE_CYC * xm) + EPI * xm;
-        if (split && kb >= s * SPLIT_MIN_KB && ck < best) best = ck, best_s = s, best_k = 1;
-      }
+    for (int j = 0; j < 2; ++j) {
+      const int s = 1 + (lane >> 3) + 4 * j;
+      if (s == 1 || rem == 0) continue;
+      const float n = static_cast<float>(rounds_of(rem * s)), sf = static_cast<float>(s);
+      const float xs = ceilf(__fdividef(xm, sf) - 1e-3f), ks = ceilf(__fdividef(kbf, sf) - 1e-3f);
+      const float cr = c_full + n * (kbf * kblock(xs) + TILE_CYC) + EPI * xs;
+      if (s <= least && cr < best) best = cr, best_s = s, best_k = 0;
+      const float ck = c_full + n * (ks * kblock(xm) + TILE_CYC + PIECE_CYC * xm) + EPI * xm;
+      if (split && kb >= s * SPLIT_MIN_KB && ck < best) best = ck, best_s = s, best_k = 1;
     }
     // costs are positive, so their bit patterns order like the values
     const uint32_t key = __float_as_uint(best);
@@ -169,6 +177,7 @@ struct Plan {
     nsplit = __shfl_sync(0xffffffffu, best_s, win);
     kcut = __shfl_sync(0xffffffffu, best_k, win);
     total = F * (t0 + t1);
+    // exact, whatever the estimates above were rounded to
     whole = nsplit > 1 ? total - total % ncl : total;
   }
 
