@@ -709,7 +709,8 @@ __global__ void __launch_bounds__(256) pack_kernel(const __nv_bfloat16* __restri
   const long long nwarps = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
   for (long long gw = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
        gw < static_cast<long long>(total) * PACK_WARPS_PER_ROW; gw += nwarps) {
-    const int r = static_cast<int>(gw / PACK_WARPS_PER_ROW);
+    // from the last row down: an image's pooled rows, 4x4 last, take the longest
+    const int r = total - 1 - static_cast<int>(gw / PACK_WARPS_PER_ROW);
     const int c0 = lane + 32 * static_cast<int>(gw % PACK_WARPS_PER_ROW);
     constexpr int CSTEP = 32 * PACK_WARPS_PER_ROW;
     int b = 0;
