@@ -1,0 +1,131 @@
+"""The bandwidth kernels and the attention's schedule where their code changes
+path: the split at the sizes where a thread's number of tokens doubles, in each
+mode and on arrays that allow no wide load; e4m3 rows at the ends of the widths
+that stay in registers; LayerNorm rows below, at and above one pass of the
+resident groups; attention over images of different length, with more query
+tiles than SMs, and more images than the offsets kept in shared memory."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import hilo_oracle as O
+from paper_2606_13898_gb300 import inputs as I
+
+from .gpu_helpers import assert_block_close, lib_ready, to_dev_i32
+from .test_gpu_kernels import bits, check_split, scaled_weights
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def H():
+    return lib_ready()
+
+
+def offset_by_one(a):
+    """A device copy of the array one element past an aligned address."""
+    t = torch.from_numpy(np.ascontiguousarray(a).reshape(-1)).cuda()
+    buf = torch.empty(t.numel() + 1, dtype=t.dtype, device="cuda")
+    buf[1:] = t
+    return buf[1:]
+
+
+@pytest.mark.parametrize("mode", ["plain1", "plain2", "regions2", "lf4"])
+@pytest.mark.parametrize("B", [1, 2])
+@pytest.mark.parametrize("Hh,W", [(4, 4), (64, 64), (64, 68), (64, 128), (64, 132), (128, 128), (128, 132)])
+def test_split_at_tokens_per_thread(H, Hh, W, B, mode):
+    rng = np.random.default_rng(Hh * W + B)
+    N = Hh * W
+    s = (rng.integers(0, 300, size=(B, N)) * 0.25).astype(np.float32)
+    mask = (rng.random((B, N)) < 0.05).astype(np.uint8)
+    kk = rng.integers(1, N // 2, size=B).astype(np.int32)
+    km = rng.integers(1, N // 2, size=B).astype(np.int32)
+    levels, lf = (2 if mode[-1] == "2" else 1), (4 if mode == "lf4" else 0)
+    sh = H.Shape(B=B, H=Hh, W=W, d=128, levels=levels, lf=lf)
+    sp = H.SplitBuffers.alloc(sh)
+    sp.labels = offset_by_one(sp.labels.cpu().numpy())
+    (H.hilo_split_regions if mode == "regions2" else H.hilo_split)(
+        sh, offset_by_one(s), offset_by_one(mask), to_dev_i32(kk), to_dev_i32(km), sp)
+    H.hilo_sync_status()
+    ref = (O.split(s, mask, kk, km, Hh, W, levels, lf=lf) if lf else
+           O.split(s, mask, kk, km, Hh, W, levels, granular=mode == "regions2"))
+    check_split(sp, ref, B, N)
+
+
+@pytest.mark.parametrize("dtype,cols", [("bf16", 8), ("bf16", 4096), ("bf16", 4104), ("bf16", 12288),
+                                        ("bf16", 12296), ("f16", 4096), ("f16", 4104), ("f16", 12296),
+                                        ("f32", 4104)])
+@pytest.mark.parametrize("rows", [1, 1000])
+def test_quantize_rows_at_register_widths(H, dtype, cols, rows):
+    rng = np.random.default_rng(cols + rows)
+    x = (rng.standard_normal((rows, cols)) * np.exp(rng.uniform(-8, 8, (rows, 1)))).astype(np.float32)
+    x[rows // 2, -1] = 20000.0  # the row's largest value in its last column
+    if dtype == "bf16":
+        xb = bits(x)
+        src, code, xf = H.bf16_from_bits(xb), H.HILO_BF16, O.bf16_to_f32(xb)
+    elif dtype == "f16":
+        xh = np.clip(x, -60000, 60000).astype(np.float16)
+        src, code, xf = torch.from_numpy(xh).cuda(), H.HILO_F16, xh.astype(np.float32)
+    else:
+        src, code, xf = torch.from_numpy(x).cuda(), H.HILO_F32, x
+    q = torch.full((rows + 1, cols), 0x55, dtype=torch.uint8, device="cuda")
+    sc = torch.empty(rows, dtype=torch.float32, device="cuda")
+    H.hilo_quantize_rows_e4m3(src, code, rows, cols, q, sc)
+    H.hilo_sync_status()
+    cref, sref = O.quantize_rows(xf)
+    got = q.cpu().numpy()
+    assert np.array_equal(got[:rows], cref) and np.all(got[rows] == 0x55)
+    assert np.array_equal(sc.cpu().numpy(), sref)
+
+
+@pytest.mark.parametrize("f32", [0, 1])
+@pytest.mark.parametrize("rows", [1, 911, 1830])
+@pytest.mark.parametrize("d", [128, 640, 4096])
+def test_layernorm_rows(H, d, rows, f32):
+    """The LayerNorm rows of a block (first region of its workspace). Each is
+    the fp64 value rounded to bf16 (2^-9 relative), after fp32 sums over d
+    elements (mean and variance within d 2^-24 of their terms, 3e-4 at most)."""
+    rng = np.random.default_rng(d + rows)
+    u = (rng.standard_normal((rows, d)) * 3 + 1).astype(np.float32)
+    if not f32:
+        u = bits(u)
+    zeros = I.BlockWeights(**{s: I.StreamWeights(
+        w_qkv=np.zeros((3 * d, d), np.uint16), b_qkv=np.zeros(3 * d, np.uint16),
+        w_o=np.zeros((d, d), np.uint16), b_o=np.zeros(d, np.uint16)) for s in ("txt", "img")})
+    sh = H.Shape(B=1, H=64, W=64, d=d, T=0, heads=d // 128, mlp=0)
+    out = torch.empty(rows, d, dtype=torch.float32, device="cuda")
+    wsb = H.hilo_block_workspace_bytes(sh, rows)
+    ws = torch.full((wsb,), 0xFF, dtype=torch.uint8, device="cuda")  # NaN
+    H.hilo_block_forward(sh, H.DeviceWeights.from_host(zeros), to_dev_i32([0, rows]), rows, None,
+                         torch.from_numpy(u).cuda() if f32 else H.bf16_from_bits(u),
+                         H.HILO_F32 if f32 else H.HILO_BF16, out, ws, wsb)
+    H.hilo_sync_status()
+    got = ws[:rows * d * 2].view(torch.bfloat16).view(rows, d).float().cpu().numpy().astype(np.float64)
+    ref = O.layer_norm(u.astype(np.float64) if f32 else O.bf16_to_f32(u).astype(np.float64))
+    assert np.all(np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 3e-4)
+
+
+@pytest.mark.parametrize("d,heads,T,lens", [
+    (1024, 16, 64, [130, 900, 5, 0]),      # 240 query tiles of images 1 to 9 tiles long
+    (1024, 8, 0, [257, 2050]),             # 160 tiles, hd 128, no text
+    (128, 2, 0, [5, 150] * 65),            # 130 images: offsets read from memory
+    (128, 1, 3, [0] * 3 + [129] * 125),    # 128 images: the last that fit in shared memory
+])
+def test_attention_images_of_different_length(H, d, heads, T, lens):
+    rng = np.random.default_rng(d + heads + len(lens))
+    B, rows = len(lens), sum(lens)
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    ut, ui = bits(rng.standard_normal((B * T, d))), bits(rng.standard_normal((rows, d)))
+    w = scaled_weights(rng, d, False, std=1.0 / np.sqrt(d))
+    sh = H.Shape(B=B, H=64, W=64, d=d, T=T, heads=heads, mlp=0)
+    out = torch.empty(B * T + rows, d, dtype=torch.float32, device="cuda")
+    wsb = H.hilo_block_workspace_bytes(sh, rows)
+    ws = torch.full((wsb,), 0xFF, dtype=torch.uint8, device="cuda")
+    H.hilo_block_forward(sh, H.DeviceWeights.from_host(w), to_dev_i32(cu), rows, H.bf16_from_bits(ut) if T else None,
+                         H.bf16_from_bits(ui), H.HILO_BF16, out, ws, wsb)
+    H.hilo_sync_status()
+    ot, oi = O.block(ut, ui, cu, T, w, heads, False)
+    got = out.cpu().numpy()
+    if T:
+        assert_block_close(got[:B * T], ot, "text rows")
+    assert_block_close(got[B * T:], oi, "image rows")
