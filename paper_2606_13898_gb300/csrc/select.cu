@@ -18,11 +18,11 @@
 //                        (magnitudes are >= +0, so their bit patterns order
 //                        like the values); the tile's maximum goes to its own
 //                        slot (no global atomics, nothing to clear).
-//   sobel_keep_kernel    one CTA per 16 x 16 tokens: the image maximum from
-//                        the tile slots, the mask tile and a halo of R
-//                        tokens in shared memory; per token: tokmax / imgmax
-//                        (one correctly rounded division) > threshold, or
-//                        any mask token within R tokens (square window).
+//   sobel_keep_kernel    one CTA per 16 x 16 tokens: the mask tile and a halo
+//                        of R tokens in shared memory, the image maximum from
+//                        the tile slots; per token: any mask token within R
+//                        tokens (square window), or tokmax / imgmax (one
+//                        correctly rounded division) > threshold.
 // Order of the magnitude, per channel c (P the replicate-padded pixels):
 //   gx = ((P(y-1,x+1) + 2 P(y,x+1)) + P(y+1,x+1)) - ((P(y-1,x-1) + 2 P(y,x-1)) + P(y+1,x-1))
 //   gy = ((P(y+1,x-1) + 2 P(y+1,x)) + P(y+1,x+1)) - ((P(y-1,x-1) + 2 P(y-1,x)) + P(y-1,x+1))
@@ -210,9 +210,12 @@ __global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float
   }
 }
 
-// One CTA per 16 x 16 tokens: the image maximum from the tile slots, the
-// mask tile with a halo of `radius` tokens in shared memory, then each
-// token's normalised maximum and its dilation window (radius <= MAX_RADIUS).
+// One CTA per 16 x 16 tokens: the mask tile with a halo of `radius` tokens in shared
+// memory and each token's dilation window (radius <= MAX_RADIUS), then the image
+// maximum from the tile slots and the token's normalised maximum. A chain of short
+// waits, no unit is busy. The mask was complete before the magnitude kernel, which
+// waits for its own predecessor, let this one start, so the dilation runs beside
+// that kernel, ahead of the wait.
 constexpr int KEEP_T = 16;
 constexpr int MAX_RADIUS = 64;
 
@@ -221,8 +224,6 @@ __global__ void __launch_bounds__(KEEP_T * KEEP_T) sobel_keep_kernel(const float
                                                                    int ntiles, const uint8_t* __restrict__ mask,
                                                                    uint8_t* __restrict__ keep, int H, int W,
                                                                    int radius, float threshold) {
-  pdl_wait();
-  pdl_trigger();
   __shared__ uint8_t mt[KEEP_T + 2 * MAX_RADIUS][KEEP_T + 2 * MAX_RADIUS];
   __shared__ uint32_t wred[KEEP_T * KEEP_T / 32];
   const int b = blockIdx.z;
@@ -231,8 +232,19 @@ __global__ void __launch_bounds__(KEEP_T * KEEP_T) sobel_keep_kernel(const float
   const uint8_t* mb = mask + static_cast<long long>(b) * H * W;
   for (int e = threadIdx.x; e < S * S; e += blockDim.x) {
     const int ii = i0 + e / S, jj = j0 + e % S;
-    mt[e / S][e % S] = (ii >= 0 && ii < H && jj >= 0 && jj < W) ? mb[ii * W + jj] : 0;
+    mt[e / S][e % S] = (ii >= 0 && ii < H && jj >= 0 && jj < W) ? __ldcg(mb + ii * W + jj) : 0;
   }
+  __syncthreads();
+  const int ti = threadIdx.x / KEEP_T, tj = threadIdx.x % KEEP_T;
+  bool k = false;
+  for (int di = 0; di <= 2 * radius && !k; ++di)
+    for (int dj = 0; dj <= 2 * radius; ++dj)
+      if (mt[ti + di][tj + dj]) {
+        k = true;
+        break;
+      }
+  pdl_wait();
+  pdl_trigger();
   uint32_t gm = 0u;
   const uint32_t* tb = tilemax + static_cast<long long>(b) * ntiles;
   for (int e = threadIdx.x; e < ntiles; e += blockDim.x) gm = max(gm, tb[e]);
@@ -242,20 +254,12 @@ __global__ void __launch_bounds__(KEEP_T * KEEP_T) sobel_keep_kernel(const float
   gm = wred[0];
 #pragma unroll
   for (int w = 1; w < KEEP_T * KEEP_T / 32; ++w) gm = max(gm, wred[w]);
-  const int ti = threadIdx.x / KEEP_T, tj = threadIdx.x % KEEP_T;
   const int i = blockIdx.y * KEEP_T + ti, j = blockIdx.x * KEEP_T + tj;
   if (i >= H || j >= W) return;
   const long long t = (static_cast<long long>(b) * H + i) * W + j;
   // 0 / 0 (an image without any gradient) is NaN and selects nothing
   const float f = __fdiv_rn(tokmax[t], __uint_as_float(gm));
-  bool k = f > threshold;
-  for (int di = 0; di <= 2 * radius && !k; ++di)
-    for (int dj = 0; dj <= 2 * radius; ++dj)
-      if (mt[ti + di][tj + dj]) {
-        k = true;
-        break;
-      }
-  keep[t] = k ? 1 : 0;
+  keep[t] = k || f > threshold ? 1 : 0;
 }
 
 }  // namespace
