@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(SCORE_THREADS) score_kernel(const __nv_bfloat1
 // ============================================================== split =====
 
 constexpr int SPLIT_THREADS = 1024;
+constexpr int SPLIT_CLUSTER = 8;  // images whose row offsets one cluster of CTAs finds
 
 // Exclusive scan of one int per thread over a 1024-thread block.
 __device__ __forceinline__ int block_excl_scan(int v, int* warp_tot, int* total) {
@@ -159,6 +160,7 @@ struct SelectShared {
   int sel_digit;
   int sel_k;
   int sel_all;
+  int rows[SPLIT_CLUSTER];  // packed rows of each image of the cluster
 };
 
 // Exclusive scans of three ints per thread at once (one pass of barriers).
@@ -389,9 +391,12 @@ __device__ void compact_image(const uint8_t* lab, int b, int H, int W, int level
 // Labels and per-image counts. One CTA per image; thread t owns the tokens
 // t CH .. t CH + CH - 1, whose scores stay in its registers (CH is the smallest of
 // 4, 8, 16, 32 for which 1024 threads cover the image, and no more threads are
-// launched than own tokens, but at least 256). With a single image (fused != 0)
-// the same CTA also writes cu_img and the packed rows, as nothing depends on
-// other images. granular != 0 is the window-granular split: every pooling window
+// launched than own tokens, but at least 256). With fused != 0 the same CTA also
+// writes cu_img and the packed rows: with 1 the image is the only one and its rows
+// begin at 0; above that it is the size of the one cluster that all images' CTAs
+// form, in which each CTA tells the others its row count. (Three images of 46x30 took
+// 7.2 us with a second kernel for the rows, 5.1 so; four of 64x64 10.0 and 7.4.)
+// granular != 0 is the window-granular split: every pooling window
 // takes the finest class of its members (an aligned 2x2 window with a kept member
 // is kept whole; with two levels an aligned 4x4 block is pooled 4x4 only when all
 // its members rank below the k_mid cut, else its non-kept members are pooled 2x2).
@@ -402,7 +407,7 @@ template <int CH, bool GRANULAR, bool LFMODE>
 __global__ void __launch_bounds__(SPLIT_THREADS) split_select_kernel(
     const float* __restrict__ score, const uint8_t* __restrict__ mask,
     const int32_t* __restrict__ k_keep, const int32_t* __restrict__ k_mid, uint8_t* labels_out,
-    int32_t* counts, int H, int W, int levels, int lf_arg, int fused, int32_t* cu_img,
+    int32_t* counts, int B, int H, int W, int levels, int lf_arg, int fused, int32_t* cu_img,
     int32_t* row_src, int32_t* tok_row) {
   // the modes are template parameters, so the plain split carries none of
   // their code (this CTA has up to 1024 threads and at most 64 registers each)
@@ -414,6 +419,14 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_select_kernel(
   __shared__ __align__(16) SelectShared sh;
   const int N = H * W;
   const int b = blockIdx.x;
+  if (fused > 1) {
+    cluster_arrive_relaxed();
+    if (b >= B) {  // the cluster is a power of two
+      cluster_wait();
+      cluster_sync();
+      return;
+    }
+  }
   uint8_t* lab = smem_raw;  // the labels, padded to the threads' tokens
   const long long base = static_cast<long long>(b) * N;
   const int k = min(max(k_keep[b], 0), N);
@@ -564,13 +577,24 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_select_kernel(
   r4 = __popc(has4);
   int nk, n2, n4;
   block_excl_scan3(rk, r2, r4, sh.warp_tot3, nk, n2, n4);
+  // the image's first packed row
+  int row0 = 0;
+  if (fused > 1) {
+    cluster_wait();  // every CTA has begun: its shared memory may be written
+    if (static_cast<int>(threadIdx.x) < fused)
+      st_shared_cluster(mapa_shared(smem_u32(&sh.rows[b]), threadIdx.x), nk + n2 + n4);
+    __syncwarp();
+    cluster_sync();
+    for (int j = 0; j < b; ++j) row0 += sh.rows[j];
+    rk += row0, r2 += row0, r4 += row0;
+  }
   if (threadIdx.x == 0) {
     counts[3 * b + 0] = nk;
     counts[3 * b + 1] = n2;
     counts[3 * b + 2] = n4;
     if (fused) {
-      cu_img[0] = 0;
-      cu_img[1] = nk + n2 + n4;
+      if (b == 0) cu_img[0] = 0;
+      cu_img[b + 1] = row0 + nk + n2 + n4;
     }
   }
   if (!fused) return;
@@ -1289,10 +1313,17 @@ cudaError_t launch_split(const float* score, const uint8_t* mask, const int32_t*
   threads = threads < 256 ? 256 : threads;
   auto* kern = lf ? split_kernel_for<false, true>(ch)
                   : (granular ? split_kernel_for<true, false>(ch) : split_kernel_for<false, false>(ch));
-  const int fused = B == 1 ? 1 : 0;
+  // One image: its rows begin at 0. Up to SPLIT_CLUSTER (8, the largest cluster every
+  // device takes): the images' CTAs are one cluster, padded to a power of two, and tell
+  // one another their row counts. More: a second kernel, once all counts are written
+  // (eight images of 64x64 took 10.3 us that way, 7.6 as a cluster).
+  int fused = 1;
+  while (fused < B && fused <= SPLIT_CLUSTER) fused *= 2;
+  if (fused > SPLIT_CLUSTER) fused = 0;
   // at most 32 KB of labels: no larger shared-memory limit to ask for
-  const cudaError_t e = launch_pdl(kern, dim3(B), dim3(threads), N, st, score, mask, k_keep, k_mid, labels, counts,
-                                   H, W, levels, lf, fused, cu_img, row_src, tok_row);
+  const cudaError_t e =
+      launch_pdl_cluster(kern, fused > 1 ? fused : 1, dim3(fused > 1 ? fused : B), dim3(threads), N, st, score, mask,
+                         k_keep, k_mid, labels, counts, B, H, W, levels, lf, fused, cu_img, row_src, tok_row);
   if (e != cudaSuccess || fused) return e;
   return launch_pdl(split_compact_kernel, dim3(B), dim3(SPLIT_THREADS), N, st,
                     static_cast<const uint8_t*>(labels), static_cast<const int32_t*>(counts), cu_img,

@@ -1,6 +1,7 @@
 """The bandwidth kernels and the attention's schedule where their code changes
-path: the split at the sizes where a thread's number of tokens doubles, in each
-mode and on arrays that allow no wide load; e4m3 rows at the ends of the widths
+path: the split at the sizes where a thread's number of tokens doubles, for one
+image, clusters of images (2, 5, 8) and more than a cluster (9), in each mode and on
+arrays that allow no wide load; e4m3 rows at the ends of the widths
 that stay in registers; LayerNorm rows below, at and above one pass of the
 resident groups; attention over images of different length, with more query
 tiles than SMs, and more images than the offsets kept in shared memory."""
@@ -31,7 +32,7 @@ def offset_by_one(a):
 
 
 @pytest.mark.parametrize("mode", ["plain1", "plain2", "regions2", "lf4"])
-@pytest.mark.parametrize("B", [1, 2])
+@pytest.mark.parametrize("B", [1, 2, 5, 8, 9])
 @pytest.mark.parametrize("Hh,W", [(4, 4), (64, 64), (64, 68), (64, 128), (64, 132), (128, 128), (128, 132)])
 def test_split_at_tokens_per_thread(H, Hh, W, B, mode):
     rng = np.random.default_rng(Hh * W + B)
