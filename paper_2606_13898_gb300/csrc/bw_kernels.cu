@@ -400,9 +400,10 @@ __device__ void compact_image(const uint8_t* lab, int b, int H, int W, int level
 // takes the finest class of its members (an aligned 2x2 window with a kept member
 // is kept whole; with two levels an aligned 4x4 block is pooled 4x4 only when all
 // its members rank below the k_mid cut, else its non-kept members are pooled 2x2).
-// Bound by one SM's latency: barriers, shared atomics and dependent loads. With
-// the keys in shared memory and re-read by each pass (contiguous chunks per
-// thread, up to 16-way bank conflicts) two levels on 128x128 took 66 us.
+// Bound by one SM's latency: barriers, shared atomics and dependent loads. (With
+// the keys in shared memory and re-read by each pass, in contiguous chunks per
+// thread with up to 16-way bank conflicts, two levels on 128x128 took 68 us, 34 so
+// on the hot path's scores, and 64x64 10.5 and 9.1.)
 template <int CH, bool GRANULAR, bool LFMODE>
 __global__ void __launch_bounds__(SPLIT_THREADS) split_select_kernel(
     const float* __restrict__ score, const uint8_t* __restrict__ mask,
@@ -734,6 +735,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const __nv_bfloat16* __restri
   for (long long gw = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
        gw < static_cast<long long>(total) * PACK_WARPS_PER_ROW; gw += nwarps) {
     // from the last row down: an image's pooled rows, 4x4 last, take the longest
+    // (128x128 with two levels 37.5 -> 35.6 us, 64x64 8.9 -> 8.1)
     const int r = total - 1 - static_cast<int>(gw / PACK_WARPS_PER_ROW);
     const int c0 = lane + 32 * static_cast<int>(gw % PACK_WARPS_PER_ROW);
     constexpr int CSTEP = 32 * PACK_WARPS_PER_ROW;
@@ -988,6 +990,8 @@ __global__ void __launch_bounds__(256) unpack_update_kernel(const float* __restr
 // Bound by memory latency: a row is one load round trip, two dependent
 // reductions and a store, so each group loads its next row before it reduces the
 // present one, and every row of a 2400-row block is asked for within two trips.
+// (One CTA per row took 6 us until the last had started: 2389 bf16 rows of 3072
+// elements 14.2 us, 5.7 so; fp32 rows 10 and 7; 10600 bf16 rows 45 and 25.)
 
 constexpr int LN_GROUP = 128;
 constexpr int LN_GROUPS = 3;
@@ -1143,7 +1147,10 @@ __global__ void __launch_bounds__(LN_THREADS, 2) layernorm_kernel(const void* __
 // multiple of 8. Rows: rows_static, or n_txt + min(cu_img[B], cap) when cu_img is
 // given (the row space of the block). Bound by memory: 16-bit rows of up to 2048 NP
 // elements (NP > 0) are read once and stay in registers while the next row is on its
-// way; longer or fp32 rows (NP = 0) are read a second time, from L1 / L2.
+// way; longer or fp32 rows (NP = 0) are read a second time, from L1 / L2. (The block
+// of 2389 rows with e4m3 operands, which has two such passes, takes 6 us less than
+// with all rows read twice. 12288 elements are what a thread can hold with three CTAs
+// per SM: 80 registers.)
 
 constexpr int QR_THREADS = 256;
 
@@ -1307,7 +1314,9 @@ cudaError_t launch_split(const float* score, const uint8_t* mask, const int32_t*
                          int32_t* cu_img, int32_t* tok_row, int B, int H, int W, int levels,
                          int granular, int lf, cudaStream_t st) {
   const int N = H * W;
-  int ch = 4;  // tokens per thread
+  // tokens per thread: as few as 1024 threads allow (half as many threads take 17.2
+  // instead of 13.4 us for 96x96 and 25.5 instead of 21.7 for 128x128)
+  int ch = 4;
   while (ch < 32 && N > ch * SPLIT_THREADS) ch *= 2;
   int threads = (((N + ch - 1) / ch + 31) / 32) * 32;
   threads = threads < 256 ? 256 : threads;

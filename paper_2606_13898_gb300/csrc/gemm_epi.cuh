@@ -13,6 +13,8 @@
 //   bf16 / fp16          neighbouring lanes exchange one value of two rows, so
 //                        that each lane stores two features of one row (a
 //                        store instruction writes 64 bytes of two rows)
+// A chunk of 32 rows takes a warp pair about 700 cycles, with a residual to load
+// 1200, which the next tile's main loop hides except at the end of a launch.
 #pragma once
 
 #include <cuda_bf16.h>
