@@ -884,7 +884,57 @@ __global__ void __launch_bounds__(256) row_sizes_kernel(const uint8_t* __restric
 }
 
 // ============================================================= unpack =====
+//
+// One warp per token, bound by HBM. Where the fp32 arrays begin on 32 bytes (WIDE) a
+// lane moves eight channels at a time, 32 bytes of fp32 in one access, and issues all
+// loads of a batch of two or four such pieces before the first store; else 16 bytes
+// at a time as the compiler unrolls it, which is the better order for those.
+// (128x128 tokens of 3072 channels: nearest 45.6 us wide and 47.5 narrow, delta 60.8
+// and 62.1; 64x64: 14.5 and 15.6, 17.9 and 19.2. Batches of 16-byte accesses took 57.7
+// and 64.2 us at 128x128. Before, delta took 67.2 and 19.0: its 16-byte stores each
+// wrote half of every 32-byte sector.)
 
+struct F8 {
+  float v[8];
+};
+
+// (volatile: the loads of a batch stay ahead of its stores)
+__device__ __forceinline__ F8 ldg8(const float* p) {
+  F8 r;
+  asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]), "=f"(r.v[4]), "=f"(r.v[5]), "=f"(r.v[6]),
+                 "=f"(r.v[7])
+               : "l"(p));
+  return r;
+}
+
+__device__ __forceinline__ void stcs8(float* p, const F8& r) {
+  asm volatile("st.global.cs.v8.f32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"f"(r.v[0]), "f"(r.v[1]), "f"(r.v[2]),
+               "f"(r.v[3]), "f"(r.v[4]), "f"(r.v[5]), "f"(r.v[6]), "f"(r.v[7]), "l"(p)
+               : "memory");
+}
+
+// One row of d channels; U pieces per lane in flight.
+template <bool WIDE, int U>
+__device__ __forceinline__ void copy_row(const float* __restrict__ s, float* __restrict__ o, int d, int lane) {
+  if (!WIDE) {
+#pragma unroll(2 * U)
+    for (int c = lane; c < (d >> 2); c += 32)
+      __stcs(reinterpret_cast<float4*>(o) + c, __ldg(reinterpret_cast<const float4*>(s) + c));
+    return;
+  }
+  for (int c = lane; c < (d >> 3); c += 32 * U) {
+    F8 v[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (c + 32 * k < (d >> 3)) v[k] = ldg8(s + 8 * (c + 32 * k));
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (c + 32 * k < (d >> 3)) stcs8(o + 8 * (c + 32 * k), v[k]);
+  }
+}
+
+template <bool WIDE>
 __global__ void __launch_bounds__(256) unpack_kernel(const float* __restrict__ out_img,
                                                      const int32_t* __restrict__ tok_row,
                                                      float* __restrict__ y, long long ntok,
@@ -897,56 +947,82 @@ __global__ void __launch_bounds__(256) unpack_kernel(const float* __restrict__ o
        t < ntok; t += wstep) {
     const int r = __ldg(tok_row + t);
     if (!HILO_DCHECK(r >= 0 && r < rows_max, DCHECK_UNPACK_ROW)) continue;
-    const float4* s = reinterpret_cast<const float4*>(out_img + static_cast<long long>(r) * d);
-    float4* o = reinterpret_cast<float4*>(y + t * d);
-    // eight loads in flight per lane (128x128, 290 MB: 48 us against 53.6 as the
-    // compiler unrolled it)
-#pragma unroll 8
-    for (int c = lane; c < (d >> 2); c += 32) __stcs(o + c, __ldg(s + c));
+    copy_row<WIDE, 4>(out_img + static_cast<long long>(r) * d, y + t * d, d, lane);
   }
 }
 
 // Delta unpool: a kept token copies its output row; a pooled member keeps
 // its own value plus its window's update, y = x + (out - packed), one fp32
-// subtract then one fp32 add (x and packed widened from bf16).
-__global__ void __launch_bounds__(256) unpack_delta_kernel(const float* __restrict__ out_img,
-                                                           const __nv_bfloat16* __restrict__ packed,
-                                                           const __nv_bfloat16* __restrict__ x,
-                                                           const uint8_t* __restrict__ labels,
-                                                           const int32_t* __restrict__ tok_row,
-                                                           float* __restrict__ y, long long ntok, int d,
-                                                           long long rows_max) {
+// subtract then one fp32 add (x and packed widened from bf16). Four CTAs per SM:
+// small grids need the warps (46x30 tokens of 1152 channels, batch of three: 9.2 us
+// with 94 registers and three pieces in flight).
+template <bool WIDE>
+__global__ void __launch_bounds__(256, WIDE ? 4 : 1) unpack_delta_kernel(const float* __restrict__ out_img,
+                                                              const __nv_bfloat16* __restrict__ packed,
+                                                              const __nv_bfloat16* __restrict__ x,
+                                                              const uint8_t* __restrict__ labels,
+                                                              const int32_t* __restrict__ tok_row,
+                                                              float* __restrict__ y, long long ntok, int d,
+                                                              long long rows_max) {
   pdl_wait();
   pdl_trigger();
+  constexpr int U = 2;
   const int lane = threadIdx.x & 31;
+  const int G = d >> 3;
   const long long wstep = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
   for (long long t = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
        t < ntok; t += wstep) {
     const int r = __ldg(tok_row + t);
     if (!HILO_DCHECK(r >= 0 && r < rows_max, DCHECK_UNPACK_DELTA_ROW)) continue;
-    const float4* s = reinterpret_cast<const float4*>(out_img + static_cast<long long>(r) * d);
-    float4* o = reinterpret_cast<float4*>(y + t * d);
+    const float* s = out_img + static_cast<long long>(r) * d;
+    float* o = y + t * d;
     if (__ldg(labels + t) == HILO_LABEL_KEEP) {
-      for (int c = lane; c < (d >> 2); c += 32) __stcs(o + c, __ldg(s + c));
+      copy_row<WIDE, U>(s, o, d, lane);
       continue;
     }
     const uint4* xr = reinterpret_cast<const uint4*>(x + t * d);
     const uint4* pr = reinterpret_cast<const uint4*>(packed + static_cast<long long>(r) * d);
-    for (int c = lane; c < (d >> 3); c += 32) {
-      float xf[8], pf[8];
-      bf16x8_to_f32(__ldg(xr + c), xf);
-      bf16x8_to_f32(__ldg(pr + c), pf);
-      const float4 o0 = __ldg(s + 2 * c), o1 = __ldg(s + 2 * c + 1);
-      const float ov[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
-      float v[8];
+    if (!WIDE) {
+      for (int c = lane; c < G; c += 32) {
+        float xf[8], pf[8];
+        bf16x8_to_f32(__ldg(xr + c), xf);
+        bf16x8_to_f32(__ldg(pr + c), pf);
+        const float4 o0 = __ldg(reinterpret_cast<const float4*>(s) + 2 * c);
+        const float4 o1 = __ldg(reinterpret_cast<const float4*>(s) + 2 * c + 1);
+        const float ov[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
+        float v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = __fadd_rn(xf[u], __fsub_rn(ov[u], pf[u]));
-      __stcs(o + 2 * c, make_float4(v[0], v[1], v[2], v[3]));
-      __stcs(o + 2 * c + 1, make_float4(v[4], v[5], v[6], v[7]));
+        for (int u = 0; u < 8; ++u) v[u] = __fadd_rn(xf[u], __fsub_rn(ov[u], pf[u]));
+        __stcs(reinterpret_cast<float4*>(o) + 2 * c, make_float4(v[0], v[1], v[2], v[3]));
+        __stcs(reinterpret_cast<float4*>(o) + 2 * c + 1, make_float4(v[4], v[5], v[6], v[7]));
+      }
+      continue;
+    }
+    for (int c = lane; c < G; c += 32 * U) {
+      uint4 xv[U], pv[U];
+      F8 v[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+        if (c + 32 * k < G) {
+          xv[k] = __ldg(xr + c + 32 * k);
+          pv[k] = __ldg(pr + c + 32 * k);
+          v[k] = ldg8(s + 8 * (c + 32 * k));
+        }
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+        if (c + 32 * k < G) {
+          float xf[8], pf[8];
+          bf16x8_to_f32(xv[k], xf);
+          bf16x8_to_f32(pv[k], pf);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) v[k].v[u] = __fadd_rn(xf[u], __fsub_rn(v[k].v[u], pf[u]));
+          stcs8(o + 8 * (c + 32 * k), v[k]);
+        }
     }
   }
 }
 
+template <bool WIDE>
 __global__ void __launch_bounds__(256) unpack_update_kernel(const float* __restrict__ out_img,
                                                             const int32_t* __restrict__ tok_row,
                                                             __nv_bfloat16* __restrict__ x,
@@ -954,28 +1030,45 @@ __global__ void __launch_bounds__(256) unpack_update_kernel(const float* __restr
                                                             long long rows_max) {
   pdl_wait();
   pdl_trigger();
+  constexpr int U = 2;
   const int lane = threadIdx.x & 31;
+  const int G = d >> 3;
   const long long wstep = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
   for (long long t = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
        t < ntok; t += wstep) {
     const int r = __ldg(tok_row + t);
     if (!HILO_DCHECK(r >= 0 && r < rows_max, DCHECK_UNPACK_UPDATE_ROW)) continue;
-    const float4* s = reinterpret_cast<const float4*>(out_img + static_cast<long long>(r) * d);
+    const float* s = out_img + static_cast<long long>(r) * d;
     uint4* xr = reinterpret_cast<uint4*>(x + t * d);
-    for (int c = lane; c < (d >> 3); c += 32) {
-      float f[8];
-      bf16x8_to_f32(xr[c], f);
-      const float4 y0 = __ldg(s + 2 * c), y1 = __ldg(s + 2 * c + 1);
-      const float yv[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
-      float o[8];
+    for (int c = lane; c < G; c += 32 * U) {
+      uint4 xv[U];
+      F8 yv[U];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) o[u] = __fsub_rn(f[u], __fmul_rn(alpha, yv[u]));
-      uint4 v;
-      v.x = pack_bf16x2(o[0], o[1]);
-      v.y = pack_bf16x2(o[2], o[3]);
-      v.z = pack_bf16x2(o[4], o[5]);
-      v.w = pack_bf16x2(o[6], o[7]);
-      xr[c] = v;
+      for (int k = 0; k < U; ++k)
+        if (c + 32 * k < G) {
+          xv[k] = xr[c + 32 * k];
+          if (WIDE) {
+            yv[k] = ldg8(s + 8 * (c + 32 * k));
+          } else {
+            const float4* s4 = reinterpret_cast<const float4*>(s) + 2 * (c + 32 * k);
+            const float4 lo = __ldg(s4), hi = __ldg(s4 + 1);
+            yv[k] = {{lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w}};
+          }
+        }
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+        if (c + 32 * k < G) {
+          float f[8], o[8];
+          bf16x8_to_f32(xv[k], f);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) o[u] = __fsub_rn(f[u], __fmul_rn(alpha, yv[k].v[u]));
+          uint4 v;
+          v.x = pack_bf16x2(o[0], o[1]);
+          v.y = pack_bf16x2(o[2], o[3]);
+          v.z = pack_bf16x2(o[4], o[5]);
+          v.w = pack_bf16x2(o[6], o[7]);
+          xr[c + 32 * k] = v;
+        }
     }
   }
 }
@@ -1352,9 +1445,16 @@ cudaError_t launch_pack(const void* x, const uint8_t* labels, const int32_t* row
   return launch_pdl(pack_kernel, grid, dim3(256), 0, st, xs, labels, row_src, counts, cu_img, ps, B, H, W, d, cap);
 }
 
+// 32-byte accesses on fp32 rows: a row is a multiple of 512 bytes, so the arrays'
+// addresses decide.
+static bool wide(const float* a, const float* b) {
+  return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 31) == 0;
+}
+
 cudaError_t launch_unpack(const float* out_img, const int32_t* tok_row, float* y, long long ntok,
                           int d, long long rows_max, int num_sms, cudaStream_t st) {
-  return launch_pdl(unpack_kernel, dim3(grid_for(ntok, 8, num_sms, 8)), dim3(256), 0, st, out_img,
+  auto* kern = wide(out_img, y) ? unpack_kernel<true> : unpack_kernel<false>;
+  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, 8)), dim3(256), 0, st, out_img,
                     tok_row, y, ntok, d, rows_max);
 }
 
@@ -1369,7 +1469,8 @@ cudaError_t launch_row_sizes(const uint8_t* labels, const int32_t* row_src, cons
 cudaError_t launch_unpack_delta(const float* out_img, const void* packed, const void* x,
                                 const uint8_t* labels, const int32_t* tok_row, float* y, long long ntok,
                                 int d, long long rows_max, int num_sms, cudaStream_t st) {
-  return launch_pdl(unpack_delta_kernel, dim3(grid_for(ntok, 8, num_sms, 8)), dim3(256), 0, st, out_img,
+  auto* kern = wide(out_img, y) ? unpack_delta_kernel<true> : unpack_delta_kernel<false>;
+  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, 8)), dim3(256), 0, st, out_img,
                     static_cast<const __nv_bfloat16*>(packed), static_cast<const __nv_bfloat16*>(x), labels,
                     tok_row, y, ntok, d, rows_max);
 }
@@ -1377,7 +1478,8 @@ cudaError_t launch_unpack_delta(const float* out_img, const void* packed, const 
 cudaError_t launch_unpack_update(const float* out_img, const int32_t* tok_row, void* x,
                                  long long ntok, int d, float alpha, long long rows_max, int num_sms,
                                  cudaStream_t st) {
-  return launch_pdl(unpack_update_kernel, dim3(grid_for(ntok, 8, num_sms, 8)), dim3(256), 0, st,
+  auto* kern = wide(out_img, out_img) ? unpack_update_kernel<true> : unpack_update_kernel<false>;
+  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, 8)), dim3(256), 0, st,
                     out_img, tok_row, static_cast<__nv_bfloat16*>(x), ntok, d, alpha, rows_max);
 }
 

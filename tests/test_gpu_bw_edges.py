@@ -1,7 +1,8 @@
 """The bandwidth kernels and the attention's schedule where their code changes
 path: the split at the sizes where a thread's number of tokens doubles, for one
 image, clusters of images (2, 5, 8) and more than a cluster (9), in each mode and on
-arrays that allow no wide load; e4m3 rows at the ends of the widths
+arrays that allow no wide load; the three unpools on fp32 arrays that allow 32-byte
+accesses and that do not; e4m3 rows at the ends of the widths
 that stay in registers; LayerNorm rows below, at and above one pass of the
 resident groups; attention over images of different length, with more query
 tiles than SMs, and more images than the offsets kept in shared memory."""
@@ -51,6 +52,39 @@ def test_split_at_tokens_per_thread(H, Hh, W, B, mode):
     ref = (O.split(s, mask, kk, km, Hh, W, levels, lf=lf) if lf else
            O.split(s, mask, kk, km, Hh, W, levels, granular=mode == "regions2"))
     check_split(sp, ref, B, N)
+
+
+@pytest.mark.parametrize("off", [0, 4])  # floats past a 32-byte boundary: 32- and 16-byte accesses
+@pytest.mark.parametrize("d", [128, 384, 3072, 4096])
+def test_unpack_at_both_alignments(H, d, off):
+    rng = np.random.default_rng(d + off)
+    B, Hh, W = 2, 8, 12
+    N = Hh * W
+    x = bits(rng.standard_normal((B, Hh, W, d)))
+    ref = O.split(O.score(x), (rng.random((B, N)) < 0.1).astype(np.uint8), np.array([N // 4, 5], np.int32),
+                  np.array([N // 4, 9], np.int32), Hh, W, 2)
+    rows = int(ref.cu_img[-1])
+    pk, out = O.pack(x, ref), rng.standard_normal((rows, d)).astype(np.float32)
+    sh = H.Shape(B=B, H=Hh, W=W, d=d, levels=2)
+    sp = H.SplitBuffers.alloc(sh)
+    sp.labels.copy_(torch.from_numpy(ref.labels.reshape(-1)))
+    sp.tok_row.copy_(torch.from_numpy(ref.tok_row.reshape(-1)))
+    buf = torch.full((rows * d + 8,), float("nan"), dtype=torch.float32, device="cuda")
+    od = buf[off:off + rows * d]
+    od.copy_(torch.from_numpy(out.reshape(-1)))
+    xd, pd = H.bf16_from_bits(x), H.bf16_from_bits(pk)
+    ybuf = torch.full((B * N * d + 8,), 7.0, dtype=torch.float32, device="cuda")
+    y = ybuf[off:off + B * N * d]
+    for want, call in ((O.unpack(out, ref), lambda: H.hilo_unpack(sh, od, sp, y)),
+                       (O.unpack_delta(out, pk, x, ref), lambda: H.hilo_unpack_delta(sh, od, pd, xd, sp, y))):
+        ybuf.fill_(7.0)
+        call()
+        H.hilo_sync_status()
+        assert np.array_equal(y.cpu().numpy().reshape(want.shape), want)
+        assert torch.all(ybuf[:off] == 7.0) and torch.all(ybuf[off + B * N * d:] == 7.0)
+    H.hilo_unpack_update(sh, od, sp, xd, 0.035)
+    H.hilo_sync_status()
+    assert np.array_equal(H.bits_from_bf16(xd).reshape(x.shape), O.update(x, O.unpack(out, ref).reshape(x.shape), 0.035))
 
 
 @pytest.mark.parametrize("dtype,cols", [("bf16", 8), ("bf16", 4096), ("bf16", 4104), ("bf16", 12288),
