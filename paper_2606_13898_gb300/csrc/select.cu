@@ -5,19 +5,24 @@
 //
 // Two kernels:
 //   sobel_tokmax_kernel  one CTA per 32 x 64 pixel tile (plus a one-pixel
-//                        halo, replicate borders) in shared memory, channel
-//                        planes; full-width tiles load their interior as
-//                        16-byte vectors. Each thread walks 8 consecutive
-//                        pixel rows of one column, so the horizontal sums of
-//                        a row serve as the bottom term of one pixel and the
-//                        top term of the pixel two rows below (the same
-//                        value, not a re-association). The largest magnitude
-//                        of each token comes from per-thread maxima, a warp
-//                        reduction over the lanes of one token and one shared
-//                        atomic per token and warp, on the float bits
-//                        (magnitudes are >= +0, so their bit patterns order
-//                        like the values); the tile's maximum goes to its own
-//                        slot (no global atomics, nothing to clear).
+//                        halo, replicate borders) in shared memory, pixels as
+//                        in the image; full-width tiles load and store their
+//                        interior as 16-byte vectors. Each thread walks 8
+//                        consecutive pixel rows of one column, so the
+//                        horizontal sums of a row serve as the bottom term of
+//                        one pixel and the top term of the pixel two rows
+//                        below (the same value, not a re-association). The
+//                        largest squared magnitude of each token comes from
+//                        per-thread maxima, a warp reduction over the lanes
+//                        of one token and one shared atomic per token and
+//                        warp, on the float bits (squares are >= +0, so their
+//                        bit patterns order like the values); the square root
+//                        is taken once per token (it keeps the order). The
+//                        tile's maximum goes to its own slot (no global
+//                        atomics, nothing to clear). Bound by instruction
+//                        issue: 1024x1024 pixels of 3 channels 7.4 us with the
+//                        keep kernel, 8.9 with channel planes and a root per
+//                        pixel; 2048x2048 20.2 and 24.1.
 //   sobel_keep_kernel    one CTA per 16 x 16 tokens: the mask tile and a halo
 //                        of R tokens in shared memory, the image maximum from
 //                        the tile slots; per token: any mask token within R
@@ -49,14 +54,31 @@ __device__ __forceinline__ float sobel_sum3(float a, float b, float c) {
   return __fadd_rn(__fadd_rn(a, __fmul_rn(2.0f, b)), c);
 }
 
+// The C channels of one pixel of the tile. (Lanes are C floats apart: one float at a
+// time meets no bank conflict for odd C, and even C takes one vector.)
+template <int C>
+__device__ __forceinline__ void load_pixel(const float* p, float (&v)[C]) {
+  if constexpr (C == 4) {
+    const float4 f = *reinterpret_cast<const float4*>(p);
+    v[0] = f.x, v[1] = f.y, v[2] = f.z, v[3] = f.w;
+  } else if constexpr (C == 2) {
+    const float2 f = *reinterpret_cast<const float2*>(p);
+    v[0] = f.x, v[1] = f.y;
+  } else {
+#pragma unroll
+    for (int c = 0; c < C; ++c) v[c] = p[c];
+  }
+}
+
 // Tiles of the tokmax grid for an H x W-token image at `patch` pixels per
 // token: one maximum slot each.
 inline int sobel_tiles(int H, int W, int patch) {
   return ((W * patch + TILE_X - 1) / TILE_X) * ((H * patch + TILE_Y - 1) / TILE_Y);
 }
 
+// Five CTAs per SM, as far as registers and tiles allow (six spill and are slower).
 template <int P, int C>
-__global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float* __restrict__ img,
+__global__ void __launch_bounds__(SOBEL_THREADS, C == 4 ? 4 : 5) sobel_tokmax_kernel(const float* __restrict__ img,
                                                                      float* __restrict__ tokmax,
                                                                      uint32_t* __restrict__ tilemax, int H,
                                                                      int W, int vec_ok) {
@@ -64,7 +86,9 @@ __global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float
   pdl_trigger();
   constexpr int TOK_Y = TILE_Y / P, TOK_X = TILE_X / P;
   static_assert(TOK_Y * TOK_X <= 32, "token maxima of a tile fit one warp");
-  __shared__ float tile[C][TILE_Y + 2][TILE_X + 2];
+  // a row: the left halo pixel ends at FIRST, where the 64 pixels begin
+  constexpr int FIRST = 4, STRIDE = TILE_X * C + 2 * FIRST;
+  __shared__ __align__(16) float tile[TILE_Y + 2][STRIDE];
   __shared__ uint32_t tmax[TOK_Y * TOK_X];
   const int Hp = H * P, Wp = W * P;
   const int b = blockIdx.z;
@@ -109,16 +133,7 @@ __global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float
       const int e = threadIdx.x + k * SOBEL_THREADS;
       if (e < NV) {
         const int yy = e / V, m = e - yy * V;
-        int px = (4 * m) / C, c = 4 * m - px * C;
-        const float f[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          tile[c][yy][1 + px] = f[i];
-          if (++c == C) {
-            c = 0;
-            ++px;
-          }
-        }
+        *reinterpret_cast<float4*>(&tile[yy][FIRST + 4 * m]) = v[k];
       }
     }
 #pragma unroll
@@ -127,7 +142,7 @@ __global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float
       if (e < NH) {
         const int yy = e / (2 * C), w = e - yy * (2 * C);
         const int side = w / C, c = w - side * C;
-        tile[c][yy][side ? TILE_X + 1 : 0] = h[k];
+        tile[yy][(side ? FIRST + TILE_X * C : FIRST - C) + c] = h[k];
       }
     }
   } else {
@@ -140,7 +155,7 @@ __global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float
       const int xx = w / C, c = w - xx * C;
       const int gy = min(max(y0 + yy - 1, 0), Hp - 1);
       const int gx = min(max(x0 + xx - 1, 0), Wp - 1);
-      tile[c][yy][xx] = __ldg(base + (static_cast<long long>(gy) * Wp + gx) * C + c);
+      tile[yy][FIRST - C + w] = __ldg(base + (static_cast<long long>(gy) * Wp + gx) * C + c);
     }
   }
   __syncthreads();
@@ -153,13 +168,20 @@ __global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float
   // sliding 3-row window per channel: up/mid/dn rows at columns q-1, q, q+1,
   // and the horizontal sums of the up and mid rows
   float up[C][3], mid[C][3], hup[C], hmid[C];
+  const int q0 = FIRST - C + (q - 1) * C;  // its left neighbour
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    float u[C], v[C];
+    load_pixel<C>(&tile[ty0][q0 + i * C], u);
+    load_pixel<C>(&tile[ty0 + 1][q0 + i * C], v);
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      up[c][i] = u[c];
+      mid[c][i] = v[c];
+    }
+  }
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      up[c][i] = tile[c][ty0][q - 1 + i];
-      mid[c][i] = tile[c][ty0 + 1][q - 1 + i];
-    }
     hup[c] = sobel_sum3(up[c][0], up[c][1], up[c][2]);
     hmid[c] = sobel_sum3(mid[c][0], mid[c][1], mid[c][2]);
   }
@@ -169,11 +191,12 @@ __global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float
   for (int j = 0; j < ROWS; ++j) {
     const int r = ty0 + 1 + j;  // row in the padded tile
     float acc = 0.0f;
+    float px[3][C];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) load_pixel<C>(&tile[r + 1][q0 + i * C], px[i]);
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      float dn[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) dn[i] = tile[c][r + 1][q - 1 + i];
+      const float dn[3] = {px[0][c], px[1][c], px[2][c]};
       const float hdn = sobel_sum3(dn[0], dn[1], dn[2]);                  // bottom
       const float right = sobel_sum3(up[c][2], mid[c][2], dn[2]);
       const float left = sobel_sum3(up[c][0], mid[c][0], dn[0]);
@@ -188,7 +211,7 @@ __global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float
       hup[c] = hmid[c];
       hmid[c] = hdn;
     }
-    if (col_ok && y0 + ty0 + j < Hp) mx = max(mx, __float_as_uint(__fsqrt_rn(acc)));
+    if (col_ok && y0 + ty0 + j < Hp) mx = max(mx, __float_as_uint(acc));
   }
   const int lane = threadIdx.x & 31;
   const uint32_t seg = (P >= 32 ? 0xffffffffu : ((1u << P) - 1u)) << (lane & ~(P - 1));
@@ -201,7 +224,8 @@ __global__ void __launch_bounds__(SOBEL_THREADS) sobel_tokmax_kernel(const float
       const int ti = blockIdx.y * TOK_Y + threadIdx.x / TOK_X;
       const int tj = blockIdx.x * TOK_X + threadIdx.x % TOK_X;
       if (ti < H && tj < W) {
-        t = tmax[threadIdx.x];
+        // a correctly rounded square root keeps the order, so one per token will do
+        t = __float_as_uint(__fsqrt_rn(__uint_as_float(tmax[threadIdx.x])));
         tokmax[(static_cast<long long>(b) * H + ti) * W + tj] = __uint_as_float(t);
       }
     }

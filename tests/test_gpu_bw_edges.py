@@ -15,6 +15,7 @@ from paper_2606_13898_gb300 import inputs as I
 
 from .gpu_helpers import assert_block_close, lib_ready, to_dev_i32
 from .test_gpu_kernels import bits, check_split, scaled_weights
+from .test_gpu_select import run_select
 
 pytestmark = pytest.mark.gpu
 
@@ -164,3 +165,24 @@ def test_attention_images_of_different_length(H, d, heads, T, lens):
     if T:
         assert_block_close(got[:B * T], ot, "text rows")
     assert_block_close(got[B * T:], oi, "image rows")
+
+
+@pytest.mark.parametrize("patch", [8, 16])
+@pytest.mark.parametrize("C", [1, 2, 3, 4])
+def test_sobel_tiles_of_every_pixel_width(H, C, patch):
+    """Full-width tiles (vector loads), a partial one at the right edge, and flat
+    image parts (magnitude 0) beside infinite and huge pixels (magnitude inf, NaN)."""
+    rng = np.random.default_rng(C + patch)
+    B, Hh, W = 2, 6, 18
+    img = rng.random((B, Hh * patch, W * patch, C)).astype(np.float32)
+    img[0, : 2 * patch] = 0.5
+    mask = np.zeros((B, Hh * W), np.uint8)
+    mask[:, 5] = 1
+    for thr in (0.1, 0.7):
+        assert np.array_equal(run_select(H, img, mask, Hh, W, patch, 1, thr),
+                              O.sobel_select(img, mask, Hh, W, patch, 1, thr))
+    img[1, patch, patch] = np.inf
+    img[1, 3 * patch + 2, 9 * patch] = 3e38
+    with np.errstate(all="ignore"):
+        assert np.array_equal(run_select(H, img, mask, Hh, W, patch, 0, 0.1),
+                              O.sobel_select(img, mask, Hh, W, patch, 0, 0.1))
