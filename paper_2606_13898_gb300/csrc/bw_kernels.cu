@@ -34,9 +34,15 @@ __device__ __forceinline__ void bf16x8_to_f32(const uint4& v, float* f) {
 }
 
 constexpr int SCORE_THREADS = 128;
-constexpr int SCORE_MAX_ITERS = 4;  // d <= 4096: at most 4 groups of 8 per thread
 
-__global__ void __launch_bounds__(SCORE_THREADS) score_kernel(const __nv_bfloat16* __restrict__ x,
+// ITERS: groups of 8 channels per thread (d <= 4096: at most 4). Bound by HBM, so by
+// the loads that the resident CTAs have in flight: with registers for four groups
+// whatever the width, 128x128 tokens of 3072 channels took 18.5 us, 16.8 so (6.0
+// TB/s), 64x64 6.8 and 6.3, 128x128 of 1024 10.8 and 8.8. Seven CTAs per SM for three
+// groups: 6.7 us for 64x64 without the limit, and for four the compiler's own count is
+// better (21.5 us at 128x128 against 22.3 with five).
+template <int ITERS>
+__global__ void __launch_bounds__(SCORE_THREADS, ITERS == 3 ? 7 : 1) score_kernel(const __nv_bfloat16* __restrict__ x,
                                                               float* __restrict__ s, int B, int H,
                                                               int W, int d) {
   pdl_wait();
@@ -56,9 +62,9 @@ __global__ void __launch_bounds__(SCORE_THREADS) score_kernel(const __nv_bfloat1
     const uint4* rb = reinterpret_cast<const uint4*>(x + (t0 + 1) * d);
     const uint4* rc = reinterpret_cast<const uint4*>(x + (t0 + W) * d);
     const uint4* rd = reinterpret_cast<const uint4*>(x + (t0 + W + 1) * d);
-    uint4 va[SCORE_MAX_ITERS], vb[SCORE_MAX_ITERS], vc[SCORE_MAX_ITERS], vd[SCORE_MAX_ITERS];
+    uint4 va[ITERS], vb[ITERS], vc[ITERS], vd[ITERS];
 #pragma unroll
-    for (int i = 0; i < SCORE_MAX_ITERS; ++i) {
+    for (int i = 0; i < ITERS; ++i) {
       const int g = j + SCORE_THREADS * i;
       if (g < G) {
         va[i] = __ldg(ra + g);
@@ -69,7 +75,7 @@ __global__ void __launch_bounds__(SCORE_THREADS) score_kernel(const __nv_bfloat1
     }
     float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f, acc3 = 0.f;
 #pragma unroll
-    for (int i = 0; i < SCORE_MAX_ITERS; ++i) {
+    for (int i = 0; i < ITERS; ++i) {
       if (j + SCORE_THREADS * i >= G) break;
       float fa[8], fb[8], fc[8], fd[8];
       bf16x8_to_f32(va[i], fa);
@@ -1388,7 +1394,9 @@ static int grid_for(long long work_items, int per_block, int num_sms, int blocks
 cudaError_t launch_score(const void* x, float* s, int B, int H, int W, int d, int num_sms,
                          cudaStream_t st) {
   const long long nwin = static_cast<long long>(B) * (H / 2) * (W / 2);
-  return launch_pdl(score_kernel, dim3(grid_for(nwin, 1, num_sms, 16)), dim3(SCORE_THREADS), 0, st,
+  const int iters = (d + 8 * SCORE_THREADS - 1) / (8 * SCORE_THREADS);
+  auto* kern = iters == 1 ? score_kernel<1> : iters == 2 ? score_kernel<2> : iters == 3 ? score_kernel<3> : score_kernel<4>;
+  return launch_pdl(kern, dim3(grid_for(nwin, 1, num_sms, 16)), dim3(SCORE_THREADS), 0, st,
                     static_cast<const __nv_bfloat16*>(x), s, B, H, W, d);
 }
 

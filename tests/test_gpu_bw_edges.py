@@ -1,11 +1,13 @@
 """The bandwidth kernels and the attention's schedule where their code changes
-path: the split at the sizes where a thread's number of tokens doubles, for one
-image, clusters of images (2, 5, 8) and more than a cluster (9), in each mode and on
-arrays that allow no wide load; the three unpools on fp32 arrays that allow 32-byte
-accesses and that do not; e4m3 rows at the ends of the widths
-that stay in registers; LayerNorm rows below, at and above one pass of the
-resident groups; attention over images of different length, with more query
-tiles than SMs, and more images than the offsets kept in shared memory."""
+path: the score where a thread takes one more group of channels; the split at
+the sizes where a thread's number of tokens doubles, for one image, clusters of
+images (2, 5, 8) and more than a cluster (9), in each mode and on arrays that
+allow no wide load; the three unpools on fp32 arrays that allow 32-byte accesses
+and that do not; e4m3 rows at the ends of the widths that stay in registers;
+LayerNorm rows below, at and above one pass of the resident groups; attention
+over images of different length, with more query tiles than SMs, and more images
+than the offsets kept in shared memory; the selector's tiles for every number of
+channels."""
 import numpy as np
 import pytest
 import torch
@@ -31,6 +33,17 @@ def offset_by_one(a):
     buf = torch.empty(t.numel() + 1, dtype=t.dtype, device="cuda")
     buf[1:] = t
     return buf[1:]
+
+
+@pytest.mark.parametrize("d", [1024, 1152, 2048, 2176, 3200, 4096])
+def test_score_at_groups_per_thread(H, d):
+    rng = np.random.default_rng(d)
+    x = bits(rng.standard_normal((2, 6, 4, d)) * rng.uniform(0.1, 10, size=(2, 6, 4, 1)))
+    s = torch.empty(48, dtype=torch.float32, device="cuda")
+    H.hilo_score(H.Shape(B=2, H=6, W=4, d=d), H.bf16_from_bits(x), s)
+    H.hilo_sync_status()
+    ref = O.score(x)
+    assert np.array_equal(s.cpu().numpy().view(np.uint32), ref.reshape(-1).view(np.uint32))
 
 
 @pytest.mark.parametrize("mode", ["plain1", "plain2", "regions2", "lf4"])
