@@ -684,9 +684,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_compact_kernel(
 // of its lanes, so a row needs one memory round trip. A kept row is a
 // 16-byte-vector copy; a pooled row sums the window's members of its class
 // in raster order (the first member initialises the sum), divides once with
-// correct rounding and rounds to bf16 (nearest even).
+// correct rounding and rounds to bf16 (nearest even). Bound by each row's chain of
+// dependent reads (offsets, counts, row source, labels, data), so by the rows in
+// flight: a CTA per row, eight to an SM (two rows per CTA: 128x128 with two levels 31.2
+// us, 27.3 so; four of 64x64 32.4 and 28.7; 64x64 9.5 and 8.9).
 
 constexpr int PACK_WARPS_PER_ROW = 4;
+constexpr int PACK_THREADS = 32 * PACK_WARPS_PER_ROW;  // of pack_kernel: a row per CTA
 
 // A low-frequency row: the mean of all LF x LF members of the window whose
 // first member is w0 (raster order, the first initialising the sum), one
@@ -724,7 +728,7 @@ __device__ __forceinline__ void pack_lf_row(const __nv_bfloat16* __restrict__ w0
   }
 }
 
-__global__ void __launch_bounds__(256) pack_kernel(const __nv_bfloat16* __restrict__ x,
+__global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __nv_bfloat16* __restrict__ x,
                                                    const uint8_t* __restrict__ labels,
                                                    const int32_t* __restrict__ row_src,
                                                    const int32_t* __restrict__ counts,
@@ -757,7 +761,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const __nv_bfloat16* __restri
     if (!HILO_DCHECK(local >= 0 && src >= 0 && src < (H / size) * (W / size), DCHECK_PACK_SRC)) continue;
     if (local < nk) {
       const uint4* sp = reinterpret_cast<const uint4*>(xb + static_cast<long long>(src) * d);
-#pragma unroll 4
+#pragma unroll 3
       for (int c = c0; c < G; c += CSTEP) dst[c] = __ldg(sp + c);
       continue;
     }
@@ -773,7 +777,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const __nv_bfloat16* __restri
     const uint32_t mm = __ballot_sync(0xffffffffu, is_member);
     const float cnt = static_cast<float>(__popc(mm));
     const int ngroups = size * size / 4;
-#pragma unroll 2
+#pragma unroll 3
     for (int c = c0; c < G; c += CSTEP) {
       float acc[8];
       bool first = true;
@@ -1450,7 +1454,13 @@ cudaError_t launch_pack(const void* x, const uint8_t* labels, const int32_t* row
   if (lf == 4) return launch_pdl(pack_lf_kernel<4>, grid, dim3(256), 0, st, xs, row_src, counts, cu_img, ps, B, H, W, d, cap);
   if (lf == 8) return launch_pdl(pack_lf_kernel<8>, grid, dim3(256), 0, st, xs, row_src, counts, cu_img, ps, B, H, W, d, cap);
   if (lf) return cudaErrorInvalidValue;
-  return launch_pdl(pack_kernel, grid, dim3(256), 0, st, xs, labels, row_src, counts, cu_img, ps, B, H, W, d, cap);
+  // A row per CTA and turn. The hardware deals further CTAs as others end, which evens
+  // out rows of one to sixteen members, but one without a row still costs its launch,
+  // and the capacity is several times the rows: 24 per SM from about 5000 rows of
+  // capacity on, else 16 (4096 rows of 2048 channels: 5.1 us with 16, 6.2 with 24; 16384
+  // of 3072 with two levels 28.6 and 26.4; 5120 rows 10.4 and 10.2).
+  const dim3 rows(grid_for(cap, 1, num_sms, cap <= 32 * num_sms ? 16 : 24));
+  return launch_pdl(pack_kernel, rows, dim3(PACK_THREADS), 0, st, xs, labels, row_src, counts, cu_img, ps, B, H, W, d, cap);
 }
 
 // 32-byte accesses on fp32 rows: a row is a multiple of 512 bytes, so the arrays'
