@@ -39,10 +39,10 @@ constexpr int SCORE_THREADS = 128;
 // the loads that the resident CTAs have in flight: with registers for four groups
 // whatever the width, 128x128 tokens of 3072 channels took 18.5 us, 16.8 so (6.0
 // TB/s), 64x64 6.8 and 6.3, 128x128 of 1024 10.8 and 8.8. Seven CTAs per SM for three
-// groups: 6.7 us for 64x64 without the limit, and for four the compiler's own count is
-// better (21.5 us at 128x128 against 22.3 with five).
+// groups (6.7 us for 64x64 without the limit); for the others the compiler's own count
+// (128x128 of 4096: 21.5 us, 22.3 with five, 26.2 with a limit of one).
 template <int ITERS>
-__global__ void __launch_bounds__(SCORE_THREADS, ITERS == 3 ? 7 : 1) score_kernel(const __nv_bfloat16* __restrict__ x,
+__global__ void __launch_bounds__(SCORE_THREADS, ITERS == 3 ? 7 : 0) score_kernel(const __nv_bfloat16* __restrict__ x,
                                                               float* __restrict__ s, int B, int H,
                                                               int W, int d) {
   pdl_wait();
@@ -899,10 +899,10 @@ __global__ void __launch_bounds__(256) row_sizes_kernel(const uint8_t* __restric
 // lane moves eight channels at a time, 32 bytes of fp32 in one access, and issues all
 // loads of a batch of two or four such pieces before the first store; else 16 bytes
 // at a time as the compiler unrolls it, which is the better order for those.
-// (128x128 tokens of 3072 channels: nearest 45.6 us wide and 47.5 narrow, delta 60.8
-// and 62.1; 64x64: 14.5 and 15.6, 17.9 and 19.2. Batches of 16-byte accesses took 57.7
-// and 64.2 us at 128x128. Before, delta took 67.2 and 19.0: its 16-byte stores each
-// wrote half of every 32-byte sector.)
+// (128x128 tokens of 3072 channels: nearest 45.3 us wide and 47.5 narrow, delta 59.9
+// and 67.2, whose 16-byte stores each write half of every 32-byte sector; 64x64: 14.5
+// and 15.6, 17.9 and 19.0. Batches of 16-byte accesses took 57.7 and 64.2 us at
+// 128x128 and 20.5 for delta at 64x64.)
 
 struct F8 {
   float v[8];
@@ -927,20 +927,20 @@ __device__ __forceinline__ void stcs8(float* p, const F8& r) {
 // One row of d channels; U pieces per lane in flight.
 template <bool WIDE, int U>
 __device__ __forceinline__ void copy_row(const float* __restrict__ s, float* __restrict__ o, int d, int lane) {
-  if (!WIDE) {
+  if constexpr (!WIDE) {
 #pragma unroll(2 * U)
     for (int c = lane; c < (d >> 2); c += 32)
       __stcs(reinterpret_cast<float4*>(o) + c, __ldg(reinterpret_cast<const float4*>(s) + c));
-    return;
-  }
-  for (int c = lane; c < (d >> 3); c += 32 * U) {
-    F8 v[U];
+  } else {
+    for (int c = lane; c < (d >> 3); c += 32 * U) {
+      F8 v[U];
 #pragma unroll
-    for (int k = 0; k < U; ++k)
-      if (c + 32 * k < (d >> 3)) v[k] = ldg8(s + 8 * (c + 32 * k));
+      for (int k = 0; k < U; ++k)
+        if (c + 32 * k < (d >> 3)) v[k] = ldg8(s + 8 * (c + 32 * k));
 #pragma unroll
-    for (int k = 0; k < U; ++k)
-      if (c + 32 * k < (d >> 3)) stcs8(o + 8 * (c + 32 * k), v[k]);
+      for (int k = 0; k < U; ++k)
+        if (c + 32 * k < (d >> 3)) stcs8(o + 8 * (c + 32 * k), v[k]);
+    }
   }
 }
 
@@ -967,7 +967,7 @@ __global__ void __launch_bounds__(256) unpack_kernel(const float* __restrict__ o
 // small grids need the warps (46x30 tokens of 1152 channels, batch of three: 9.2 us
 // with 94 registers and three pieces in flight).
 template <bool WIDE>
-__global__ void __launch_bounds__(256, WIDE ? 4 : 1) unpack_delta_kernel(const float* __restrict__ out_img,
+__global__ void __launch_bounds__(256, WIDE ? 4 : 0) unpack_delta_kernel(const float* __restrict__ out_img,
                                                               const __nv_bfloat16* __restrict__ packed,
                                                               const __nv_bfloat16* __restrict__ x,
                                                               const uint8_t* __restrict__ labels,
@@ -992,7 +992,7 @@ __global__ void __launch_bounds__(256, WIDE ? 4 : 1) unpack_delta_kernel(const f
     }
     const uint4* xr = reinterpret_cast<const uint4*>(x + t * d);
     const uint4* pr = reinterpret_cast<const uint4*>(packed + static_cast<long long>(r) * d);
-    if (!WIDE) {
+    if constexpr (!WIDE) {
       for (int c = lane; c < G; c += 32) {
         float xf[8], pf[8];
         bf16x8_to_f32(__ldg(xr + c), xf);
@@ -1006,28 +1006,28 @@ __global__ void __launch_bounds__(256, WIDE ? 4 : 1) unpack_delta_kernel(const f
         __stcs(reinterpret_cast<float4*>(o) + 2 * c, make_float4(v[0], v[1], v[2], v[3]));
         __stcs(reinterpret_cast<float4*>(o) + 2 * c + 1, make_float4(v[4], v[5], v[6], v[7]));
       }
-      continue;
-    }
-    for (int c = lane; c < G; c += 32 * U) {
-      uint4 xv[U], pv[U];
-      F8 v[U];
+    } else {
+      for (int c = lane; c < G; c += 32 * U) {
+        uint4 xv[U], pv[U];
+        F8 v[U];
 #pragma unroll
-      for (int k = 0; k < U; ++k)
-        if (c + 32 * k < G) {
-          xv[k] = __ldg(xr + c + 32 * k);
-          pv[k] = __ldg(pr + c + 32 * k);
-          v[k] = ldg8(s + 8 * (c + 32 * k));
-        }
+        for (int k = 0; k < U; ++k)
+          if (c + 32 * k < G) {
+            xv[k] = __ldg(xr + c + 32 * k);
+            pv[k] = __ldg(pr + c + 32 * k);
+            v[k] = ldg8(s + 8 * (c + 32 * k));
+          }
 #pragma unroll
-      for (int k = 0; k < U; ++k)
-        if (c + 32 * k < G) {
-          float xf[8], pf[8];
-          bf16x8_to_f32(xv[k], xf);
-          bf16x8_to_f32(pv[k], pf);
+        for (int k = 0; k < U; ++k)
+          if (c + 32 * k < G) {
+            float xf[8], pf[8];
+            bf16x8_to_f32(xv[k], xf);
+            bf16x8_to_f32(pv[k], pf);
 #pragma unroll
-          for (int u = 0; u < 8; ++u) v[k].v[u] = __fadd_rn(xf[u], __fsub_rn(v[k].v[u], pf[u]));
-          stcs8(o + 8 * (c + 32 * k), v[k]);
-        }
+            for (int u = 0; u < 8; ++u) v[k].v[u] = __fadd_rn(xf[u], __fsub_rn(v[k].v[u], pf[u]));
+            stcs8(o + 8 * (c + 32 * k), v[k]);
+          }
+      }
     }
   }
 }
@@ -1463,6 +1463,10 @@ cudaError_t launch_pack(const void* x, const uint8_t* labels, const int32_t* row
   return launch_pdl(pack_kernel, rows, dim3(PACK_THREADS), 0, st, xs, labels, row_src, counts, cu_img, ps, B, H, W, d, cap);
 }
 
+// CTAs per SM on the unpacks' grids: more than are resident, so that the hardware deals
+// them as others end (128x128, delta: 60.8 us with 8, 59.9 with 32; small grids alike).
+constexpr int UNPACK_CTAS = 32;
+
 // 32-byte accesses on fp32 rows: a row is a multiple of 512 bytes, so the arrays'
 // addresses decide.
 static bool wide(const float* a, const float* b) {
@@ -1472,7 +1476,7 @@ static bool wide(const float* a, const float* b) {
 cudaError_t launch_unpack(const float* out_img, const int32_t* tok_row, float* y, long long ntok,
                           int d, long long rows_max, int num_sms, cudaStream_t st) {
   auto* kern = wide(out_img, y) ? unpack_kernel<true> : unpack_kernel<false>;
-  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, 8)), dim3(256), 0, st, out_img,
+  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, UNPACK_CTAS)), dim3(256), 0, st, out_img,
                     tok_row, y, ntok, d, rows_max);
 }
 
@@ -1488,7 +1492,7 @@ cudaError_t launch_unpack_delta(const float* out_img, const void* packed, const 
                                 const uint8_t* labels, const int32_t* tok_row, float* y, long long ntok,
                                 int d, long long rows_max, int num_sms, cudaStream_t st) {
   auto* kern = wide(out_img, y) ? unpack_delta_kernel<true> : unpack_delta_kernel<false>;
-  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, 8)), dim3(256), 0, st, out_img,
+  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, UNPACK_CTAS)), dim3(256), 0, st, out_img,
                     static_cast<const __nv_bfloat16*>(packed), static_cast<const __nv_bfloat16*>(x), labels,
                     tok_row, y, ntok, d, rows_max);
 }
@@ -1497,7 +1501,7 @@ cudaError_t launch_unpack_update(const float* out_img, const int32_t* tok_row, v
                                  long long ntok, int d, float alpha, long long rows_max, int num_sms,
                                  cudaStream_t st) {
   auto* kern = wide(out_img, out_img) ? unpack_update_kernel<true> : unpack_update_kernel<false>;
-  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, 8)), dim3(256), 0, st,
+  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, UNPACK_CTAS)), dim3(256), 0, st,
                     out_img, tok_row, static_cast<__nv_bfloat16*>(x), ntok, d, alpha, rows_max);
 }
 
