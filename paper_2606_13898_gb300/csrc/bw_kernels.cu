@@ -690,42 +690,53 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_compact_kernel(
 // us, 27.3 so; four of 64x64 32.4 and 28.7; 64x64 9.5 and 8.9).
 
 constexpr int PACK_WARPS_PER_ROW = 4;
-constexpr int PACK_THREADS = 32 * PACK_WARPS_PER_ROW;  // of pack_kernel: a row per CTA
+constexpr int PACK_THREADS = 32 * PACK_WARPS_PER_ROW;  // a row, or a slice of a window row, per CTA
 
-// A low-frequency row: the mean of all LF x LF members of the window whose
-// first member is w0 (raster order, the first initialising the sum), one
-// correctly rounded division; this lane's 8-channel chunks c0, c0 + cstep, ...
+// CTAs per low-frequency row: a slice of 128 chunks of eight channels each, but the
+// rows of 2x2 windows, of which there are many, whole (128x128, d = 3072: 26.4 us whole
+// and 30.1 in slices; 4x4 windows 27.6 and 23.5, 8x8 62.7 and 23.8).
+__host__ __device__ constexpr int lf_slices(int lf, int d) {
+  return lf == 2 ? 1 : (d / 8 + PACK_THREADS - 1) / PACK_THREADS;
+}
+
+// (volatile: a batch's loads stay together)
+__device__ __forceinline__ uint4 ldg16(const uint4* p) {
+  uint4 r;
+  asm volatile("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+  return r;
+}
+
+// Eight channels (c) of a low-frequency row: the mean of all LF x LF members of the
+// window whose first member is w0 (raster order, the first initialising the sum), one
+// correctly rounded division.
 template <int LF>
-__device__ __forceinline__ void pack_lf_row(const __nv_bfloat16* __restrict__ w0, int W, int d, int c0, int G,
-                                            int cstep, uint4* __restrict__ dst) {
-  constexpr int NM = LF * LF;
+__device__ __forceinline__ void pack_lf_chunk(const __nv_bfloat16* __restrict__ w0, int W, int d, int c,
+                                              uint4* __restrict__ dst) {
+  constexpr int NM = LF * LF, LOADS = NM < 16 ? NM : 16;
   const float cnt = static_cast<float>(NM);
+  float acc[8];
 #pragma unroll 1
-  for (int c = c0; c < G; c += cstep) {
-    float acc[8];
-#pragma unroll 1
-    for (int g = 0; g < NM; g += 4) {
-      uint4 v[4];
+  for (int g = 0; g < NM; g += LOADS) {
+    uint4 v[LOADS];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int m = g + q;
-        v[q] = __ldg(reinterpret_cast<const uint4*>(w0 + static_cast<long long>((m / LF) * W + (m % LF)) * d) + c);
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float f[8];
-        bf16x8_to_f32(v[q], f);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) acc[u] = (g == 0 && q == 0) ? f[u] : __fadd_rn(acc[u], f[u]);
-      }
+    for (int q = 0; q < LOADS; ++q) {
+      const int m = g + q;
+      v[q] = ldg16(reinterpret_cast<const uint4*>(w0 + static_cast<long long>((m / LF) * W + (m % LF)) * d) + c);
     }
-    uint4 o;
-    o.x = pack_bf16x2(__fdiv_rn(acc[0], cnt), __fdiv_rn(acc[1], cnt));
-    o.y = pack_bf16x2(__fdiv_rn(acc[2], cnt), __fdiv_rn(acc[3], cnt));
-    o.z = pack_bf16x2(__fdiv_rn(acc[4], cnt), __fdiv_rn(acc[5], cnt));
-    o.w = pack_bf16x2(__fdiv_rn(acc[6], cnt), __fdiv_rn(acc[7], cnt));
-    dst[c] = o;
+#pragma unroll
+    for (int q = 0; q < LOADS; ++q) {
+      float f[8];
+      bf16x8_to_f32(v[q], f);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc[u] = (g == 0 && q == 0) ? f[u] : __fadd_rn(acc[u], f[u]);
+    }
   }
+  uint4 o;
+  o.x = pack_bf16x2(__fdiv_rn(acc[0], cnt), __fdiv_rn(acc[1], cnt));
+  o.y = pack_bf16x2(__fdiv_rn(acc[2], cnt), __fdiv_rn(acc[3], cnt));
+  o.z = pack_bf16x2(__fdiv_rn(acc[4], cnt), __fdiv_rn(acc[5], cnt));
+  o.w = pack_bf16x2(__fdiv_rn(acc[6], cnt), __fdiv_rn(acc[7], cnt));
+  dst[c] = o;
 }
 
 __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __nv_bfloat16* __restrict__ x,
@@ -818,43 +829,60 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __nv_bfloat16*
 }
 
 // Low-frequency mode: per image, the kept rows (copies) and then one row per
-// LF x LF window of the grid (the mean of all its members). Same row
-// assignment as pack_kernel: four warps per packed row.
+// LF x LF window of the grid (the mean of all its members). The window rows come
+// first, in slices of 128 chunks of eight channels where they are few and long, with
+// 16 of a lane's loads in flight; then a CTA per row copies the kept ones. Bound by
+// the chain of a window's loads and sums. (With four loads in flight and a lane's
+// chunks one after another, 64x64 tokens of 3072 channels took 17.2 us for 4x4
+// windows, 7.5 so, and 51 for 8x8, 12.3.)
 template <int LF>
-__global__ void __launch_bounds__(256) pack_lf_kernel(const __nv_bfloat16* __restrict__ x,
-                                                      const int32_t* __restrict__ row_src,
-                                                      const int32_t* __restrict__ counts,
-                                                      const int32_t* __restrict__ cu_img,
-                                                      __nv_bfloat16* __restrict__ packed, int B, int H, int W,
-                                                      int d, int cap) {
+__global__ void __launch_bounds__(PACK_THREADS) pack_lf_kernel(const __nv_bfloat16* __restrict__ x,
+                                                               const int32_t* __restrict__ row_src,
+                                                               const int32_t* __restrict__ counts,
+                                                               const int32_t* __restrict__ cu_img,
+                                                               __nv_bfloat16* __restrict__ packed, int B, int H,
+                                                               int W, int d, int cap) {
   pdl_wait();
   pdl_trigger();
-  const int lane = threadIdx.x & 31;
   const int N = H * W;
   const int G = d >> 3;
   const int total = min(cu_img[B], cap);
-  const long long nwarps = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
-  constexpr int CSTEP = 32 * PACK_WARPS_PER_ROW;
-  for (long long gw = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-       gw < static_cast<long long>(total) * PACK_WARPS_PER_ROW; gw += nwarps) {
-    const int r = static_cast<int>(gw / PACK_WARPS_PER_ROW);
-    const int c0 = lane + 32 * static_cast<int>(gw % PACK_WARPS_PER_ROW);
-    int b = 0;
-    while (b + 1 < B && cu_img[b + 1] <= r) ++b;
-    const int local = r - cu_img[b];
+  const int slices = lf_slices(LF, d);
+  const int nw = (H / LF) * (W / LF);  // window rows of an image
+  const long long nwin = static_cast<long long>(B) * nw * slices;
+  for (long long i = blockIdx.x; i < nwin + total; i += gridDim.x) {
+    int b = 0, r;
+    int c = threadIdx.x;
+    const bool window = i < nwin;
+    if (window) {
+      const int w = static_cast<int>(i / slices);
+      c += static_cast<int>(i - static_cast<long long>(w) * slices) * PACK_THREADS;
+      b = w / nw;
+      r = cu_img[b] + counts[3 * b] + (w - b * nw);
+      if (r >= total) continue;
+    } else {
+      r = static_cast<int>(i - nwin);
+      while (b + 1 < B && cu_img[b + 1] <= r) ++b;
+      if (r - cu_img[b] >= counts[3 * b]) continue;
+    }
     const int src = row_src[r];
     const __nv_bfloat16* xb = x + static_cast<long long>(b) * N * d;
     uint4* dst = reinterpret_cast<uint4*>(packed + static_cast<long long>(r) * d);
-    const int size = local < counts[3 * b] ? 1 : LF;
-    if (!HILO_DCHECK(local >= 0 && src >= 0 && src < (H / size) * (W / size), DCHECK_PACK_LF_SRC)) continue;
-    if (local < counts[3 * b]) {
+    const int size = window ? LF : 1;
+    if (!HILO_DCHECK(r >= cu_img[b] && src >= 0 && src < (H / size) * (W / size), DCHECK_PACK_LF_SRC)) continue;
+    if (window) {
+      const int t0 = (LF * (src / (W / LF))) * W + LF * (src % (W / LF));
+      const __nv_bfloat16* w0 = xb + static_cast<long long>(t0) * d;
+      if constexpr (LF == 2) {  // not in slices
+        for (; c < G; c += PACK_THREADS) pack_lf_chunk<LF>(w0, W, d, c, dst);
+      } else {
+        if (c < G) pack_lf_chunk<LF>(w0, W, d, c, dst);
+      }
+    } else {
       const uint4* sp = reinterpret_cast<const uint4*>(xb + static_cast<long long>(src) * d);
-#pragma unroll 4
-      for (int c = c0; c < G; c += CSTEP) dst[c] = __ldg(sp + c);
-      continue;
+#pragma unroll 3
+      for (; c < G; c += PACK_THREADS) dst[c] = __ldg(sp + c);
     }
-    const int t0 = (LF * (src / (W / LF))) * W + LF * (src % (W / LF));
-    pack_lf_row<LF>(xb + static_cast<long long>(t0) * d, W, d, c0, G, CSTEP, dst);
   }
 }
 
@@ -1444,22 +1472,27 @@ cudaError_t launch_split(const float* score, const uint8_t* mask, const int32_t*
                     row_src, tok_row, H, W, levels, lf);
 }
 
+// CTAs per SM on pack_kernel's grid: a row per CTA and turn. The hardware deals further
+// CTAs as others end, which evens out rows of one to sixteen members, but one without a
+// row still costs its launch, and the capacity is several times the rows: 24 per SM
+// from about 5000 rows of capacity on, else 16 (4096 rows of 2048 channels: 5.1 us with
+// 16, 6.2 with 24; 16384 of 3072 with two levels 28.6 and 26.4; 5120 rows 10.4 and 10.2).
+static int pack_ctas(long long items, int num_sms) { return items <= 32LL * num_sms ? 16 : 24; }
+
 cudaError_t launch_pack(const void* x, const uint8_t* labels, const int32_t* row_src,
                         const int32_t* counts, const int32_t* cu_img, void* packed, int B, int H,
                         int W, int d, int cap, int lf, int num_sms, cudaStream_t st) {
-  const dim3 grid(grid_for(static_cast<long long>(cap) * PACK_WARPS_PER_ROW, 8, num_sms, 8));
   const auto* xs = static_cast<const __nv_bfloat16*>(x);
   auto* ps = static_cast<__nv_bfloat16*>(packed);
-  if (lf == 2) return launch_pdl(pack_lf_kernel<2>, grid, dim3(256), 0, st, xs, row_src, counts, cu_img, ps, B, H, W, d, cap);
-  if (lf == 4) return launch_pdl(pack_lf_kernel<4>, grid, dim3(256), 0, st, xs, row_src, counts, cu_img, ps, B, H, W, d, cap);
-  if (lf == 8) return launch_pdl(pack_lf_kernel<8>, grid, dim3(256), 0, st, xs, row_src, counts, cu_img, ps, B, H, W, d, cap);
+  if (lf == 2 || lf == 4 || lf == 8) {
+    auto* kern = lf == 2 ? pack_lf_kernel<2> : lf == 4 ? pack_lf_kernel<4> : pack_lf_kernel<8>;
+    const long long items = cap + static_cast<long long>(B) * (H / lf) * (W / lf) * lf_slices(lf, d);
+    // (24 per SM at every size: 8x8 windows of 64x64 tokens 12.3 us, 12.7 with 16)
+    return launch_pdl(kern, dim3(grid_for(items, 1, num_sms, 24)), dim3(PACK_THREADS), 0, st, xs, row_src, counts, cu_img,
+                      ps, B, H, W, d, cap);
+  }
   if (lf) return cudaErrorInvalidValue;
-  // A row per CTA and turn. The hardware deals further CTAs as others end, which evens
-  // out rows of one to sixteen members, but one without a row still costs its launch,
-  // and the capacity is several times the rows: 24 per SM from about 5000 rows of
-  // capacity on, else 16 (4096 rows of 2048 channels: 5.1 us with 16, 6.2 with 24; 16384
-  // of 3072 with two levels 28.6 and 26.4; 5120 rows 10.4 and 10.2).
-  const dim3 rows(grid_for(cap, 1, num_sms, cap <= 32 * num_sms ? 16 : 24));
+  const dim3 rows(grid_for(cap, 1, num_sms, pack_ctas(cap, num_sms)));
   return launch_pdl(pack_kernel, rows, dim3(PACK_THREADS), 0, st, xs, labels, row_src, counts, cu_img, ps, B, H, W, d, cap);
 }
 

@@ -2,7 +2,7 @@
 path: the score where a thread takes one more group of channels; the split at
 the sizes where a thread's number of tokens doubles, for one image, clusters of
 images (2, 5, 8) and more than a cluster (9), in each mode and on arrays that
-allow no wide load; the three unpools on fp32 arrays that allow 32-byte accesses
+allow no wide load; low-frequency rows in one and several slices; the three unpools on fp32 arrays that allow 32-byte accesses
 and that do not; e4m3 rows at the ends of the widths that stay in registers;
 LayerNorm rows below, at and above one pass of the resident groups; attention
 over images of different length, with more query tiles than SMs, and more images
@@ -66,6 +66,28 @@ def test_split_at_tokens_per_thread(H, Hh, W, B, mode):
     ref = (O.split(s, mask, kk, km, Hh, W, levels, lf=lf) if lf else
            O.split(s, mask, kk, km, Hh, W, levels, granular=mode == "regions2"))
     check_split(sp, ref, B, N)
+
+
+@pytest.mark.parametrize("B", [1, 2])
+@pytest.mark.parametrize("lf,d", [(2, 1152), (4, 1024), (4, 1152), (8, 128), (8, 2176), (8, 4096)])
+def test_pack_low_frequency_slices(H, lf, d, B):
+    rng = np.random.default_rng(lf + d + B)
+    Hh, W = 16, 24
+    N = Hh * W
+    x = bits(rng.standard_normal((B, Hh, W, d)))
+    kk = rng.integers(0, N + 1, size=B).astype(np.int32)
+    ref = O.split(O.score(x), (rng.random((B, N)) < 0.1).astype(np.uint8), kk, kk, Hh, W, 1, lf=lf)
+    sh = H.Shape(B=B, H=Hh, W=W, d=d, lf=lf)
+    cap, rows = H.hilo_row_capacity(sh), int(ref.cu_img[-1])
+    sp = H.SplitBuffers.alloc(sh)
+    for name in ("labels", "counts", "cu_img", "tok_row"):
+        getattr(sp, name).copy_(torch.from_numpy(getattr(ref, name).reshape(-1)))
+    sp.row_src[:rows].copy_(torch.from_numpy(ref.row_src))
+    packed = torch.full((cap, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+    H.hilo_pack(sh, H.bf16_from_bits(x), sp, packed, cap)
+    H.hilo_sync_status()
+    assert np.array_equal(H.bits_from_bf16(packed[:rows]), O.pack(x, ref, lf))
+    assert torch.isnan(packed[rows:].float()).all()
 
 
 @pytest.mark.parametrize("off", [0, 4])  # floats past a 32-byte boundary: 32- and 16-byte accesses
