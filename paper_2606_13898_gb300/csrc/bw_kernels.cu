@@ -1131,7 +1131,7 @@ constexpr int LN_THREADS = LN_GROUP * LN_GROUPS;
 // Over one group: `red` is 4 floats of its own, used by no other reduction
 // until the group has met at two further barriers or ends its row.
 __device__ __forceinline__ void ln_group_sync() {
-  asm volatile("bar.sync %0, %1;" ::"r"(1 + static_cast<int>(threadIdx.x) / LN_GROUP), "n"(LN_GROUP) : "memory");
+  named_bar_sync(1 + static_cast<int>(threadIdx.x) / LN_GROUP, LN_GROUP);
 }
 
 __device__ __forceinline__ float ln_group_sum(float v, float* red) {

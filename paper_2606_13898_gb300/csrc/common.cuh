@@ -279,6 +279,34 @@ __device__ __forceinline__ void tmem_st_wait() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
+// --------------------------------------------------------------- barriers --
+// bar.* and barrier.cluster.*.aligned are for whole, converged warps, and code
+// that only some lanes ran (a store by lane 0, a guarded row) need not have
+// reconverged before them: every barrier here brings its warp together first,
+// which also orders those lanes' shared-memory accesses before the arrival.
+
+// Named barrier `id` (1..15) over `nthreads` threads (a multiple of 32).
+__device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
+  __syncwarp();
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
+// Named barrier over `nthreads` threads (a multiple of 32) that also returns
+// whether `pred` held for any of them.
+__device__ __forceinline__ bool bar_red_or(int id, int nthreads, bool pred) {
+  __syncwarp();
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, %2, %3, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(pred ? 1u : 0u), "r"(id), "r"(nthreads)
+      : "memory");
+  return r != 0;
+}
+
 // ------------------------------------------------- CTA pairs (2-SM MMA) --
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -288,6 +316,7 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
 }
 
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -300,9 +329,11 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
 
 // The two halves of a cluster barrier that orders nothing: all CTAs have come here.
 __device__ __forceinline__ void cluster_arrive_relaxed() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 

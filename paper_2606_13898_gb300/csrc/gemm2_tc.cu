@@ -502,6 +502,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
           for (int j = 0; j < 32; ++j) rc[j] = rn[j];
           if (c + 2 < tl.units)
             epi_load_resid(resid, resid_f32, r + 2 * UNIT, tl.rows - (r + 2 * UNIT), ch.feat, N, rn);
+          __syncwarp();  // a ragged chunk is loaded by some lanes only; the TMEM wait below is for all
         }
         ch.nvalid = min(UNIT, tl.rows - r);
         ch.row = tl.row_base + r;
