@@ -403,6 +403,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
+      // X comes after the previous kernel's end anyway; the limit of the waits
+      // below is for this kernel's own work
+      pdl_wait();
       while (ok && it.next(w)) {
         const uint32_t idesc = p.idesc | (static_cast<uint32_t>(pl.get(p, w).units * (UNIT / 8)) << 17);
         if (!mbar_wait_warp(&tempty[acc], acc_phase ^ 1u, abort_flag, err, DEV_TIMEOUT_GEMM + 256 * 2)) break;
