@@ -61,6 +61,7 @@
 // Every mbarrier wait is bounded (error latched, TMEM freed, CTA returns).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 
 #include "common.cuh"
@@ -120,6 +121,7 @@ struct Cfg {
   static constexpr int OFF_W = DATA_BYTES + 256;
   static constexpr int OFF_X = OFF_W + (PROP ? 8 * 2 * BKV * 4 : 0);
   static constexpr int SMEM_BYTES = OFF_X + static_cast<int>(sizeof(Shared)) + 1024;  // + alignment of the base
+  static_assert(SMEM_BYTES % 4 == 0, "the row offsets follow");
 };
 
 struct AttnParams {
@@ -193,17 +195,17 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return y;
 }
 
-// The images' packed-row offsets within the capacity: from shared memory, where
-// the kernel puts them when they fit (CU_SMEM), else from global memory.
-constexpr int CU_SMEM = 128;
+// The images' packed-row offsets within the capacity: in shared memory up to
+// CU_SMEM images (what is left of it beside the tiles), else in global memory.
+constexpr int CU_SMEM = 4096;
 struct Offsets {
   const int* s;
   const AttnParams& p;
-  __device__ __forceinline__ int operator()(int b) const {
-    return s ? s[b] : min(ld_l2(p.cu_img + b), p.cap);
-  }
+  __device__ __forceinline__ int operator()(int b) const { return s ? s[b] : min(p.cu_img[b], p.cap); }
   // packed rows of image b
   __device__ __forceinline__ int len(int b) const { return (*this)(b + 1) - (*this)(b); }
+  // query (and key) tiles of image b
+  __device__ __forceinline__ int tiles(int b) const { return p.qt_txt + (len(b) + BQ - 1) / BQ; }
 };
 
 // Row range of tile j of image b (text tiles first, then image tiles); used
@@ -220,60 +222,153 @@ __device__ __forceinline__ void seq_tile(const AttnParams& p, const Offsets& cu,
   }
 }
 
-// The flat query tiles (ordered by image, head, tile) are cut into one contiguous
-// range per CTA: first tile of CTA x of G, x in [0, G]. Where all images have the
-// same number of tiles, or there are no more tiles than CTAs, the ranges are
-// ceil(tiles / G) tiles long. Else they are of equal cost: a tile costs as many steps
-// as its image has key tiles, plus JOB_STEPS for its prologue and epilogue. (Cut by
-// count, the CTAs of the longest of four images of 18 to 25 tiles had 24% more steps
-// than the mean, and attention took 344 us instead of 303.)
-constexpr int JOB_STEPS = 2;
-__device__ long long range_start(const AttnParams& p, const Offsets& cu, long long x, long long G) {
-  auto image_tiles = [&](int b) -> long long { return p.qt_txt + (cu.len(b) + BQ - 1) / BQ; };
-  long long cost = 0, tiles = 0;
-  bool same = true;
-  const long long first = image_tiles(0);
-  for (int b = 0; b < p.B; ++b) {
-    const long long nq = image_tiles(b);
-    same = same && nq == first;
-    tiles += nq * p.heads;
-    cost += nq * p.heads * (nq + JOB_STEPS);
+// A place in the flat query tiles (ordered by image, head, tile): tile g, and an
+// image b at or before the tile's, whose tiles begin at `base`. (Fewer than 2^31
+// tiles: at most 2 R d / 64 over R rows, whose q, k and v alone take 6 R d bytes.)
+struct Cursor {
+  int g, base, b;
+};
+struct Range {
+  Cursor cur;
+  int end;
+};
+
+__device__ __forceinline__ int warp_incl_scan(int v) {
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int n = __shfl_up_sync(0xffffffffu, v, off);
+    if (lane_id() >= off) v += n;
   }
-  if (same || tiles <= G) return min(tiles, x * ((tiles + G - 1) / G));
-  long long want = (x * cost + G - 1) / G, g = 0;
-  for (int b = 0; b < p.B; ++b) {
-    const long long nq = image_tiles(b), c = nq + JOB_STEPS, all = nq * p.heads * c;
-    if (want < all) return g + (want + c - 1) / c;
-    want -= all;
-    g += nq * p.heads;
-  }
-  return g;
+  return v;
 }
 
-// The next job of the flat query-tile range [g, end) (tiles ordered by image,
-// head, tile): two tiles of one group form a pair, a lone tile at the edge of
-// the range or of its group is a split job.
-__device__ bool next_job(const AttnParams& p, const Offsets& cu, long long& g, long long end, Job& jb) {
-  if (g >= end) return false;
-  long long base = 0;
-  int b = 0, nq = 0, L = 0;
-  for (; b < p.B; ++b) {
-    L = cu.len(b);
-    nq = p.qt_txt + (L + BQ - 1) / BQ;
-    const long long cnt = static_cast<long long>(nq) * p.heads;
-    if (g < base + cnt) break;
-    base += cnt;
+// The flat query tiles are cut into one contiguous range per CTA: those of CTA x of
+// G, [cur.g, end). Where all images have the same number of tiles, or there are no
+// more tiles than CTAs, the ranges are ceil(tiles / G) tiles long. Else they are of
+// equal cost: a tile costs as many steps as its image has key tiles, plus JOB_STEPS
+// for its prologue and epilogue. (Cut by count, the CTAs of the longest of four
+// images of 18 to 25 tiles had 24% more steps than the mean, and attention took 344 us
+// instead of 303.)
+constexpr int JOB_STEPS = 2;
+__device__ __forceinline__ Range range_by_count(int tiles, int x, int G) {
+  const int per = (tiles + G - 1) / G, g = min(tiles, x * per);
+  return {{g, 0, 0}, min(tiles, g + per)};
+}
+
+// (By count also where the cost might not fit 31 bits: more tiles than a device
+// holds, unless single images have far more than 2^15 rows.)
+__device__ __forceinline__ bool cost_fits(int tiles, int most) {
+  return static_cast<float>(tiles) * static_cast<float>(most + JOB_STEPS) < 2.0e9f;
+}
+// The cost of what comes before CTA x: ceil(x cost / G).
+__device__ __forceinline__ int cost_before(int x, int cost, int G) {
+  return x * (cost / G) + (x * (cost % G) + G - 1) / G;
+}
+
+// A few images, one after another.
+__device__ __forceinline__ Range range_of_few(const AttnParams& p, const Offsets& cu, int x, int G) {
+  int tiles = 0, cost = 0, least = INT_MAX, most = 0;
+  for (int b = 0; b < p.B; ++b) {
+    const int nq = cu.tiles(b);
+    tiles += nq;
+    cost += nq * (nq + JOB_STEPS);
+    least = min(least, nq);
+    most = max(most, nq);
   }
-  if (b >= p.B) return false;
-  const uint32_t r = static_cast<uint32_t>(g - base);  // < nq * heads: row indices are int32
-  jb.b = b;
+  tiles *= p.heads;
+  if (least == most || tiles <= G || !cost_fits(tiles, most)) return range_by_count(tiles, x, G);
+  const int want0 = cost_before(x, cost * p.heads, G), want1 = cost_before(x + 1, cost * p.heads, G);
+  Range r = {{tiles, tiles, p.B}, tiles};
+  int t_before = 0, c_before = 0;
+  for (int b = 0; b < p.B; ++b) {
+    const int nq = cu.tiles(b), unit = nq + JOB_STEPS, c_after = c_before + nq * p.heads * unit;
+    // the first tile at or past what is wanted, in the first image that reaches beyond it
+    if (want0 >= c_before && want0 < c_after) r.cur = {t_before + (want0 - c_before + unit - 1) / unit, t_before, b};
+    if (want1 >= c_before && want1 < c_after) r.end = t_before + (want1 - c_before + unit - 1) / unit;
+    t_before += nq * p.heads;
+    c_before = c_after;
+  }
+  return r;
+}
+
+// Many images, by whole warps: a lane per image, 32 images at a time. (A call of its
+// own: inlined, its registers made the softmax spill.)
+constexpr int FEW_IMAGES = 8;
+__device__ __noinline__ Range range_of_many(const AttnParams& p, const Offsets& cu, int x, int G) {
+  const int lane = lane_id();
+  int tiles = 0, least = INT_MAX, most = 0;
+  uint32_t sum = 0;
+  for (int b = lane; b < p.B; b += 32) {
+    const int nq = cu.tiles(b);
+    tiles += nq * p.heads;
+    sum += static_cast<uint32_t>(nq * p.heads) * static_cast<uint32_t>(nq + JOB_STEPS);
+    least = min(least, nq);
+    most = max(most, nq);
+  }
+  tiles = __reduce_add_sync(0xffffffffu, tiles);
+  least = __reduce_min_sync(0xffffffffu, least);
+  most = __reduce_max_sync(0xffffffffu, most);
+  const int cost = static_cast<int>(__reduce_add_sync(0xffffffffu, sum));
+  Range r = range_by_count(tiles, x, G);
+  if (least == most) {
+    const int t = max(1, most * p.heads);
+    r.cur.b = min(r.cur.g / t, p.B);
+    r.cur.base = r.cur.b * t;
+    return r;
+  }
+  const bool by_count = tiles <= G || !cost_fits(tiles, most);
+  // the images in which the range begins and ends
+  const int want0 = by_count ? r.cur.g : cost_before(x, cost, G);
+  const int want1 = by_count ? r.end : cost_before(x + 1, cost, G);
+  r = {{tiles, tiles, p.B}, tiles};
+  int t_before = 0, c_before = 0;  // of the images before this group of 32
+  bool found = false;
+  for (int b0 = 0; b0 < p.B; b0 += 32) {
+    const int nq = b0 + lane < p.B ? cu.tiles(b0 + lane) : 0;
+    const int unit = by_count ? 1 : nq + JOB_STEPS, t = nq * p.heads, c = t * unit;
+    const int ti = warp_incl_scan(t), ci = warp_incl_scan(c);
+    auto find = [&](int want, Cursor& o) {
+      const uint32_t hit = __ballot_sync(0xffffffffu, want < c_before + ci);
+      if (hit == 0u) return false;
+      const int l = __ffs(hit) - 1;
+      const int g = t_before + ti - t + (want - (c_before + ci - c) + unit - 1) / unit;
+      o.b = b0 + l;
+      o.base = __shfl_sync(0xffffffffu, t_before + ti - t, l);
+      o.g = __shfl_sync(0xffffffffu, g, l);
+      return true;
+    };
+    if (!found) found = find(want0, r.cur);
+    Cursor e;
+    if (find(want1, e)) {
+      r.end = e.g;
+      break;
+    }
+    t_before += __shfl_sync(0xffffffffu, ti, 31);
+    c_before += __shfl_sync(0xffffffffu, ci, 31);
+  }
+  return r;
+}
+
+// The next job of the range up to `end`: two tiles of one group form a pair, a lone
+// tile at the edge of the range or of its group is a split job.
+__device__ bool next_job(const AttnParams& p, const Offsets& cu, Cursor& cur, int end, Job& jb) {
+  if (cur.g >= end) return false;
+  int nq = 0;
+  for (; cur.b < p.B; ++cur.b) {
+    nq = cu.tiles(cur.b);
+    const int cnt = nq * p.heads;
+    if (cur.g < cur.base + cnt) break;
+    cur.base += cnt;
+  }
+  if (cur.b >= p.B) return false;
+  const uint32_t r = static_cast<uint32_t>(cur.g - cur.base);
+  jb.b = cur.b;
   jb.h = static_cast<int>(r / static_cast<uint32_t>(nq));
   jb.j0 = static_cast<int>(r % static_cast<uint32_t>(nq));
   jb.nkv = nq;
-  jb.L = L;
-  const long long grp_end = base + static_cast<long long>(jb.h + 1) * nq;
-  jb.pair = (end < grp_end ? end : grp_end) - g >= 2;
-  g += jb.pair ? 2 : 1;
+  jb.L = cu.len(cur.b);
+  jb.pair = min(end, cur.base + (jb.h + 1) * nq) - cur.g >= 2;
+  cur.g += jb.pair ? 2 : 1;
   return true;
 }
 
@@ -287,27 +382,30 @@ template <int HD, bool PROP>
 __global__ void __launch_bounds__(ATTN_THREADS, 1)
     attn_kernel(const __grid_constant__ CUtensorMap tm, const __grid_constant__ AttnParams p) {
   using C = Cfg<HD, PROP>;
+  extern __shared__ unsigned char smem_raw[];
   // The row offsets were written before the previous kernel started: the
   // schedule, the barriers and tensor memory are ready when it ends.
-  __shared__ int cu_s[CU_SMEM + 1];
+  int* cu_s = reinterpret_cast<int*>(smem_raw + C::SMEM_BYTES);
   const bool in_smem = p.B <= CU_SMEM;
   if (in_smem) {
     for (int b = threadIdx.x; b <= p.B; b += ATTN_THREADS) cu_s[b] = min(ld_l2(p.cu_img + b), p.cap);
     __syncthreads();
+  } else {
+    pdl_wait();
   }
   const Offsets cu{in_smem ? cu_s : nullptr, p};
   // ---- this CTA's share of the query tiles of all (image, head) groups
-  const long long g_begin = range_start(p, cu, blockIdx.x, gridDim.x);
-  const long long g_end = range_start(p, cu, blockIdx.x + 1LL, gridDim.x);
-  long long g = g_begin;
+  const Range range = p.B <= FEW_IMAGES ? range_of_few(p, cu, blockIdx.x, gridDim.x)
+                                        : range_of_many(p, cu, blockIdx.x, gridDim.x);
+  Cursor cur = range.cur;
+  const int g_end = range.end;
   Job jb;
-  bool more = next_job(p, cu, g, g_end, jb);
+  bool more = next_job(p, cu, cur, g_end, jb);
   if (!more) {  // uniform across the CTA: nothing allocated yet
     pdl_wait();
     return;
   }
 
-  extern __shared__ unsigned char smem_raw[];
   // (an offset from smem_raw, so that accesses stay 32-bit shared-memory ones)
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::DATA_BYTES);
@@ -382,7 +480,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
       uint32_t kt = 0;
       uint64_t* full = kq ? k_full : v_full;
       uint64_t* empty = kq ? k_empty : v_empty;
-      for (uint32_t jn = 0; ok && more; ++jn, more = next_job(p, cu, g, g_end, jb)) {
+      for (uint32_t jn = 0; ok && more; ++jn, more = next_job(p, cu, cur, g_end, jb)) {
         if (kq) {
           // Q of this job once the previous job's MMAs are done with Q
           if (jn > 0 && !mbar_wait(q_empty, (jn - 1) & 1u, abort_flag, err, DEV_TIMEOUT_ATTN + 256 * 16)) {
@@ -489,7 +587,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
     };
     bool ok = true;
     uint32_t kt = 0, sc0 = 0, sc1 = 0;
-    for (uint32_t jn = 0; ok && more; ++jn, more = next_job(p, cu, g, g_end, jb)) {
+    for (uint32_t jn = 0; ok && more; ++jn, more = next_job(p, cu, cur, g_end, jb)) {
       const int n0 = job_steps(jb, 0), n1 = job_steps(jb, 1);
       const int qb1 = jb.pair ? 1 : 0;  // the Q buffer of warpgroup 1
       auto wait_k = [&](int t) {
@@ -592,7 +690,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1)
       // ---------------- warp 11, the softmax's job list: the next job is ready
       // when the present one's last barrier is met
       for (uint32_t jn = 1; more; ++jn) {
-        more = next_job(p, cu, g, g_end, jb);
+        more = next_job(p, cu, cur, g_end, jb);
         if (lane == 0) {
           shr.job[jn & 1u] = jb;
           shr.more[jn & 1u] = more;
@@ -945,7 +1043,7 @@ cudaError_t launch_hd(const AttnArgs& a, const AttnParams& p, int grid, cudaStre
   if (!encode_tmap_bf16_2d(&tm, a.qkv, 3ull * a.d, a.R, 3ull * a.d, 64, 128))
     return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(attn_kernel<HD, PROP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       Cfg<HD, PROP>::SMEM_BYTES);
+                                       Cfg<HD, PROP>::SMEM_BYTES + (CU_SMEM + 4) * 4);
   if (e != cudaSuccess) return e;
   // the register split must fit what the CTA is launched with, or the
   // softmax warpgroups' setmaxnreg.inc would wait for registers forever
@@ -958,8 +1056,9 @@ cudaError_t launch_hd(const AttnArgs& a, const AttnParams& p, int grid, cudaStre
   }
   if (static_cast<long long>(regs) * ATTN_THREADS < 256LL * SOFTMAX_REGS + 128LL * CONTROL_REGS)
     return cudaErrorInvalidConfiguration;
-  return launch_pdl(attn_kernel<HD, PROP>, dim3(grid), dim3(ATTN_THREADS), Cfg<HD, PROP>::SMEM_BYTES, st, tm,
-                    p);
+  const int offsets = p.B <= CU_SMEM ? (p.B + 1) * 4 : 0;
+  return launch_pdl(attn_kernel<HD, PROP>, dim3(grid), dim3(ATTN_THREADS), Cfg<HD, PROP>::SMEM_BYTES + offsets, st,
+                    tm, p);
 }
 
 }  // namespace
