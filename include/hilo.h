@@ -319,6 +319,13 @@ size_t hilo_block_workspace_bytes(const hilo_shape* shape, int32_t cap);
  * QKV / out-projection GEMM operands and attention inputs are bf16, the MLP
  * GEMM operands fp16 (saturating conversion), all with fp32 accumulation; the
  * residual stream stays fp32.
+ * Repeatability: with the same inputs and row counts a call gives the same
+ * bits every time, but for one case. Where d is a multiple of 256 and at least
+ * 1024 and the rows make more tiles of 256 rows x 256 channels than the device
+ * has SM pairs (text and image rows in tiles of their own), the second MLP
+ * product, and the out-projection of an in-place call, may sum a tile in
+ * pieces of K that meet in any order: `out` then varies in the last bits of
+ * its fp32 sums. The same holds for the other block entry points.
  */
 int hilo_block_forward(const hilo_shape* shape, const hilo_block_weights* weights,
                        const int32_t* cu_img, int32_t cap, const void* in_txt,

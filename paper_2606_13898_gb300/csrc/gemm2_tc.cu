@@ -119,14 +119,21 @@ struct Plan {
 
   // Chosen by cost: lane l tries image tiles of at most u1 = 8 - l % 8 units (and
   // text tiles of at most two more), whole or with the tiles left over after the last
-  // full round cut into 2 to 8 pieces, by rows or (fp32 += only) along K, of which
+  // full round cut into 2 to 8 pieces, by rows or (see below) along K, of which
   // lane l takes the counts 1 + l / 8 and 5 + l / 8; the cheapest wins, the higher
   // tile and the fewer pieces among equals. The cost is that of pair 0, which has the
   // most tiles: its rounds of whole tiles, its pieces, and the epilogue that nothing
   // hides. Called by whole warps. Every cycle here is one before the first product
   // wherever the previous kernel held the SM to its end.
+  //
+  // A K cut costs the call its bitwise repeatability: the pieces' partial sums meet
+  // in whatever order they come. So only calls of many tiles make one, as hilo.h
+  // says: widths that are a multiple of 256 from 1024 on, more tiles of 256 x 256
+  // than pairs, and the last round of those a partial one. (K cuts at fewer rows are
+  // faster: a block of 777 rows of 1024 channels took 60.4 us, 66.4 without; of 300 rows
+  // 46.8 and 54.6. Added up in order, through scratch and a counter per tile, they
+  // took 61 to 72 and 53.)
   __device__ void init(const Params& p, int dev0, int dev1, int ncl, int kb) {
-    const bool split = p.epilogue == EPI_BIAS_RESID_F32;
     const float EPI = p.epilogue == EPI_BIAS_RESIDIN_F32 ? EPI_RESID_CYC : EPI_CYC;
     // a device row count is bounded by the group's capacity (rows_static)
     rows0 = max(0, p.rows_dev[0] ? min(dev0, p.rows_static[0]) : p.rows_static[0]);
@@ -134,6 +141,8 @@ struct Plan {
     U0 = (rows0 + UNIT - 1) / UNIT;
     U1 = (rows1 + UNIT - 1) / UNIT;
     const int F = (p.N + PF - 1) / PF;
+    const int full = F * ((U0 + MAXU - 1) / MAXU + (U1 + MAXU - 1) / MAXU);  // tiles of 256 x 256
+    const bool split = p.epilogue == EPI_BIAS_RESID_F32 && p.N >= 1024 && p.N % PF == 0 && full > ncl && full % ncl != 0;
     const int lane = lane_id();
     const int u1 = MAXU - (lane & 7), u0 = min(MAXU, u1 + 2);
     const int a0 = (U0 + u0 - 1) / u0, a1 = (U1 + u1 - 1) / u1;

@@ -2,8 +2,8 @@
 
 Each result copied back to the host must equal y from HotPath.run on the
 same inputs, batch by batch, whatever the overlap of copies and kernels.
-The 32x32 layer (no stream-K accumulation) is deterministic, so y is
-compared bit for bit.
+The 32x32 layer has no GEMM that is cut along K and repeats itself exactly, so
+y is compared bit for bit.
 """
 import numpy as np
 import pytest
