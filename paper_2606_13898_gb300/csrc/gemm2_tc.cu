@@ -62,12 +62,15 @@ constexpr int THREADS = 32 * (2 + EPI_WARPS);
 constexpr uint32_t TMEM_COLS = 512;         // two 128 x 256 fp32 accumulators
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
 constexpr int SPLIT_MIN_KB = 16;            // shortest piece of a tile cut along K
-constexpr int SPLIT_MAX = 8;                // most pieces per tile
 // the plan's costs in SM cycles beside those of the k-blocks
 constexpr float TILE_CYC = 400.f;           // going from one tile to the next
 constexpr float EPI_CYC = 700.f;            // the last epilogue, per 32 rows
 constexpr float EPI_RESID_CYC = 1200.f;     // the same with a residual to load
-constexpr float PIECE_CYC = 300.f;          // a K piece's reductions, per 32 rows
+// where K is short (up to SHORT_K) and epilogues follow one another: a latency per tile
+constexpr int SHORT_K = 512;
+constexpr float SHORT_CYC = 2800.f;
+constexpr float SHORT_RESID_CYC = 3500.f;
+constexpr float PIECE_CYC = 300.f;           // a K piece's reductions, per 32 rows
 
 struct Maps {
   CUtensorMap x[4];  // boxes of 128, 64, 32, 16 rows
@@ -87,6 +90,10 @@ struct Params {
   void* out;
   const void* resid_src[2];
   int resid_f32;
+  // for the plan, by epilogue and K: cycles of 32 rows in the last epilogue; with short
+  // K the latency of an epilogue and its 32 rows, else 0 and 0; 0 with short K, else far
+  // more than any main loop takes
+  float epi_cyc, short_cyc, short_epi_cyc, long_k;
 };
 
 // One unit of a pair's work: k-blocks [k0, k1) of piece `part` of `parts` (cut by
@@ -123,8 +130,13 @@ struct Plan {
   // lane l takes the counts 1 + l / 8 and 5 + l / 8; the cheapest wins, the higher
   // tile and the fewer pieces among equals. The cost is that of pair 0, which has the
   // most tiles: its rounds of whole tiles, its pieces, and the epilogue that nothing
-  // hides. Called by whole warps. Every cycle here is one before the first product
-  // wherever the previous kernel held the SM to its end.
+  // hides. Up to K = 512 the epilogues take longer than the main loops: a round costs
+  // the longer of the two, and the epilogue has a latency of its own per tile. (Priced
+  // like longer K, short K was cut into many small pieces: at K = 128, 384 features of
+  // 2389 rows took 7.8 us, 5.8 so, of 4096 rows 7.2 and 6.1; at K = 512, 1536 features
+  // of 2389 rows 10.5 and 8.9. At 640 and 768 that price was 27% worse for some shapes
+  // and 11% better for others.) Called by whole warps. Every cycle here is one before
+  // the first product wherever the previous kernel held the SM to its end.
   //
   // A K cut costs the call its bitwise repeatability: the pieces' partial sums meet
   // in whatever order they come. So only calls of many tiles make one, as hilo.h
@@ -134,7 +146,7 @@ struct Plan {
   // 46.8 and 54.6. Added up in order, through scratch and a counter per tile, they
   // took 61 to 72 and 53.)
   __device__ void init(const Params& p, int dev0, int dev1, int ncl, int kb) {
-    const float EPI = p.epilogue == EPI_BIAS_RESIDIN_F32 ? EPI_RESID_CYC : EPI_CYC;
+    const float EPI = p.epi_cyc;
     // a device row count is bounded by the group's capacity (rows_static)
     rows0 = max(0, p.rows_dev[0] ? min(dev0, p.rows_static[0]) : p.rows_static[0]);
     rows1 = max(0, p.rows_dev[1] ? min(dev1, p.rows_static[1]) : p.rows_static[1]);
@@ -157,7 +169,10 @@ struct Plan {
     };
     const int least = min(least_of(U0, a0, x0), least_of(U1, a1, x1));
     const float kbf = static_cast<float>(kb);
-    const float c0 = kbf * kblock(x0) + TILE_CYC, c1 = kbf * kblock(x1) + TILE_CYC;
+    auto loop_of = [&](float x) { return kbf * kblock(x) + TILE_CYC; };
+    auto tile_of = [&](float x) { return fmaxf(loop_of(x), p.short_cyc + p.short_epi_cyc * x); };
+    auto tail_of = [&](float x) { return fminf(loop_of(x) + p.long_k, p.short_cyc + EPI * x); };
+    const float c0 = tile_of(x0), c1 = tile_of(x1);
     // ceil(n / ncl) for the small counts here (n + 0.5 keeps the product away
     // from the whole numbers)
     const float inv = __fdividef(1.0f, static_cast<float>(ncl));
@@ -168,7 +183,7 @@ struct Plan {
       return g0 * c0 + (n - g0) * c1;
     };
     const int rem = T > 0 && rounds * ncl != T ? T - (rounds - 1) * ncl : 0;  // of a partial last round
-    float best = rounds_cost(rounds) + EPI * xm;
+    float best = rounds_cost(rounds) + tail_of(xm);
     int best_s = 1, best_k = 0;
     const float c_full = rounds_cost(rounds - 1);
 #pragma unroll
@@ -177,7 +192,7 @@ struct Plan {
       if (s == 1 || rem == 0) continue;
       const float n = static_cast<float>(rounds_of(rem * s)), sf = static_cast<float>(s);
       const float xs = ceilf(__fdividef(xm, sf) - 1e-3f), ks = ceilf(__fdividef(kbf, sf) - 1e-3f);
-      const float cr = c_full + n * (kbf * kblock(xs) + TILE_CYC) + EPI * xs;
+      const float cr = c_full + n * tile_of(xs) + tail_of(xs);
       if (s <= least && cr < best) best = cr, best_s = s, best_k = 0;
       const float ck = c_full + n * (ks * kblock(xm) + TILE_CYC + PIECE_CYC * xm) + EPI * xm;
       if (split && kb >= s * SPLIT_MIN_KB && ck < best) best = ck, best_s = s, best_k = 1;
@@ -597,6 +612,11 @@ cudaError_t launch_gemm(const GemmArgs& a, int num_sms, cudaStream_t st) {
   p.epilogue = a.epilogue;
   p.out = a.out;
   p.resid_f32 = a.resid_f32;
+  const bool resid = a.epilogue == EPI_BIAS_RESIDIN_F32, short_k = a.K <= SHORT_K;
+  p.epi_cyc = resid ? EPI_RESID_CYC : EPI_CYC;
+  p.short_cyc = short_k ? (resid ? SHORT_RESID_CYC : SHORT_CYC) : 0.f;
+  p.short_epi_cyc = short_k ? p.epi_cyc : 0.f;
+  p.long_k = short_k ? 0.f : 1e30f;
   if (units <= 0) return cudaSuccess;
   auto* kern = a.fp8 ? gemm2_kernel<true> : gemm2_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
