@@ -24,10 +24,10 @@
 //                        keep kernel, 8.9 with channel planes and a root per
 //                        pixel; 2048x2048 20.2 and 24.1.
 //   sobel_keep_kernel    one CTA per 16 x 16 tokens: the mask tile and a halo
-//                        of R tokens in shared memory, the image maximum from
-//                        the tile slots; per token: any mask token within R
-//                        tokens (square window), or tokmax / imgmax (one
-//                        correctly rounded division) > threshold.
+//                        of R tokens as bits in shared memory, the image
+//                        maximum from the tile slots; per token: any mask
+//                        token within R tokens (square window), or tokmax /
+//                        imgmax (one correctly rounded division) > threshold.
 // Order of the magnitude, per channel c (P the replicate-padded pixels):
 //   gx = ((P(y-1,x+1) + 2 P(y,x+1)) + P(y+1,x+1)) - ((P(y-1,x-1) + 2 P(y,x-1)) + P(y+1,x-1))
 //   gy = ((P(y+1,x-1) + 2 P(y+1,x)) + P(y+1,x+1)) - ((P(y-1,x-1) + 2 P(y-1,x)) + P(y-1,x+1))
@@ -234,39 +234,74 @@ __global__ void __launch_bounds__(SOBEL_THREADS, C == 4 ? 4 : 5) sobel_tokmax_ke
   }
 }
 
-// One CTA per 16 x 16 tokens: the mask tile with a halo of `radius` tokens in shared
-// memory and each token's dilation window (radius <= MAX_RADIUS), then the image
-// maximum from the tile slots and the token's normalised maximum. A chain of short
-// waits, no unit is busy. The mask was complete before the magnitude kernel, which
-// waits for its own predecessor, let this one start, so the dilation runs beside
-// that kernel, ahead of the wait.
+// One CTA per 16 x 16 tokens: the mask tile with a halo of `radius` tokens as bits, the
+// tokens' dilation windows (radius <= MAX_RADIUS) from them, then the image maximum from
+// the tile slots and the token's normalised maximum. A chain of short waits, no unit is
+// busy. The mask was complete before the magnitude kernel, which waits for its own
+// predecessor, let this one start, so the dilation runs beside that kernel, ahead of the
+// wait. A warp reads a row of the halo at a time; its first lanes find which of the 16
+// columns have a mask token within reach in that row, and a token looks at one such
+// word per row. (Every token walking its whole window of bytes here, selected by its
+// magnitude or not, took 991 us at 64x64 tokens of 16 pixels and radius 64, 13.5 so;
+// radius 16 74.6 and 7.6, radius 4 12.3 and 7.3, radius 1 6.9 and 7.0.)
 constexpr int KEEP_T = 16;
 constexpr int MAX_RADIUS = 64;
+constexpr int KEEP_WARPS = KEEP_T * KEEP_T / 32;
+constexpr int KEEP_WORDS = (KEEP_T + 2 * MAX_RADIUS + 31) / 32;  // of a row of the halo
 
+// Unused shared memory that spreads these CTAs over the SMs: without it many share one
+// SM, the next magnitude kernel's CTAs find the others fuller, and three images of 46x30
+// tokens, one selection after another, take 13.0 us instead of 10.2.
+constexpr int KEEP_SMEM = 20480;
+
+// WORDS: 32-bit words of a row of the halo (1 up to radius 8)
+template <int WORDS>
 __global__ void __launch_bounds__(KEEP_T * KEEP_T) sobel_keep_kernel(const float* __restrict__ tokmax,
                                                                    const uint32_t* __restrict__ tilemax,
                                                                    int ntiles, const uint8_t* __restrict__ mask,
                                                                    uint8_t* __restrict__ keep, int H, int W,
                                                                    int radius, float threshold) {
-  __shared__ uint8_t mt[KEEP_T + 2 * MAX_RADIUS][KEEP_T + 2 * MAX_RADIUS];
-  __shared__ uint32_t wred[KEEP_T * KEEP_T / 32];
+  __shared__ uint32_t near[KEEP_T + 2 * MAX_RADIUS];  // bit c: a mask token within reach of column c
+  __shared__ uint32_t wred[KEEP_WARPS];
   const int b = blockIdx.z;
   const int i0 = blockIdx.y * KEEP_T - radius, j0 = blockIdx.x * KEEP_T - radius;
   const int S = KEEP_T + 2 * radius;
+  const int lane = threadIdx.x & 31;
   const uint8_t* mb = mask + static_cast<long long>(b) * H * W;
-  for (int e = threadIdx.x; e < S * S; e += blockDim.x) {
-    const int ii = i0 + e / S, jj = j0 + e % S;
-    mt[e / S][e % S] = (ii >= 0 && ii < H && jj >= 0 && jj < W) ? __ldcg(mb + ii * W + jj) : 0;
+  // four rows of each warp at a time, all their loads in flight
+  for (int r0 = threadIdx.x >> 5; r0 < S; r0 += 4 * KEEP_WARPS) {
+    uint32_t v[4][WORDS];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = r0 + q * KEEP_WARPS, ii = i0 + r;
+#pragma unroll
+      for (int w = 0; w < WORDS; ++w) {
+        const int c = 32 * w + lane, jj = j0 + c;
+        v[q][w] = 0u;
+        if (r < S && c < S && ii >= 0 && ii < H && jj >= 0 && jj < W) v[q][w] = __ldcg(mb + ii * W + jj);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      bool any = false;  // column `lane` reaches the bits lane .. lane + 2 radius of the row
+#pragma unroll
+      for (int w = 0; w < WORDS; ++w) {
+        if (w > 0 && 32 * w >= S) break;
+        const uint32_t m = __ballot_sync(0xffffffffu, v[q][w] != 0u);
+        const int lo = lane - 32 * w, hi = lane + 2 * radius - 32 * w;
+        if (hi >= 0) any |= (m & (0xffffffffu << max(lo, 0)) & (0xffffffffu >> (31 - min(hi, 31)))) != 0u;
+      }
+      const uint32_t cols = __ballot_sync(0xffffffffu, any && lane < KEEP_T);
+      const int r = r0 + q * KEEP_WARPS;
+      if (lane == 0 && r < S) near[r] = cols;
+    }
   }
   __syncthreads();
   const int ti = threadIdx.x / KEEP_T, tj = threadIdx.x % KEEP_T;
-  bool k = false;
-  for (int di = 0; di <= 2 * radius && !k; ++di)
-    for (int dj = 0; dj <= 2 * radius; ++dj)
-      if (mt[ti + di][tj + dj]) {
-        k = true;
-        break;
-      }
+  uint32_t reach = 0u;
+#pragma unroll 8
+  for (int di = 0; di <= 2 * radius; ++di) reach |= near[ti + di];
+  const bool k = (reach >> tj) & 1u;
   pdl_wait();
   pdl_trigger();
   uint32_t gm = 0u;
@@ -277,7 +312,7 @@ __global__ void __launch_bounds__(KEEP_T * KEEP_T) sobel_keep_kernel(const float
   __syncthreads();
   gm = wred[0];
 #pragma unroll
-  for (int w = 1; w < KEEP_T * KEEP_T / 32; ++w) gm = max(gm, wred[w]);
+  for (int w = 1; w < KEEP_WARPS; ++w) gm = max(gm, wred[w]);
   const int i = blockIdx.y * KEEP_T + ti, j = blockIdx.x * KEEP_T + tj;
   if (i >= H || j >= W) return;
   const long long t = (static_cast<long long>(b) * H + i) * W + j;
@@ -315,7 +350,8 @@ cudaError_t launch_sobel_select(const float* img, int B, int H, int W, int C, in
 #undef HILO_SOBEL_CASE
   if (e != cudaSuccess) return e;
   const dim3 kgrid((W + KEEP_T - 1) / KEEP_T, (H + KEEP_T - 1) / KEEP_T, B);
-  return launch_pdl(sobel_keep_kernel, kgrid, dim3(KEEP_T * KEEP_T), 0, st, static_cast<const float*>(tokmax),
+  auto* keep_kernel = KEEP_T + 2 * radius <= 32 ? sobel_keep_kernel<1> : sobel_keep_kernel<KEEP_WORDS>;
+  return launch_pdl(keep_kernel, kgrid, dim3(KEEP_T * KEEP_T), KEEP_SMEM, st, static_cast<const float*>(tokmax),
                     static_cast<const uint32_t*>(tilemax), sobel_tiles(H, W, patch), mask, keep, H, W, radius,
                     threshold);
 }
