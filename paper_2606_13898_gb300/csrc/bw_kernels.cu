@@ -972,7 +972,7 @@ __device__ __forceinline__ void copy_row(const float* __restrict__ s, float* __r
   }
 }
 
-template <bool WIDE>
+template <bool WIDE, int U>
 __global__ void __launch_bounds__(256) unpack_kernel(const float* __restrict__ out_img,
                                                      const int32_t* __restrict__ tok_row,
                                                      float* __restrict__ y, long long ntok,
@@ -985,7 +985,7 @@ __global__ void __launch_bounds__(256) unpack_kernel(const float* __restrict__ o
        t < ntok; t += wstep) {
     const int r = __ldg(tok_row + t);
     if (!HILO_DCHECK(r >= 0 && r < rows_max, DCHECK_UNPACK_ROW)) continue;
-    copy_row<WIDE, 4>(out_img + static_cast<long long>(r) * d, y + t * d, d, lane);
+    copy_row<WIDE, U>(out_img + static_cast<long long>(r) * d, y + t * d, d, lane);
   }
 }
 
@@ -994,8 +994,8 @@ __global__ void __launch_bounds__(256) unpack_kernel(const float* __restrict__ o
 // subtract then one fp32 add (x and packed widened from bf16). Four CTAs per SM:
 // small grids need the warps (46x30 tokens of 1152 channels, batch of three: 9.2 us
 // with 94 registers and three pieces in flight).
-template <bool WIDE>
-__global__ void __launch_bounds__(256, WIDE ? 4 : 0) unpack_delta_kernel(const float* __restrict__ out_img,
+template <bool WIDE, int U>
+__global__ void __launch_bounds__(256, WIDE && U > 1 ? 4 : 0) unpack_delta_kernel(const float* __restrict__ out_img,
                                                               const __nv_bfloat16* __restrict__ packed,
                                                               const __nv_bfloat16* __restrict__ x,
                                                               const uint8_t* __restrict__ labels,
@@ -1004,7 +1004,6 @@ __global__ void __launch_bounds__(256, WIDE ? 4 : 0) unpack_delta_kernel(const f
                                                               long long rows_max) {
   pdl_wait();
   pdl_trigger();
-  constexpr int U = 2;
   const int lane = threadIdx.x & 31;
   const int G = d >> 3;
   const long long wstep = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
@@ -1060,7 +1059,7 @@ __global__ void __launch_bounds__(256, WIDE ? 4 : 0) unpack_delta_kernel(const f
   }
 }
 
-template <bool WIDE>
+template <bool WIDE, int U>
 __global__ void __launch_bounds__(256) unpack_update_kernel(const float* __restrict__ out_img,
                                                             const int32_t* __restrict__ tok_row,
                                                             __nv_bfloat16* __restrict__ x,
@@ -1068,7 +1067,6 @@ __global__ void __launch_bounds__(256) unpack_update_kernel(const float* __restr
                                                             long long rows_max) {
   pdl_wait();
   pdl_trigger();
-  constexpr int U = 2;
   const int lane = threadIdx.x & 31;
   const int G = d >> 3;
   const long long wstep = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
@@ -1497,19 +1495,28 @@ cudaError_t launch_pack(const void* x, const uint8_t* labels, const int32_t* row
 }
 
 // CTAs per SM on the unpacks' grids: more than are resident, so that the hardware deals
-// them as others end (128x128, delta: 60.8 us with 8, 59.9 with 32; small grids alike).
-constexpr int UNPACK_CTAS = 32;
+// them as others end (128x128 of 3072 channels, delta: 60.8 us with 8, 59.9 with 32;
+// small grids alike). Rows of up to 256 channels are one piece per lane: no batches, so
+// as many warps as the registers allow, and with little to do per token a grid of what
+// is resident (128x128 of 128 channels, buffers not in L2: nearest 5.5 us, 4.0 so, delta
+// 6.8 and 5.8, update 5.1 and 4.2; of 256 channels 6.3 and 5.4, 8.2 and 7.5, 5.6 and 5.1).
+constexpr int UNPACK_CTAS = 32, UNPACK_CTAS_SHORT = 8;
+static bool short_row(int d) { return d <= 256; }
+static dim3 unpack_grid(long long ntok, int d, int num_sms) {
+  return dim3(grid_for(ntok, 8, num_sms, short_row(d) ? UNPACK_CTAS_SHORT : UNPACK_CTAS));
+}
 
-// 32-byte accesses on fp32 rows: a row is a multiple of 512 bytes, so the arrays'
-// addresses decide.
-static bool wide(const float* a, const float* b) {
-  return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 31) == 0;
+// 32-byte accesses on fp32 rows, where a row keeps a whole warp busy with them: it is a
+// multiple of 512 bytes, so beyond that the arrays' addresses decide.
+static bool wide(const float* a, const float* b, int d) {
+  return d >= 256 && ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 31) == 0;
 }
 
 cudaError_t launch_unpack(const float* out_img, const int32_t* tok_row, float* y, long long ntok,
                           int d, long long rows_max, int num_sms, cudaStream_t st) {
-  auto* kern = wide(out_img, y) ? unpack_kernel<true> : unpack_kernel<false>;
-  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, UNPACK_CTAS)), dim3(256), 0, st, out_img,
+  const bool w = wide(out_img, y, d), one = short_row(d);
+  auto* kern = w ? (one ? unpack_kernel<true, 1> : unpack_kernel<true, 4>) : (one ? unpack_kernel<false, 1> : unpack_kernel<false, 4>);
+  return launch_pdl(kern, unpack_grid(ntok, d, num_sms), dim3(256), 0, st, out_img,
                     tok_row, y, ntok, d, rows_max);
 }
 
@@ -1524,8 +1531,9 @@ cudaError_t launch_row_sizes(const uint8_t* labels, const int32_t* row_src, cons
 cudaError_t launch_unpack_delta(const float* out_img, const void* packed, const void* x,
                                 const uint8_t* labels, const int32_t* tok_row, float* y, long long ntok,
                                 int d, long long rows_max, int num_sms, cudaStream_t st) {
-  auto* kern = wide(out_img, y) ? unpack_delta_kernel<true> : unpack_delta_kernel<false>;
-  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, UNPACK_CTAS)), dim3(256), 0, st, out_img,
+  const bool w = wide(out_img, y, d), one = short_row(d);
+  auto* kern = w ? (one ? unpack_delta_kernel<true, 1> : unpack_delta_kernel<true, 2>) : (one ? unpack_delta_kernel<false, 1> : unpack_delta_kernel<false, 2>);
+  return launch_pdl(kern, unpack_grid(ntok, d, num_sms), dim3(256), 0, st, out_img,
                     static_cast<const __nv_bfloat16*>(packed), static_cast<const __nv_bfloat16*>(x), labels,
                     tok_row, y, ntok, d, rows_max);
 }
@@ -1533,8 +1541,9 @@ cudaError_t launch_unpack_delta(const float* out_img, const void* packed, const 
 cudaError_t launch_unpack_update(const float* out_img, const int32_t* tok_row, void* x,
                                  long long ntok, int d, float alpha, long long rows_max, int num_sms,
                                  cudaStream_t st) {
-  auto* kern = wide(out_img, out_img) ? unpack_update_kernel<true> : unpack_update_kernel<false>;
-  return launch_pdl(kern, dim3(grid_for(ntok, 8, num_sms, UNPACK_CTAS)), dim3(256), 0, st,
+  const bool w = wide(out_img, out_img, d), one = short_row(d);
+  auto* kern = w ? (one ? unpack_update_kernel<true, 1> : unpack_update_kernel<true, 2>) : (one ? unpack_update_kernel<false, 1> : unpack_update_kernel<false, 2>);
+  return launch_pdl(kern, unpack_grid(ntok, d, num_sms), dim3(256), 0, st,
                     out_img, tok_row, static_cast<__nv_bfloat16*>(x), ntok, d, alpha, rows_max);
 }
 

@@ -90,11 +90,9 @@ def test_pack_low_frequency_slices(H, lf, d, B):
     assert torch.isnan(packed[rows:].float()).all()
 
 
-@pytest.mark.parametrize("off", [0, 4])  # floats past a 32-byte boundary: 32- and 16-byte accesses
-@pytest.mark.parametrize("d", [128, 384, 3072, 4096])
-def test_unpack_at_both_alignments(H, d, off):
+def check_unpacks(H, B, Hh, W, d, off):
+    """The three unpools on fp32 arrays `off` floats past a 32-byte boundary."""
     rng = np.random.default_rng(d + off)
-    B, Hh, W = 2, 8, 12
     N = Hh * W
     x = bits(rng.standard_normal((B, Hh, W, d)))
     ref = O.split(O.score(x), (rng.random((B, N)) < 0.1).astype(np.uint8), np.array([N // 4, 5], np.int32),
@@ -121,6 +119,18 @@ def test_unpack_at_both_alignments(H, d, off):
     H.hilo_unpack_update(sh, od, sp, xd, 0.035)
     H.hilo_sync_status()
     assert np.array_equal(H.bits_from_bf16(xd).reshape(x.shape), O.update(x, O.unpack(out, ref).reshape(x.shape), 0.035))
+
+
+@pytest.mark.parametrize("off", [0, 4])  # floats past a 32-byte boundary: 32- and 16-byte accesses
+@pytest.mark.parametrize("d", [128, 384, 3072, 4096])
+def test_unpack_at_both_alignments(H, d, off):
+    check_unpacks(H, 2, 8, 12, d, off)
+
+
+@pytest.mark.parametrize("off", [0, 4])
+@pytest.mark.parametrize("d", [128, 256])  # one piece per lane; more tokens than resident warps
+def test_unpack_of_short_rows(H, d, off):
+    check_unpacks(H, 2, 64, 132, d, off)
 
 
 @pytest.mark.parametrize("dtype,cols", [("bf16", 8), ("bf16", 4096), ("bf16", 4104), ("bf16", 12288),
