@@ -680,8 +680,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_compact_kernel(
 
 // =============================================================== pack =====
 //
-// Four warps per packed image row, each owning every fourth 8-channel chunk
-// of its lanes, so a row needs one memory round trip. A kept row is a
+// One to four warps per packed image row, each owning every first to fourth
+// 8-channel chunk of its lanes, so a row needs one memory round trip. A kept row is a
 // 16-byte-vector copy; a pooled row sums the window's members of its class
 // in raster order (the first member initialises the sum), divides once with
 // correct rounding and rounds to bf16 (nearest even). Bound by each row's chain of
@@ -689,8 +689,15 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_compact_kernel(
 // flight: a CTA per row, eight to an SM (two rows per CTA: 128x128 with two levels 31.2
 // us, 27.3 so; four of 64x64 32.4 and 28.7; 64x64 9.5 and 8.9).
 
-constexpr int PACK_WARPS_PER_ROW = 4;
-constexpr int PACK_THREADS = 32 * PACK_WARPS_PER_ROW;  // a row, or a slice of a window row, per CTA
+constexpr int PACK_WARPS = 4;
+constexpr int PACK_THREADS = 32 * PACK_WARPS;
+constexpr int PACK_THREADS_SHORT = 256;  // rows of up to 512 channels, several to a CTA
+
+// Warps per row (or slice of a window row): as many as have a chunk of eight channels per
+// lane. (A CTA of four warps per row at every width, of 128 channels a quarter kept and
+// the rest pooled 2x2: 64x64 tokens 3.7 us, 2.8 so, 128x128 9.1 and 4.0; low-frequency
+// rows of 2x2 windows, none kept, 64x64 4.3 and 2.4, of 512 channels 4.3 and 2.8.)
+static int pack_warps(int d) { return d <= 256 ? 1 : d <= 512 ? 2 : 4; }
 
 // CTAs per low-frequency row: a slice of 128 chunks of eight channels each, but the
 // rows of 2x2 windows, of which there are many, whole (128x128, d = 3072: 26.4 us whole
@@ -739,7 +746,11 @@ __device__ __forceinline__ void pack_lf_chunk(const __nv_bfloat16* __restrict__ 
   dst[c] = o;
 }
 
-__global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __nv_bfloat16* __restrict__ x,
+// CHUNKS: chunks of a kept row that a lane has in flight, no more than it has (three at
+// every width: 16 images of 32x32 tokens of 4096 channels, all kept, 45.8 us, 42.1 with
+// four; 128x128 of 1024 10.7, 9.9 with one; 3072 channels with four 39.2, 34.6 with three)
+template <int WPR, int THREADS, int CHUNKS>
+__global__ void __launch_bounds__(THREADS) pack_kernel(const __nv_bfloat16* __restrict__ x,
                                                    const uint8_t* __restrict__ labels,
                                                    const int32_t* __restrict__ row_src,
                                                    const int32_t* __restrict__ counts,
@@ -754,12 +765,12 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __nv_bfloat16*
   const int total = min(cu_img[B], cap);
   const long long nwarps = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
   for (long long gw = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-       gw < static_cast<long long>(total) * PACK_WARPS_PER_ROW; gw += nwarps) {
+       gw < static_cast<long long>(total) * WPR; gw += nwarps) {
     // from the last row down: an image's pooled rows, 4x4 last, take the longest
     // (128x128 with two levels 37.5 -> 35.6 us, 64x64 8.9 -> 8.1)
-    const int r = total - 1 - static_cast<int>(gw / PACK_WARPS_PER_ROW);
-    const int c0 = lane + 32 * static_cast<int>(gw % PACK_WARPS_PER_ROW);
-    constexpr int CSTEP = 32 * PACK_WARPS_PER_ROW;
+    const int r = total - 1 - static_cast<int>(gw / WPR);
+    const int c0 = lane + 32 * static_cast<int>(gw % WPR);
+    constexpr int CSTEP = 32 * WPR;
     int b = 0;
     while (b + 1 < B && cu_img[b + 1] <= r) ++b;
     const int local = r - cu_img[b];
@@ -772,7 +783,7 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __nv_bfloat16*
     if (!HILO_DCHECK(local >= 0 && src >= 0 && src < (H / size) * (W / size), DCHECK_PACK_SRC)) continue;
     if (local < nk) {
       const uint4* sp = reinterpret_cast<const uint4*>(xb + static_cast<long long>(src) * d);
-#pragma unroll 3
+#pragma unroll(CHUNKS)
       for (int c = c0; c < G; c += CSTEP) dst[c] = __ldg(sp + c);
       continue;
     }
@@ -829,14 +840,16 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __nv_bfloat16*
 }
 
 // Low-frequency mode: per image, the kept rows (copies) and then one row per
-// LF x LF window of the grid (the mean of all its members). The window rows come
-// first, in slices of 128 chunks of eight channels where they are few and long, with
-// 16 of a lane's loads in flight; then a CTA per row copies the kept ones. Bound by
-// the chain of a window's loads and sums. (With four loads in flight and a lane's
-// chunks one after another, 64x64 tokens of 3072 channels took 17.2 us for 4x4
-// windows, 7.5 so, and 51 for 8x8, 12.3.)
-template <int LF>
-__global__ void __launch_bounds__(PACK_THREADS) pack_lf_kernel(const __nv_bfloat16* __restrict__ x,
+// LF x LF window of the grid (the mean of all its members). Rows of 2x2 windows are many
+// and short: all rows in one go, from the last down. Larger windows first, in slices of
+// 128 chunks of eight channels, with 16 of a lane's loads in flight; then the kept rows.
+// Bound by the chain of a window's loads and sums. (With four loads in flight and a
+// lane's chunks one after another, 64x64 tokens of 3072 channels took 17.2 us for 4x4
+// windows, 7.5 so, and 51 for 8x8, 12.3. The 2x2 windows first, too: 4x 64x64 tokens of
+// 1152 channels 11.1 us, 10.1 so. 4x4 windows not first: 128x128 of 512, none kept, 5.4
+// and 4.2.)
+template <int LF, int WPR, int THREADS>
+__global__ void __launch_bounds__(THREADS) pack_lf_kernel(const __nv_bfloat16* __restrict__ x,
                                                                const int32_t* __restrict__ row_src,
                                                                const int32_t* __restrict__ counts,
                                                                const int32_t* __restrict__ cu_img,
@@ -849,21 +862,24 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_lf_kernel(const __nv_bfloat
   const int total = min(cu_img[B], cap);
   const int slices = lf_slices(LF, d);
   const int nw = (H / LF) * (W / LF);  // window rows of an image
-  const long long nwin = static_cast<long long>(B) * nw * slices;
-  for (long long i = blockIdx.x; i < nwin + total; i += gridDim.x) {
+  const long long nwin = LF > 2 ? static_cast<long long>(B) * nw * slices : 0;
+  constexpr int STEP = 32 * WPR, ROWS = THREADS / STEP;  // rows per CTA and turn, chunks of a row per turn
+  for (long long i = static_cast<long long>(blockIdx.x) * ROWS + threadIdx.x / STEP; i < nwin + total;
+       i += static_cast<long long>(gridDim.x) * ROWS) {
     int b = 0, r;
-    int c = threadIdx.x;
-    const bool window = i < nwin;
+    int c = threadIdx.x % STEP;
+    bool window = i < nwin;
     if (window) {
       const int w = static_cast<int>(i / slices);
-      c += static_cast<int>(i - static_cast<long long>(w) * slices) * PACK_THREADS;
+      c += static_cast<int>(i - static_cast<long long>(w) * slices) * STEP;
       b = w / nw;
       r = cu_img[b] + counts[3 * b] + (w - b * nw);
       if (r >= total) continue;
     } else {
-      r = static_cast<int>(i - nwin);
+      r = static_cast<int>(nwin + total - 1 - i);
       while (b + 1 < B && cu_img[b + 1] <= r) ++b;
-      if (r - cu_img[b] >= counts[3 * b]) continue;
+      window = r - cu_img[b] >= counts[3 * b];
+      if (LF > 2 && window) continue;
     }
     const int src = row_src[r];
     const __nv_bfloat16* xb = x + static_cast<long long>(b) * N * d;
@@ -874,14 +890,14 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_lf_kernel(const __nv_bfloat
       const int t0 = (LF * (src / (W / LF))) * W + LF * (src % (W / LF));
       const __nv_bfloat16* w0 = xb + static_cast<long long>(t0) * d;
       if constexpr (LF == 2) {  // not in slices
-        for (; c < G; c += PACK_THREADS) pack_lf_chunk<LF>(w0, W, d, c, dst);
+        for (; c < G; c += STEP) pack_lf_chunk<LF>(w0, W, d, c, dst);
       } else {
         if (c < G) pack_lf_chunk<LF>(w0, W, d, c, dst);
       }
     } else {
       const uint4* sp = reinterpret_cast<const uint4*>(xb + static_cast<long long>(src) * d);
 #pragma unroll 3
-      for (; c < G; c += PACK_THREADS) dst[c] = __ldg(sp + c);
+      for (; c < G; c += STEP) dst[c] = __ldg(sp + c);
     }
   }
 }
@@ -1482,16 +1498,34 @@ cudaError_t launch_pack(const void* x, const uint8_t* labels, const int32_t* row
                         int W, int d, int cap, int lf, int num_sms, cudaStream_t st) {
   const auto* xs = static_cast<const __nv_bfloat16*>(x);
   auto* ps = static_cast<__nv_bfloat16*>(packed);
+  const int wpr = pack_warps(d);
+  const bool small = wpr < 4;
+  const int threads = small ? PACK_THREADS_SHORT : PACK_THREADS, rows = threads / (32 * wpr);  // rows per CTA and turn
   if (lf == 2 || lf == 4 || lf == 8) {
-    auto* kern = lf == 2 ? pack_lf_kernel<2> : lf == 4 ? pack_lf_kernel<4> : pack_lf_kernel<8>;
-    const long long items = cap + static_cast<long long>(B) * (H / lf) * (W / lf) * lf_slices(lf, d);
-    // (24 per SM at every size: 8x8 windows of 64x64 tokens 12.3 us, 12.7 with 16)
-    return launch_pdl(kern, dim3(grid_for(items, 1, num_sms, 24)), dim3(PACK_THREADS), 0, st, xs, row_src, counts, cu_img,
-                      ps, B, H, W, d, cap);
+    // rows of 8x8 windows: 64 loads per lane whatever the width, so one to a CTA
+    const bool few = small && lf < 8;
+    auto* kern = lf == 8   ? pack_lf_kernel<8, 4, PACK_THREADS>
+                 : lf == 4 ? (!few       ? pack_lf_kernel<4, 4, PACK_THREADS>
+                              : wpr == 1 ? pack_lf_kernel<4, 1, PACK_THREADS_SHORT>
+                                         : pack_lf_kernel<4, 2, PACK_THREADS_SHORT>)
+                           : (!few       ? pack_lf_kernel<2, 4, PACK_THREADS>
+                              : wpr == 1 ? pack_lf_kernel<2, 1, PACK_THREADS_SHORT>
+                                         : pack_lf_kernel<2, 2, PACK_THREADS_SHORT>);
+    const long long items = cap + (lf > 2 ? static_cast<long long>(B) * (H / lf) * (W / lf) * lf_slices(lf, d) : 0);
+    // (24 per SM at every size: 8x8 windows of 64x64 tokens of 3072 channels 12.3 us, 12.7 with 16)
+    const int ctas = few ? 8 : lf > 2 ? 24 : pack_ctas(cap, num_sms);
+    return launch_pdl(kern, dim3(grid_for(items, few ? rows : 1, num_sms, ctas)),
+                      dim3(few ? PACK_THREADS_SHORT : PACK_THREADS), 0, st, xs, row_src, counts, cu_img, ps, B, H, W, d,
+                      cap);
   }
   if (lf) return cudaErrorInvalidValue;
-  const dim3 rows(grid_for(cap, 1, num_sms, pack_ctas(cap, num_sms)));
-  return launch_pdl(pack_kernel, rows, dim3(PACK_THREADS), 0, st, xs, labels, row_src, counts, cu_img, ps, B, H, W, d, cap);
+  auto* kern = wpr == 1     ? pack_kernel<1, PACK_THREADS_SHORT, 1>
+               : wpr == 2   ? pack_kernel<2, PACK_THREADS_SHORT, 1>
+               : d <= 1024  ? pack_kernel<4, PACK_THREADS, 1>
+               : d <= 3072  ? pack_kernel<4, PACK_THREADS, 3>
+                            : pack_kernel<4, PACK_THREADS, 4>;
+  return launch_pdl(kern, dim3(grid_for(cap, rows, num_sms, small ? 8 : pack_ctas(cap, num_sms))), dim3(threads), 0, st,
+                    xs, labels, row_src, counts, cu_img, ps, B, H, W, d, cap);
 }
 
 // CTAs per SM on the unpacks' grids: more than are resident, so that the hardware deals

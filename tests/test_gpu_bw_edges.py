@@ -68,6 +68,34 @@ def test_split_at_tokens_per_thread(H, Hh, W, B, mode):
     check_split(sp, ref, B, N)
 
 
+@pytest.mark.parametrize("levels,lf", [(1, 0), (2, 0), (1, 2), (1, 4), (1, 8)])
+@pytest.mark.parametrize("d", [128, 256, 384, 512, 640, 1024, 1152, 3072, 3200])
+def test_pack_at_warps_per_row(H, d, levels, lf):
+    """Every number of warps per row, of rows per CTA and of chunks in flight, for rows
+    that are no multiple of a CTA's, and a capacity that ends within an image."""
+    rng = np.random.default_rng(d + levels + lf)
+    B, Hh, W = 3, 16, 24
+    N = Hh * W
+    x = bits(rng.standard_normal((B, Hh, W, d)))
+    kk = np.array([0, N // 3, N], np.int32)
+    mask = (rng.random((B, N)) < 0.02).astype(np.uint8)
+    ref = O.split(O.score(x), mask, kk, kk // 2, Hh, W, levels, **({"lf": lf} if lf else {}))
+    sh = H.Shape(B=B, H=Hh, W=W, d=d, levels=levels, lf=lf)
+    rows = int(ref.cu_img[-1])
+    sp = H.SplitBuffers.alloc(sh)
+    for name in ("labels", "counts", "cu_img", "tok_row"):
+        getattr(sp, name).copy_(torch.from_numpy(getattr(ref, name).reshape(-1)))
+    sp.row_src[:rows].copy_(torch.from_numpy(ref.row_src))
+    want = O.pack(x, ref, lf) if lf else O.pack(x, ref)
+    for cap in (rows + 3, rows - 7):
+        packed = torch.full((rows + 3, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+        H.hilo_pack(sh, H.bf16_from_bits(x), sp, packed, cap)
+        H.hilo_sync_status()
+        n = min(cap, rows)
+        assert np.array_equal(H.bits_from_bf16(packed[:n]), want[:n])
+        assert torch.isnan(packed[n:].float()).all()
+
+
 @pytest.mark.parametrize("B", [1, 2])
 @pytest.mark.parametrize("lf,d", [(2, 1152), (4, 1024), (4, 1152), (8, 128), (8, 2176), (8, 4096)])
 def test_pack_low_frequency_slices(H, lf, d, B):
