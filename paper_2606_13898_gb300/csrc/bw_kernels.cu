@@ -1295,7 +1295,11 @@ __global__ void __launch_bounds__(LN_THREADS, 2) layernorm_kernel(const void* __
 // way; longer or fp32 rows (NP = 0) are read a second time, from L1 / L2. (The block
 // of 2389 rows with e4m3 operands, which has two such passes, takes 6 us less than
 // with all rows read twice. 12288 elements are what a thread can hold with three CTAs
-// per SM: 80 registers.)
+// per SM: 80 registers. NP is the least that holds the row: with two pieces for all up to
+// 4096 elements and six above, 2400 rows of 5120 took 7.5 us, 5.7 so; 10000 of 512 11.7
+// and 8.7. The loops over fp32 rows are not unrolled, so that eight CTAs fit: 10000 rows
+// of 2048 19.4 us unrolled, 25.3 with at most 42 registers, 16.2 so; longer 16-bit rows
+// are, one row of 16384 3.3 us not unrolled and 2.3 so.)
 
 constexpr int QR_THREADS = 256;
 
@@ -1344,8 +1348,11 @@ __device__ __forceinline__ float quant_amax(float am, float* red) {
   return am;
 }
 
+// CTAs per SM
+__host__ __device__ constexpr int quant_ctas(int np) { return np == 6 ? 3 : np == 3 ? 5 : np == 2 ? 6 : 8; }
+
 template <int TYPE, int NP>
-__global__ void __launch_bounds__(QR_THREADS, NP == 6 ? 3 : 6)
+__global__ void __launch_bounds__(QR_THREADS, NP ? quant_ctas(NP) : TYPE == 2 ? 0 : 6)
     quant_rows_kernel(const void* __restrict__ src, int cols, int rows_static, const int32_t* __restrict__ cu_img,
                       int B, int n_txt, int cap, uint8_t* __restrict__ dst, float* __restrict__ scale) {
   constexpr bool REG = NP > 0;
@@ -1388,6 +1395,7 @@ __global__ void __launch_bounds__(QR_THREADS, NP == 6 ? 3 : 6)
         if (g < g8) reinterpret_cast<uint2*>(dst)[base8 + g] = quant8(f, inv);
       }
     } else {
+#pragma unroll(TYPE == 2 ? 1 : 4)
       for (int g = threadIdx.x; g < g8; g += QR_THREADS) {
         float f[8];
         load8(src, TYPE, base8 + g, f);
@@ -1396,6 +1404,7 @@ __global__ void __launch_bounds__(QR_THREADS, NP == 6 ? 3 : 6)
       }
       e4m3_row_scale(quant_amax(am, red[h]), inv, sc);
       // second pass: the row is in L1 / L2 from the first
+#pragma unroll(TYPE == 2 ? 1 : 4)
       for (int g = threadIdx.x; g < g8; g += QR_THREADS) {
         float f[8];
         load8(src, TYPE, base8 + g, f);
@@ -1586,12 +1595,13 @@ cudaError_t launch_quant_rows(const void* src, int type, int cols, int rows_stat
                               cudaStream_t st) {
   const long long rmax = cu_img ? static_cast<long long>(n_txt) + cap : rows_static;
   if (rmax <= 0) return cudaSuccess;
-  const int np = type == 2 || cols > 6 * 2048 ? 0 : (cols > 2 * 2048 ? 6 : 2);
-  auto* kern = type == 2 ? quant_rows_kernel<2, 0>
-               : type == 0
-                   ? (np == 2 ? quant_rows_kernel<0, 2> : np == 6 ? quant_rows_kernel<0, 6> : quant_rows_kernel<0, 0>)
-                   : (np == 2 ? quant_rows_kernel<1, 2> : np == 6 ? quant_rows_kernel<1, 6> : quant_rows_kernel<1, 0>);
-  return launch_pdl(kern, dim3(grid_for(rmax, 1, num_sms, np == 6 ? 3 : np == 2 ? 6 : 8)), dim3(QR_THREADS), 0, st,
+  const int np = type == 2 || cols > 6 * 2048 ? 0 : cols > 3 * 2048 ? 6 : (cols + 2047) / 2048;
+#define HILO_QUANT(T) \
+  (np == 1 ? quant_rows_kernel<T, 1> : np == 2 ? quant_rows_kernel<T, 2> : np == 3 ? quant_rows_kernel<T, 3> \
+   : np == 6 ? quant_rows_kernel<T, 6> : quant_rows_kernel<T, 0>)
+  auto* kern = type == 2 ? quant_rows_kernel<2, 0> : type == 0 ? HILO_QUANT(0) : HILO_QUANT(1);
+#undef HILO_QUANT
+  return launch_pdl(kern, dim3(grid_for(rmax, 1, num_sms, quant_ctas(np))), dim3(QR_THREADS), 0, st,
                     src, cols, rows_static, cu_img, B, n_txt, cap, dst, scale);
 }
 

@@ -187,6 +187,12 @@ def test_quantize_rows_at_register_widths(H, dtype, cols, rows):
     assert np.array_equal(sc.cpu().numpy(), sref)
 
 
+@pytest.mark.parametrize("dtype,cols", [("bf16", 2048), ("bf16", 2056), ("f16", 6144), ("f16", 6152), ("f32", 2048)])
+def test_quantize_rows_at_piece_counts(H, dtype, cols):
+    """One to two and three to six pieces of a row per thread, more rows than CTAs."""
+    test_quantize_rows_at_register_widths(H, dtype, cols, 1300)
+
+
 @pytest.mark.parametrize("f32", [0, 1])
 @pytest.mark.parametrize("rows", [1, 911, 1830])
 @pytest.mark.parametrize("d", [128, 640, 4096])
