@@ -1127,41 +1127,46 @@ __global__ void __launch_bounds__(256) unpack_update_kernel(const float* __restr
 
 // ========================================================== layernorm =====
 //
-// A row of the row space per group of 128 threads, three groups per CTA, two
-// CTAs per SM looping over the rows. Rows [0, n_txt) come from in_txt, rows
-// [n_txt, n_txt + cu_img[B]) from in_img (bf16 or fp32). Thread t of a group holds
-// elements 4t + 512k. Writes the normalised row (no affine, eps 1e-6, biased
-// variance) as bf16, fp16 or e4m3.
+// A row of the row space per group of 128 threads (64 up to 256 elements, a warp up to
+// 128), 384 threads per CTA, two CTAs per SM looping over the rows. Rows [0, n_txt) come
+// from in_txt, rows [n_txt, n_txt + cu_img[B]) from in_img (bf16 or fp32). Thread t of a
+// group of G holds elements 4t + 4G k. Writes the normalised row (no affine, eps 1e-6,
+// biased variance) as bf16, fp16 or e4m3.
 // Bound by memory latency: a row is one load round trip, two dependent
 // reductions and a store, so each group loads its next row before it reduces the
 // present one, and every row of a 2400-row block is asked for within two trips.
 // (One CTA per row took 6 us until the last had started: 2389 bf16 rows of 3072
-// elements 14.2 us, 5.7 so; fp32 rows 10 and 7; 10600 bf16 rows 45 and 25.)
+// elements 14.2 us, 5.7 so; fp32 rows 10 and 7; 10600 bf16 rows 45 and 25. 128 threads
+// for a row of 128 elements: 10000 rows 7.6 us, 2.8 so; of 256 7.0 and 5.3.)
 
-constexpr int LN_GROUP = 128;
-constexpr int LN_GROUPS = 3;
-constexpr int LN_THREADS = LN_GROUP * LN_GROUPS;
+constexpr int LN_THREADS = 384;
+constexpr int ln_group(int d) { return d <= 128 ? 32 : d <= 256 ? 64 : 128; }
 
 // Over one group: `red` is 4 floats of its own, used by no other reduction
 // until the group has met at two further barriers or ends its row.
+template <int GROUP>
 __device__ __forceinline__ void ln_group_sync() {
-  named_bar_sync(1 + static_cast<int>(threadIdx.x) / LN_GROUP, LN_GROUP);
+  named_bar_sync(1 + static_cast<int>(threadIdx.x) / GROUP, GROUP);
 }
 
+template <int GROUP>
 __device__ __forceinline__ float ln_group_sum(float v, float* red) {
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  if ((threadIdx.x & 31) == 0) red[(threadIdx.x >> 5) & 3] = v;
-  ln_group_sync();
-  return (red[0] + red[1]) + (red[2] + red[3]);
+  if (GROUP == 32) return v;
+  if ((threadIdx.x & 31) == 0) red[(threadIdx.x >> 5) % (GROUP / 32)] = v;
+  ln_group_sync<GROUP>();
+  return GROUP == 64 ? red[0] + red[1] : (red[0] + red[1]) + (red[2] + red[3]);
 }
 
+template <int GROUP>
 __device__ __forceinline__ float ln_group_max(float v, float* red) {
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
-  if ((threadIdx.x & 31) == 0) red[(threadIdx.x >> 5) & 3] = v;
-  ln_group_sync();
-  return fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
+  if (GROUP == 32) return v;
+  if ((threadIdx.x & 31) == 0) red[(threadIdx.x >> 5) % (GROUP / 32)] = v;
+  ln_group_sync<GROUP>();
+  return GROUP == 64 ? fmaxf(red[0], red[1]) : fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
 }
 
 // e4m3 row quantisation constants from the row's largest magnitude: inv =
@@ -1174,7 +1179,7 @@ __device__ __forceinline__ void e4m3_row_scale(float amax, float& inv, float& sc
 
 // ln_mode: 0 bf16, 1 fp16 (saturating), 2 e4m3 per row (ln_scale[r] = the
 // row's dequantisation scale)
-template <int NCH, bool F32>
+template <int NCH, bool F32, int GROUP>
 __global__ void __launch_bounds__(LN_THREADS, 2) layernorm_kernel(const void* __restrict__ in_txt,
                                                                   const void* __restrict__ in_img,
                                                                   void* __restrict__ ln, int ln_mode,
@@ -1183,11 +1188,12 @@ __global__ void __launch_bounds__(LN_THREADS, 2) layernorm_kernel(const void* __
                                                                   int n_txt, int cap, int d) {
   pdl_wait();
   pdl_trigger();
-  __shared__ float red_s[LN_GROUPS][3][4];
-  const int group = threadIdx.x / LN_GROUP, tid = threadIdx.x % LN_GROUP;
+  constexpr int GROUPS = LN_THREADS / GROUP;
+  __shared__ float red_s[GROUPS][3][4];
+  const int group = threadIdx.x / GROUP, tid = threadIdx.x % GROUP;
   float(*red)[4] = red_s[group];
   const int rows = n_txt + min(cu_img[B], cap);
-  const int step = gridDim.x * LN_GROUPS;
+  const int step = gridDim.x * GROUPS;
   const float inv_d = 1.0f / static_cast<float>(d);
   uint4 raw[NCH];  // the next row as it is in memory (bf16: .x and .y)
   auto load = [&](int r) {
@@ -1195,7 +1201,7 @@ __global__ void __launch_bounds__(LN_THREADS, 2) layernorm_kernel(const void* __
     const void* base = r < n_txt ? in_txt : in_img;
 #pragma unroll
     for (int t = 0; t < NCH; ++t) {
-      const int c = 512 * t + 4 * tid;
+      const int c = 4 * GROUP * t + 4 * tid;
       raw[t] = make_uint4(0u, 0u, 0u, 0u);
       if (c < d) {
         if (F32) {
@@ -1230,11 +1236,11 @@ __global__ void __launch_bounds__(LN_THREADS, 2) layernorm_kernel(const void* __
     float sum = 0.f;
 #pragma unroll
     for (int i = 0; i < NCH * 4; ++i) sum += v[i];
-    const float mean = ln_group_sum(sum, red[0]) * inv_d;
+    const float mean = ln_group_sum<GROUP>(sum, red[0]) * inv_d;
     float sq = 0.f;
 #pragma unroll
     for (int t = 0; t < NCH; ++t) {
-      if (512 * t + 4 * tid < d) {
+      if (4 * GROUP * t + 4 * tid < d) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float e = v[4 * t + i] - mean;
@@ -1242,21 +1248,21 @@ __global__ void __launch_bounds__(LN_THREADS, 2) layernorm_kernel(const void* __
         }
       }
     }
-    const float rstd = rsqrtf(ln_group_sum(sq, red[1]) * inv_d + 1e-6f);
+    const float rstd = rsqrtf(ln_group_sum<GROUP>(sq, red[1]) * inv_d + 1e-6f);
     if (ln_mode == 2) {
       float am = 0.f;
 #pragma unroll
       for (int t = 0; t < NCH; ++t)
-        if (512 * t + 4 * tid < d) {
+        if (4 * GROUP * t + 4 * tid < d) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) am = fmaxf(am, fabsf((v[4 * t + i] - mean) * rstd));
         }
       float inv, scale;
-      e4m3_row_scale(ln_group_max(am, red[2]), inv, scale);
+      e4m3_row_scale(ln_group_max<GROUP>(am, red[2]), inv, scale);
       uint8_t* q = static_cast<uint8_t*>(ln) + static_cast<long long>(r) * d;
 #pragma unroll
       for (int t = 0; t < NCH; ++t) {
-        const int c = 512 * t + 4 * tid;
+        const int c = 4 * GROUP * t + 4 * tid;
         if (c >= d) continue;
         *reinterpret_cast<uint32_t*>(q + c) =
             pack_e4m3x4(__fmul_rn((v[4 * t] - mean) * rstd, inv), __fmul_rn((v[4 * t + 1] - mean) * rstd, inv),
@@ -1268,7 +1274,7 @@ __global__ void __launch_bounds__(LN_THREADS, 2) layernorm_kernel(const void* __
     uint16_t* lo = static_cast<uint16_t*>(ln) + static_cast<long long>(r) * d;
 #pragma unroll
     for (int t = 0; t < NCH; ++t) {
-      const int c = 512 * t + 4 * tid;
+      const int c = 4 * GROUP * t + 4 * tid;
       if (c >= d) continue;
       const float y0 = (v[4 * t] - mean) * rstd, y1 = (v[4 * t + 1] - mean) * rstd;
       const float y2 = (v[4 * t + 2] - mean) * rstd, y3 = (v[4 * t + 3] - mean) * rstd;
@@ -1616,14 +1622,19 @@ cudaError_t launch_bf16_to_f16(const void* src, void* dst, long long n, int num_
 cudaError_t launch_layernorm(const void* in_txt, const void* in_img, int in_f32, void* ln, int ln_mode,
                              float* ln_scale, const int32_t* cu_img, int B, int n_txt, int cap, int d, int num_sms,
                              cudaStream_t st) {
-  const dim3 grid(grid_for(static_cast<long long>(n_txt) + cap, LN_GROUPS, num_sms, 2));
+  const int group = ln_group(d);
+  const dim3 grid(grid_for(static_cast<long long>(n_txt) + cap, LN_THREADS / group, num_sms, 2));
+#define HILO_LN(NC, G)                                                                                            \
+  (in_f32 ? launch_pdl(layernorm_kernel<NC, true, G>, grid, dim3(LN_THREADS), 0, st, in_txt, in_img, ln, ln_mode, \
+                       ln_scale, cu_img, B, n_txt, cap, d)                                                        \
+          : launch_pdl(layernorm_kernel<NC, false, G>, grid, dim3(LN_THREADS), 0, st, in_txt, in_img, ln, ln_mode, \
+                       ln_scale, cu_img, B, n_txt, cap, d))
+  if (group == 32) return HILO_LN(1, 32);
+  if (group == 64) return HILO_LN(1, 64);
   switch ((d + 511) / 512) {
-#define HILO_LN_CASE(NC)                                                                                     \
-  case NC:                                                                                                   \
-    return in_f32 ? launch_pdl(layernorm_kernel<NC, true>, grid, dim3(LN_THREADS), 0, st, in_txt, in_img, ln, \
-                               ln_mode, ln_scale, cu_img, B, n_txt, cap, d)                                  \
-                  : launch_pdl(layernorm_kernel<NC, false>, grid, dim3(LN_THREADS), 0, st, in_txt, in_img, ln, \
-                               ln_mode, ln_scale, cu_img, B, n_txt, cap, d);
+#define HILO_LN_CASE(NC) \
+  case NC:               \
+    return HILO_LN(NC, 128);
     HILO_LN_CASE(1)
     HILO_LN_CASE(2)
     HILO_LN_CASE(3)
@@ -1633,6 +1644,7 @@ cudaError_t launch_layernorm(const void* in_txt, const void* in_img, int in_f32,
     HILO_LN_CASE(7)
     HILO_LN_CASE(8)
 #undef HILO_LN_CASE
+#undef HILO_LN
     default:
       return cudaErrorInvalidValue;
   }

@@ -220,6 +220,12 @@ def test_layernorm_rows(H, d, rows, f32):
     assert np.all(np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 3e-4)
 
 
+@pytest.mark.parametrize("d,rows", [(128, 1), (128, 3647), (128, 3649), (256, 1825), (256, 5000), (384, 2000)])
+def test_layernorm_rows_of_narrow_groups(H, d, rows):
+    """A warp or 64 threads per row: 12 or 6 rows per CTA, below and above one pass."""
+    test_layernorm_rows(H, d, rows, rows % 2)
+
+
 @pytest.mark.parametrize("d,heads,T,lens", [
     (1024, 16, 64, [130, 900, 5, 0]),      # 240 query tiles of images 1 to 9 tiles long
     (1024, 8, 0, [257, 2050]),             # 160 tiles, hd 128, no text
