@@ -39,10 +39,12 @@ constexpr int SCORE_THREADS = 128;
 // the loads that the resident CTAs have in flight: with registers for four groups
 // whatever the width, 128x128 tokens of 3072 channels took 18.5 us, 16.8 so (6.0
 // TB/s), 64x64 6.8 and 6.3, 128x128 of 1024 10.8 and 8.8. Seven CTAs per SM for three
-// groups (6.7 us for 64x64 without the limit); for the others the compiler's own count
-// (128x128 of 4096: 21.5 us, 22.3 with five, 26.2 with a limit of one).
+// groups (6.7 us for 64x64 without the limit), eight for two (64x64 of 2048, in L2, 4.2
+// us without, 3.7 so, 3.9 with four groups' registers; 16 images of 1536 34.6 and 35.9);
+// for the others the compiler's own count (128x128 of 4096: 21.5 us, 22.3 with five, 26.2
+// with a limit of one).
 template <int ITERS>
-__global__ void __launch_bounds__(SCORE_THREADS, ITERS == 3 ? 7 : 0) score_kernel(const __nv_bfloat16* __restrict__ x,
+__global__ void __launch_bounds__(SCORE_THREADS, ITERS == 3 ? 7 : ITERS == 2 ? 8 : 0) score_kernel(const __nv_bfloat16* __restrict__ x,
                                                               float* __restrict__ s, int B, int H,
                                                               int W, int d) {
   pdl_wait();
