@@ -39,32 +39,27 @@ int cuda_fail(cudaError_t e, const char* where) {
 }
 
 struct DevInfo {
-  int num_sms = 0;
-  int major = 0, minor = 0;
+  int ordinal, num_sms;
 };
 
-// per-device cache (index = device ordinal)
-DevInfo g_dev[64];
-
-int current_device(DevInfo** out) {
+int current_device(DevInfo* out) {
+  static hilo::PerDevice known;  // SMs | minor << 16 | major << 24
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
-  if (dev < 0 || dev >= 64) return fail(HILO_ERR_UNSUPPORTED, "device ordinal %d", dev);
-  DevInfo& d = g_dev[dev];
-  if (d.num_sms == 0) {
-    e = cudaDeviceGetAttribute(&d.major, cudaDevAttrComputeCapabilityMajor, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.minor, cudaDevAttrComputeCapabilityMinor, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) {
-      d.num_sms = 0;
-      return cuda_fail(e, "cudaDeviceGetAttribute");
-    }
-  }
-  if (d.major != 10 || d.minor != 3)
-    return fail(HILO_ERR_UNSUPPORTED, "libhilo is built for sm_103a; device is sm_%d%d", d.major,
-                d.minor);
-  *out = &d;
+  if (dev < 0 || dev >= hilo::MAX_DEVICES) return fail(HILO_ERR_UNSUPPORTED, "device ordinal %d", dev);
+  const int v = known.get(dev, [&] {
+    int major = 0, minor = 0, sms = 0;
+    e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return e == cudaSuccess ? major << 24 | minor << 16 | sms : 0;
+  });
+  if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
+  const int major = v >> 24, minor = v >> 16 & 255;
+  if (major != 10 || minor != 3)
+    return fail(HILO_ERR_UNSUPPORTED, "libhilo is built for sm_103a; device is sm_%d%d", major, minor);
+  *out = {dev, v & 0xffff};
   return HILO_OK;
 }
 
@@ -159,7 +154,8 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
 // The driver's tensor-map encoder, resolved through the runtime so that the
 // library does not link libcuda (and loads on hosts without a driver).
 static EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
+  static std::atomic<EncodeTiledFn> known{nullptr};
+  EncodeTiledFn fn = known.load(std::memory_order_relaxed);
   if (!fn) {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -167,6 +163,7 @@ static EncodeTiledFn encode_fn() {
             cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
       fn = reinterpret_cast<EncodeTiledFn>(p);
+    known.store(fn, std::memory_order_relaxed);
   }
   return fn;
 }
@@ -258,9 +255,9 @@ int hilo_score(const hilo_shape* shape, const void* x, float* score, void* strea
   int st = check_shape(shape, false);
   if (st) return st;
   if (!x || !score) return fail(HILO_ERR_ARG, "hilo_score: NULL pointer");
-  DevInfo* dev;
+  DevInfo dev;
   if ((st = current_device(&dev))) return st;
-  cudaError_t e = hilo::launch_score(x, score, shape->B, shape->H, shape->W, shape->d, dev->num_sms,
+  cudaError_t e = hilo::launch_score(x, score, shape->B, shape->H, shape->W, shape->d, dev.num_sms,
                                      static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess) count(1);
   return e == cudaSuccess ? HILO_OK : cuda_fail(e, "hilo_score");
@@ -279,7 +276,7 @@ static int split_common(const char* name, const hilo_shape* shape, const float* 
   if ((st = check_split(out))) return st;
   if (!score || !mask || !k_keep) return fail(HILO_ERR_ARG, "%s: NULL pointer", name);
   if (shape->levels == 2 && !k_mid) return fail(HILO_ERR_ARG, "%s: k_mid is NULL with levels=2", name);
-  DevInfo* dev;
+  DevInfo dev;
   if ((st = current_device(&dev))) return st;
   cudaError_t e = hilo::launch_split(score, mask, k_keep, shape->levels == 2 ? k_mid : k_keep,
                                      out->labels, out->row_src, out->counts, out->cu_img,
@@ -329,10 +326,10 @@ int hilo_sobel_select(const hilo_shape* shape, const float* img, int channels, i
   const size_t need = hilo::sobel_workspace_bytes(shape->B, shape->H, shape->W);
   if (ws_bytes < need)
     return fail(HILO_ERR_WORKSPACE, "hilo_sobel_select: workspace %zu < %zu bytes", ws_bytes, need);
-  DevInfo* dev;
+  DevInfo dev;
   if ((st = current_device(&dev))) return st;
   cudaError_t e = hilo::launch_sobel_select(img, shape->B, shape->H, shape->W, channels, patch, mask, radius,
-                                            threshold, keep, ws, dev->num_sms, static_cast<cudaStream_t>(stream));
+                                            threshold, keep, ws, dev.num_sms, static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess) count(2);
   return e == cudaSuccess ? HILO_OK : cuda_fail(e, "hilo_sobel_select");
 }
@@ -344,11 +341,11 @@ int hilo_pack(const hilo_shape* shape, const void* x, const hilo_split_out* spli
   if ((st = check_split(split))) return st;
   if (!x || !packed) return fail(HILO_ERR_ARG, "hilo_pack: NULL pointer");
   if (cap < 0) return fail(HILO_ERR_ARG, "hilo_pack: cap=%d", cap);
-  DevInfo* dev;
+  DevInfo dev;
   if ((st = current_device(&dev))) return st;
   cudaError_t e = hilo::launch_pack(x, split->labels, split->row_src, split->counts, split->cu_img,
                                     packed, shape->B, shape->H, shape->W, shape->d, cap, shape->lf,
-                                    dev->num_sms, static_cast<cudaStream_t>(stream));
+                                    dev.num_sms, static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess) count(1);
   return e == cudaSuccess ? HILO_OK : cuda_fail(e, "hilo_pack");
 }
@@ -390,7 +387,7 @@ static int block_forward_impl(const hilo_shape* shape, const hilo_block_weights*
   const BlockWs L = block_ws_layout(shape, cap);
   if (!ws || ws_bytes < L.total)
     return fail(HILO_ERR_WORKSPACE, "hilo_block_forward: workspace %zu < %zu bytes", ws_bytes, L.total);
-  DevInfo* dev;
+  DevInfo dev;
   if ((st = current_device(&dev))) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int B = shape->B, T = shape->T, d = shape->d;
@@ -409,7 +406,7 @@ static int block_forward_impl(const hilo_shape* shape, const hilo_block_weights*
   // the residual is read from the input by the out-projection epilogue (no
   // fp32 copy of it is made) unless the input already is the output buffer
   cudaError_t e = hilo::launch_layernorm(in_txt, in_img, in_f32, ln, 0, nullptr, cu_img, B, BT, cap, d,
-                                         dev->num_sms, s);
+                                         dev.num_sms, s);
   if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward: layernorm 1");
   count(1);
   stage_mark(1, s);
@@ -431,7 +428,7 @@ static int block_forward_impl(const hilo_shape* shape, const hilo_block_weights*
     g.out = o;
     g.g[0] = {0, BT, nullptr, wt, bt, BT};
     g.g[1] = {BT, 0, cu_img + B, wi, bi, cap};
-    cudaError_t ge = hilo::launch_gemm(g, dev->num_sms, s);
+    cudaError_t ge = hilo::launch_gemm(g, dev.ordinal, dev.num_sms, s);
     if (ge == cudaSuccess) count(1);
     return ge;
   };
@@ -450,7 +447,7 @@ static int block_forward_impl(const hilo_shape* shape, const hilo_block_weights*
   aa.head_dim = d / shape->heads;
   aa.d = d;
   aa.R = R;
-  e = hilo::launch_attention(aa, dev->num_sms, s);
+  e = hilo::launch_attention(aa, dev.num_sms, s);
   if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward: attention");
   count(1);
   stage_mark(3, s);
@@ -460,7 +457,7 @@ static int block_forward_impl(const hilo_shape* shape, const hilo_block_weights*
   stage_mark(4, s);
   if (shape->mlp) {
     e = hilo::launch_layernorm(out, out + static_cast<size_t>(BT) * d, 1, ln, 1, nullptr, cu_img, B, BT,
-                               cap, d, dev->num_sms, s);
+                               cap, d, dev.num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward: layernorm 2");
     count(1);
     stage_mark(5, s);
@@ -501,13 +498,13 @@ int hilo_quantize_rows_e4m3(const void* src, int src_dtype, int64_t rows, int32_
                 static_cast<long long>(rows), cols);
   if ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15)
     return fail(HILO_ERR_ARG, "hilo_quantize_rows_e4m3: src and dst must be 16-byte aligned");
-  DevInfo* dev;
+  DevInfo dev;
   int st;
   if ((st = current_device(&dev))) return st;
   if (rows == 0 || cols == 0) return HILO_OK;
   const int type = src_dtype == HILO_BF16 ? 0 : (src_dtype == HILO_F16 ? 1 : 2);
   cudaError_t e = hilo::launch_quant_rows(src, type, cols, static_cast<int>(rows), nullptr, 0, 0, 0, dst, scale,
-                                          dev->num_sms, static_cast<cudaStream_t>(stream));
+                                          dev.num_sms, static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess) count(1);
   return e == cudaSuccess ? HILO_OK : cuda_fail(e, "hilo_quantize_rows_e4m3");
 }
@@ -551,7 +548,7 @@ static int block_forward_fp8_impl(const hilo_shape* shape, const hilo_block_weig
   const BlockWs8 L = block_fp8_ws_layout(shape, cap);
   if (!ws || ws_bytes < L.total)
     return fail(HILO_ERR_WORKSPACE, "hilo_block_forward_fp8: workspace %zu < %zu bytes", ws_bytes, L.total);
-  DevInfo* dev;
+  DevInfo dev;
   if ((st = current_device(&dev))) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int B = shape->B, T = shape->T, d = shape->d;
@@ -569,7 +566,7 @@ static int block_forward_fp8_impl(const hilo_shape* shape, const hilo_block_weig
 
   stage_mark(0, s);
   cudaError_t e = hilo::launch_layernorm(in_txt, in_img, in_f32, q8, 2, qs, cu_img, B, BT, cap, d,
-                                         dev->num_sms, s);
+                                         dev.num_sms, s);
   if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward_fp8: layernorm 1");
   count(1);
   stage_mark(1, s);
@@ -592,7 +589,7 @@ static int block_forward_fp8_impl(const hilo_shape* shape, const hilo_block_weig
     g.out = o;
     g.g[0] = {0, BT, nullptr, wt, bt, BT, st_};
     g.g[1] = {BT, 0, cu_img + B, wi, bi, cap, si};
-    cudaError_t ge = hilo::launch_gemm(g, dev->num_sms, s);
+    cudaError_t ge = hilo::launch_gemm(g, dev.ordinal, dev.num_sms, s);
     if (ge == cudaSuccess) count(1);
     return ge;
   };
@@ -611,10 +608,10 @@ static int block_forward_fp8_impl(const hilo_shape* shape, const hilo_block_weig
   aa.head_dim = d / shape->heads;
   aa.d = d;
   aa.R = R;
-  e = hilo::launch_attention(aa, dev->num_sms, s);
+  e = hilo::launch_attention(aa, dev.num_sms, s);
   if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward_fp8: attention");
   count(1);
-  e = hilo::launch_quant_rows(attn, 0, d, 0, cu_img, B, BT, cap, q8, qs, dev->num_sms, s);
+  e = hilo::launch_quant_rows(attn, 0, d, 0, cu_img, B, BT, cap, q8, qs, dev.num_sms, s);
   if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward_fp8: attention quantisation");
   count(1);
   stage_mark(3, s);
@@ -624,13 +621,13 @@ static int block_forward_fp8_impl(const hilo_shape* shape, const hilo_block_weig
   stage_mark(4, s);
   if (shape->mlp) {
     e = hilo::launch_layernorm(out, out + static_cast<size_t>(BT) * d, 1, q8, 2, qs, cu_img, B, BT, cap,
-                               d, dev->num_sms, s);
+                               d, dev.num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward_fp8: layernorm 2");
     count(1);
     stage_mark(5, s);
     e = gemm(4 * d, d, hilo::EPI_BIAS_GELU_F16, hid, wt.w_1, wt.s_1, wt.b_1, wi.w_1, wi.s_1, wi.b_1);
     if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward_fp8: mlp1 gemm");
-    e = hilo::launch_quant_rows(hid, 1, 4 * d, 0, cu_img, B, BT, cap, q8, qs, dev->num_sms, s);
+    e = hilo::launch_quant_rows(hid, 1, 4 * d, 0, cu_img, B, BT, cap, q8, qs, dev.num_sms, s);
     if (e != cudaSuccess) return cuda_fail(e, "hilo_block_forward_fp8: hidden quantisation");
     count(1);
     stage_mark(6, s);
@@ -665,10 +662,10 @@ int hilo_row_sizes(const hilo_shape* shape, const hilo_split_out* split, float* 
   if ((st = check_split(split))) return st;
   if (!n_img) return fail(HILO_ERR_ARG, "hilo_row_sizes: NULL pointer");
   if (cap < 0) return fail(HILO_ERR_ARG, "hilo_row_sizes: cap=%d", cap);
-  DevInfo* dev;
+  DevInfo dev;
   if ((st = current_device(&dev))) return st;
   cudaError_t e = hilo::launch_row_sizes(split->labels, split->row_src, split->counts, split->cu_img, n_img,
-                                         shape->B, shape->H, shape->W, cap, shape->lf, dev->num_sms,
+                                         shape->B, shape->H, shape->W, cap, shape->lf, dev.num_sms,
                                          static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess && cap > 0) count(1);
   return e == cudaSuccess ? HILO_OK : cuda_fail(e, "hilo_row_sizes");
@@ -680,11 +677,11 @@ int hilo_unpack(const hilo_shape* shape, const float* out_img, const hilo_split_
   if (st) return st;
   if ((st = check_split(split))) return st;
   if (!out_img || !y) return fail(HILO_ERR_ARG, "hilo_unpack: NULL pointer");
-  DevInfo* dev;
+  DevInfo dev;
   if ((st = current_device(&dev))) return st;
   const long long ntok = static_cast<long long>(shape->B) * shape->H * shape->W;
   const long long rows_max = static_cast<long long>(hilo_row_capacity(shape));
-  cudaError_t e = hilo::launch_unpack(out_img, split->tok_row, y, ntok, shape->d, rows_max, dev->num_sms,
+  cudaError_t e = hilo::launch_unpack(out_img, split->tok_row, y, ntok, shape->d, rows_max, dev.num_sms,
                                       static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess) count(1);
   return e == cudaSuccess ? HILO_OK : cuda_fail(e, "hilo_unpack");
@@ -699,12 +696,12 @@ int hilo_unpack_delta(const hilo_shape* shape, const float* out_img, const void*
   if ((reinterpret_cast<uintptr_t>(out_img) | reinterpret_cast<uintptr_t>(packed) |
        reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15)
     return fail(HILO_ERR_ARG, "hilo_unpack_delta: pointers must be 16-byte aligned");
-  DevInfo* dev;
+  DevInfo dev;
   if ((st = current_device(&dev))) return st;
   const long long ntok = static_cast<long long>(shape->B) * shape->H * shape->W;
   cudaError_t e = hilo::launch_unpack_delta(out_img, packed, x, split->labels, split->tok_row, y, ntok,
                                             shape->d, static_cast<long long>(hilo_row_capacity(shape)),
-                                            dev->num_sms, static_cast<cudaStream_t>(stream));
+                                            dev.num_sms, static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess) count(1);
   return e == cudaSuccess ? HILO_OK : cuda_fail(e, "hilo_unpack_delta");
 }
@@ -715,11 +712,11 @@ int hilo_unpack_update(const hilo_shape* shape, const float* out_img, const hilo
   if (st) return st;
   if ((st = check_split(split))) return st;
   if (!out_img || !x) return fail(HILO_ERR_ARG, "hilo_unpack_update: NULL pointer");
-  DevInfo* dev;
+  DevInfo dev;
   if ((st = current_device(&dev))) return st;
   const long long ntok = static_cast<long long>(shape->B) * shape->H * shape->W;
   cudaError_t e = hilo::launch_unpack_update(out_img, split->tok_row, x, ntok, shape->d, alpha,
-                                             static_cast<long long>(hilo_row_capacity(shape)), dev->num_sms,
+                                             static_cast<long long>(hilo_row_capacity(shape)), dev.num_sms,
                                              static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess) count(1);
   return e == cudaSuccess ? HILO_OK : cuda_fail(e, "hilo_unpack_update");
@@ -730,11 +727,11 @@ int hilo_convert_bf16_to_f16(const void* src, void* dst, size_t n, void* stream)
   if (n % 8) return fail(HILO_ERR_ARG, "hilo_convert_bf16_to_f16: n=%zu is not a multiple of 8", n);
   if ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15)
     return fail(HILO_ERR_ARG, "hilo_convert_bf16_to_f16: pointers must be 16-byte aligned");
-  DevInfo* dev;
+  DevInfo dev;
   int st;
   if ((st = current_device(&dev))) return st;
   if (n == 0) return HILO_OK;
-  cudaError_t e = hilo::launch_bf16_to_f16(src, dst, static_cast<long long>(n), dev->num_sms,
+  cudaError_t e = hilo::launch_bf16_to_f16(src, dst, static_cast<long long>(n), dev.num_sms,
                                            static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess) count(1);
   return e == cudaSuccess ? HILO_OK : cuda_fail(e, "hilo_convert_bf16_to_f16");

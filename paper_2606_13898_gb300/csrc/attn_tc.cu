@@ -1047,12 +1047,15 @@ cudaError_t launch_hd(const AttnArgs& a, const AttnParams& p, int grid, cudaStre
   if (e != cudaSuccess) return e;
   // the register split must fit what the CTA is launched with, or the
   // softmax warpgroups' setmaxnreg.inc would wait for registers forever
-  static int regs = -1;
-  if (regs < 0) {
+  // (one number for every device: the library holds one binary)
+  static std::atomic<int> known{0};
+  int regs = known.load(std::memory_order_relaxed);
+  if (regs == 0) {
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, attn_kernel<HD, PROP>);
     if (e != cudaSuccess) return e;
     regs = fa.numRegs;
+    known.store(regs, std::memory_order_relaxed);
   }
   if (static_cast<long long>(regs) * ATTN_THREADS < 256LL * SOFTMAX_REGS + 128LL * CONTROL_REGS)
     return cudaErrorInvalidConfiguration;

@@ -581,7 +581,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 
 }  // namespace
 
-cudaError_t launch_gemm(const GemmArgs& a, int num_sms, cudaStream_t st) {
+// CTA pairs of one kernel that the current device holds at a time.
+template <bool FP8>
+static int resident_pairs(int device, int num_sms) {
+  static PerDevice pairs;
+  const int n = pairs.get(device, [&] {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * (num_sms / 2), 1, 1);
+    cfg.blockDim = dim3(THREADS, 1, 1);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 2;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int found = 0;
+    if (cudaOccupancyMaxActiveClusters(&found, gemm2_kernel<FP8>, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      found = 0;
+    }
+    return found;
+  });
+  return n > 0 ? n : num_sms / 2;
+}
+
+cudaError_t launch_gemm(const GemmArgs& a, int device, int num_sms, cudaStream_t st) {
   // FP8: bytes are the elements, 128 per swizzled row
   const TmapType tt = a.fp8 ? TMAP_U8 : TMAP_BF16;
   const uint32_t bk = a.fp8 ? 128 : BK;
@@ -622,27 +648,8 @@ cudaError_t launch_gemm(const GemmArgs& a, int num_sms, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
   if (e != cudaSuccess) return e;
   // persistent grid: as many co-resident CTA pairs as the device holds
-  static int max_pairs = 0;
-  if (max_pairs == 0) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * (num_sms / 2), 1, 1);
-    cfg.blockDim = dim3(THREADS, 1, 1);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n <= 0) {
-      cudaGetLastError();
-      n = num_sms / 2;
-    }
-    max_pairs = n;
-  }
-  return launch_pdl(kern, dim3(2 * max_pairs), dim3(THREADS), SMEM_BYTES, st, m, p);
+  const int pairs = a.fp8 ? resident_pairs<true>(device, num_sms) : resident_pairs<false>(device, num_sms);
+  return launch_pdl(kern, dim3(2 * pairs), dim3(THREADS), SMEM_BYTES, st, m, p);
 }
 
 int gemm_take_device_error() {

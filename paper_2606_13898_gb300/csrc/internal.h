@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/hilo.h"
 
 #define HILO_LABEL_KEEP 0
@@ -14,6 +16,20 @@
 #define HILO_LABEL_LF 3
 
 namespace hilo {
+
+// ---- what the host code finds out once per device: a positive number, looked up by
+// the device's ordinal. Threads that are first at the same time find the same one.
+constexpr int MAX_DEVICES = 64;
+struct PerDevice {
+  std::atomic<int> value[MAX_DEVICES];
+  // find() <= 0: nothing to keep
+  template <typename Find>
+  int get(int device, Find find) {
+    int v = value[device].load(std::memory_order_relaxed);
+    if (v <= 0 && (v = find()) > 0) value[device].store(v, std::memory_order_relaxed);
+    return v;
+  }
+};
 
 // ---- bandwidth kernels (bw_kernels.cu)
 cudaError_t launch_score(const void* x, float* s, int B, int H, int W, int d, int num_sms,
@@ -90,7 +106,8 @@ struct GemmArgs {
   int resid_f32 = 0;
 };
 
-cudaError_t launch_gemm(const GemmArgs& a, int num_sms, cudaStream_t st);
+// device: the current device's ordinal, below MAX_DEVICES
+cudaError_t launch_gemm(const GemmArgs& a, int device, int num_sms, cudaStream_t st);
 int gemm_take_device_error();
 
 // ---- tcgen05 joint varlen attention (attn_tc.cu)
