@@ -4,9 +4,12 @@ Shape, SplitBuffers and DeviceWeights build their ctypes structs once per
 object. These checks run on the CPU (torch CPU tensors stand in for device
 buffers; no library call is made): the cached struct carries the tensors'
 current addresses, a replaced split tensor gives a rebuilt struct, and equal
-shapes stay equal and hash alike.
+shapes stay equal and hash alike. The current stream is found with and without
+torch's undocumented accessor.
 """
 import ctypes
+import importlib.util
+import types
 
 import torch
 
@@ -45,3 +48,21 @@ def test_weights_struct_carries_every_pointer():
             want = t[(s, f)].data_ptr() if t[(s, f)] is not None else None
             assert getattr(st, f) == want, (s, f)
     assert ctypes.sizeof(c) == 16 * ctypes.sizeof(ctypes.c_void_p)
+
+
+def test_current_stream_without_the_raw_accessor(monkeypatch):
+    def fresh():
+        spec = importlib.util.spec_from_file_location("paper_2606_13898_gb300.hilo_copy", H.__file__)
+        m = importlib.util.module_from_spec(spec)
+        monkeypatch.setitem(__import__("sys").modules, spec.name, m)  # dataclasses look their module up
+        spec.loader.exec_module(m)
+        return m
+
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda dev: 100 + dev, raising=False)
+    assert fresh()._stream(None) == 103
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    m = fresh()
+    assert m._stream(None) == 77
+    assert m._stream(5) == 5 and m._stream(types.SimpleNamespace(cuda_stream=9)) == 9
