@@ -28,7 +28,7 @@ def test_parity_tests_pass_on_checks_build():
     lib = build.build(variant="checks")
     env = dict(os.environ, HILO_LIBRARY=lib)
     cmd = [sys.executable, "-m", "pytest", "-q", "-x", "-m", "gpu", "-p", "no:cacheprovider",
-           "tests/test_gpu_kernels.py", "tests/test_gpu_regions.py", "tests/test_gpu_lf.py",
+           "tests/test_gpu_kernels.py", "tests/test_gpu_regions.py", "tests/test_gpu_lf.py", "tests/test_gpu_bw_edges.py",
            "-k", "(score or split or pack or unpack or row_sizes or regions or delta or lf) and not block"]
     r = subprocess.run(cmd, cwd=ROOT, env=env, capture_output=True, text=True, timeout=1800)
     assert r.returncode == 0, r.stdout[-4000:] + r.stderr[-2000:]

@@ -200,3 +200,68 @@ def test_block_forward_fp8_prop_against_oracle(H, d, heads, T, lens):
         assert 0.005 < e_ex < 0.1, e_ex
         # the weights are applied: the unweighted FP8 block is much further away
         assert np.linalg.norm(got - plain) / delta > 3 * e_emu
+
+
+@pytest.mark.parametrize("d,T,lens", [
+    (1024, 0, [1]),           # one row: a single one-unit tile
+    (1024, 33, [31]),         # a row above and a row below a 32-row unit
+    (1280, 1, [257, 95]),     # groups cut to different heights
+    (1280, 31, [1300]),       # several rounds of row passes and of tiles
+])
+def test_fp8_gemm_at_tile_edges(H, d, T, lens):
+    """Out-projection and row scales of an attention-only block, every row, as in the
+    isolated test above; rows past the used ones are not written."""
+    r = _run(H, d, d // 128, T, lens, 0, d + T)
+    sh, cap, rows = r["sh"], r["cap"], r["rows"]
+    BT = sh.B * sh.T
+    nr = BT + rows
+    q8, qs, qkv, att = _ws8(H, sh, cap, r["ws"])
+    codes, scale = O.quantize_rows(O.bf16_to_f32(H.bits_from_bf16(att[:nr])))
+    assert np.array_equal(q8[:nr].cpu().numpy(), codes)
+    assert np.array_equal(qs[:nr].cpu().numpy(), scale)
+    wq = O.quantize_weights(r["w"])
+    u = np.concatenate([O.bf16_to_f32(r["ut"]), O.bf16_to_f32(r["ui"])]).astype(np.float64)
+    dq = O.e4m3_decode(codes)
+    for lo, hi, s in ((0, BT, wq.txt), (BT, nr, wq.img)):
+        if hi == lo:
+            continue
+        cw, sw = s.w_o
+        ref = u[lo:hi] + (dq[lo:hi] @ O.e4m3_decode(cw).T) * scale[lo:hi, None].astype(np.float64) \
+            * sw[None, :].astype(np.float64) + O.bf16_to_f32(s.b_o)
+        assert np.max(np.abs(r["out"][lo:hi] - ref)) <= 1e-4 * (1 + np.max(np.abs(ref)))
+    for t in (q8, qkv.view(torch.uint8), att.view(torch.uint8)):  # the workspace's fill
+        assert bool((t[nr:] == 0xFF).all())
+
+
+@pytest.mark.parametrize("f32", [0, 1])
+@pytest.mark.parametrize("d,rows", [(1024, 1), (1280, 911), (1024, 1900)])
+def test_e4m3_layernorm_rows(H, d, rows, f32):
+    """LayerNorm rows as e4m3, seen through a QKV matrix whose every output picks one
+    input (a weight of 1 is code 448 with scale 1 / 448, and the products are exact up to
+    three fp32 roundings). A normalised value is within 3e-6 of the fp64 one, so its code
+    may differ by one step (2^-3 of the value, 2^-9 of the row's unit below the smallest
+    normal code), and only near a rounding boundary: in at most 1 of 1000 here."""
+    rng = np.random.default_rng(d + rows)
+    u = (rng.standard_normal((rows, d)) * 3 + 1).astype(np.float32)
+    if not f32:
+        u = bits(u)
+    pick = np.zeros((3 * d, d), np.float32)
+    pick[np.arange(3 * d), np.arange(3 * d) % d] = 1.0
+    sw = I.StreamWeights(w_qkv=bits(pick), b_qkv=np.zeros(3 * d, np.uint16), w_o=np.zeros((d, d), np.uint16),
+                         b_o=np.zeros(d, np.uint16))
+    sh = H.Shape(B=1, H=64, W=64, d=d, T=0, heads=d // 128, mlp=0)
+    out = torch.empty(rows, d, dtype=torch.float32, device="cuda")
+    wsb = H.hilo_block_fp8_workspace_bytes(sh, rows)
+    ws = torch.full((wsb,), 0xFF, dtype=torch.uint8, device="cuda")
+    H.hilo_block_forward_fp8(sh, H.DeviceWeightsFP8.from_host(I.BlockWeights(txt=sw, img=sw)), to_dev_i32([0, rows]),
+                             rows, None, torch.from_numpy(u).cuda() if f32 else H.bf16_from_bits(u),
+                             H.HILO_F32 if f32 else H.HILO_BF16, out, ws, wsb)
+    H.hilo_sync_status()
+    qkv = _ws8(H, sh, rows, ws)[2].float().cpu().numpy().astype(np.float64)
+    codes, scale = O.quantize_rows(O.layer_norm(u.astype(np.float64) if f32 else
+                                                O.bf16_to_f32(u).astype(np.float64)).astype(np.float32))
+    ref = O.e4m3_decode(codes) * scale[:, None].astype(np.float64)
+    for part in np.split(qkv, 3, axis=1):
+        err = np.abs(part - ref)
+        assert np.all(err <= (2.0 ** -3 + 2.0 ** -8) * np.abs(ref) + 2.0 ** -9 * scale[:, None] * 1.01)
+        assert np.mean(err > 2.0 ** -7 * np.abs(ref)) <= 1e-3  # another code (bf16 rounding is 2^-9)
