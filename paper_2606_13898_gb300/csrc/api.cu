@@ -282,7 +282,7 @@ static int split_common(const char* name, const hilo_shape* shape, const float* 
                                      out->labels, out->row_src, out->counts, out->cu_img,
                                      out->tok_row, shape->B, shape->H, shape->W, shape->levels, granular,
                                      shape->lf, static_cast<cudaStream_t>(stream));
-  if (e == cudaSuccess) count(shape->B <= 8 ? 1 : 2);  // up to 8 images: the select kernel also compacts
+  if (e == cudaSuccess) count(shape->B <= hilo::SPLIT_CLUSTER ? 1 : 2);  // the select kernel of a cluster also compacts
   return e == cudaSuccess ? HILO_OK : cuda_fail(e, name);
 }
 

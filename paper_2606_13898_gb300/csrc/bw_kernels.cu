@@ -126,7 +126,6 @@ __global__ void __launch_bounds__(SCORE_THREADS, ITERS == 3 ? 7 : ITERS == 2 ? 8
 // ============================================================== split =====
 
 constexpr int SPLIT_THREADS = 1024;
-constexpr int SPLIT_CLUSTER = 8;  // images whose row offsets one cluster of CTAs finds
 
 // Exclusive scan of one int per thread over a 1024-thread block.
 __device__ __forceinline__ int block_excl_scan(int v, int* warp_tot, int* total) {
@@ -436,7 +435,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_select_kernel(
       return;
     }
   }
-  uint8_t* lab = smem_raw;  // the labels, padded to the threads' tokens
+  uint8_t* lab = smem_raw;  // the labels, N bytes
   const long long base = static_cast<long long>(b) * N;
   const int k = min(max(k_keep[b], 0), N);
   const int km = levels == 2 ? min(max(k_mid[b], 0), N) : 0;

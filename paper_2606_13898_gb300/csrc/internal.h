@@ -34,6 +34,8 @@ struct PerDevice {
 // ---- bandwidth kernels (bw_kernels.cu)
 cudaError_t launch_score(const void* x, float* s, int B, int H, int W, int d, int num_sms,
                          cudaStream_t st);
+// Images whose row offsets one cluster of CTAs finds, in one kernel; more take two.
+constexpr int SPLIT_CLUSTER = 8;
 cudaError_t launch_split(const float* score, const uint8_t* mask, const int32_t* k_keep,
                          const int32_t* k_mid, uint8_t* labels, int32_t* row_src, int32_t* counts,
                          int32_t* cu_img, int32_t* tok_row, int B, int H, int W, int levels,

@@ -3,8 +3,8 @@ oracle: the kept tokens followed by every lf x lf window mean of the grid
 (Sec. 2.3's downsampled-image tokens in token space).
 
 Labels, offsets, row sources, the token -> row map, packed rows, row sizes
-and the delta-unpooled grid match bit for bit, for one image (one kernel)
-and batches (two kernels), lf = 2, 4, 8, including every token kept (the
+and the delta-unpooled grid match bit for bit, for one image
+and batches, lf = 2, 4, 8, including every token kept (the
 largest row count, N + N/lf^2 per image) and nothing kept. The hot path in
 this mode is checked at the 32 x 32 layer within the block tolerance, and a
 block called with more image rows than its capacity computes the clamped

@@ -2,8 +2,7 @@
 oracle (Sec. 2.3's coherent, region-level selection read in token space).
 
 Labels, offsets, row sources and the token -> row map must match bit for
-bit, for one image (the single-kernel path) and for batches (two kernels),
-with one and two pooling levels; packed rows and the delta-unpooled grid are
+bit, for one image and for batches, with one and two pooling levels; packed rows and the delta-unpooled grid are
 bit-exact as well (fp32 subtract then add on both sides). The whole hot path
 in this mode is then checked at the 32 x 32 layer: index sets and packed
 rows exactly, block output and unpooled grid within the block tolerance.

@@ -4,7 +4,8 @@ The objects of the library are linked with a stand-in for the CUDA runtime that
 has two devices of different size: SM counts, and CTA pairs that fit at once,
 which also differ between the bf16 and the e4m3 GEMM. A program runs blocks on
 both devices, then on eight threads that change devices, and checks the grid of
-every GEMM launch against its own device and kernel. Nothing touches a GPU.
+every GEMM launch against its own device and kernel, and the library's count of
+its launches, splits of one to many images among them. Nothing touches a GPU.
 """
 import os
 import shutil
@@ -31,7 +32,7 @@ PROGRAM = r"""
 static thread_local int g_dev = 0;
 static const int SMS[2] = {152, 120};
 static std::map<const void*, std::string> g_names;  // host stub -> mangled kernel name
-static std::atomic<int> g_bad{0}, g_gemms{0};
+static std::atomic<int> g_bad{0}, g_gemms{0}, g_launches{0};
 
 static bool is_gemm(const void* f, bool* fp8) {
   auto it = g_names.find(f);
@@ -90,6 +91,7 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaun
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
   bool fp8;
+  ++g_launches;
   if (is_gemm(f, &fp8)) {
     ++g_gemms;
     if (static_cast<int>(c->gridDim.x) != 2 * pairs(g_dev, fp8)) {
@@ -114,11 +116,19 @@ static int block(bool fp8) {
                                   reinterpret_cast<float*>(mem), mem, big, nullptr);
 }
 
+static int split(int B) {
+  static char mem[64] __attribute__((aligned(256)));
+  hilo_shape s = {B, 8, 8, 1024, 0, 8, 1, 1, 0};
+  int* p = reinterpret_cast<int*>(mem);
+  hilo_split_out o = {reinterpret_cast<uint8_t*>(mem), p, p, p, p};
+  return hilo_split(&s, reinterpret_cast<float*>(mem), reinterpret_cast<uint8_t*>(mem), p, p, &o, nullptr, 0, nullptr);
+}
+
 int main(int argc, char** argv) {
   auto run = [](int first, int n) {
     for (int i = 0; i < n; ++i) {
       g_dev = (first + i / 2) % 2;
-      const int rc = block((first + i) % 2);
+      const int rc = block((first + i) % 2) | split(1 + i);
       if (rc != HILO_OK) {
         printf("block: %d (%s)\n", rc, hilo_last_error());
         ++g_bad;
@@ -131,7 +141,11 @@ int main(int argc, char** argv) {
     for (int t = 0; t < 8; ++t) ts.emplace_back(run, t, 40);
     for (auto& t : ts) t.join();
   } else {
-    run(0, 8);
+    run(0, 20);
+  }
+  if (hilo_launch_count() != static_cast<unsigned long long>(g_launches)) {
+    printf("hilo_launch_count %llu of %d launches\n", hilo_launch_count(), g_launches.load());
+    ++g_bad;
   }
   printf("%d GEMM launches, %d bad\n", g_gemms.load(), g_bad.load());
   return g_bad || !g_gemms;
