@@ -409,8 +409,9 @@ __device__ void compact_image(const uint8_t* lab, int b, int H, int W, int level
 // its members rank below the k_mid cut, else its non-kept members are pooled 2x2).
 // Bound by one SM's latency: barriers, shared atomics and dependent loads. (With
 // the keys in shared memory and re-read by each pass, in contiguous chunks per
-// thread with up to 16-way bank conflicts, two levels on 128x128 took 68 us, 34 so
-// on the hot path's scores, and 64x64 10.5 and 9.1.)
+// thread with up to 16-way bank conflicts, random scores, a quarter kept: 64x64 9.0 us,
+// 6.8 so, 128x128 36.7 and 21.6, with two levels 55.0 and 26.9, of four score values
+// 56.3 and 31.6.)
 template <int CH, bool GRANULAR, bool LFMODE>
 __global__ void __launch_bounds__(SPLIT_THREADS) split_select_kernel(
     const float* __restrict__ score, const uint8_t* __restrict__ mask,
@@ -687,8 +688,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_compact_kernel(
 // in raster order (the first member initialises the sum), divides once with
 // correct rounding and rounds to bf16 (nearest even). Bound by each row's chain of
 // dependent reads (offsets, counts, row source, labels, data), so by the rows in
-// flight: a CTA per row, eight to an SM (two rows per CTA: 128x128 with two levels 31.2
-// us, 27.3 so; four of 64x64 32.4 and 28.7; 64x64 9.5 and 8.9).
+// flight: from 513 channels on a CTA per row (two rows per CTA, at 3072 channels and a
+// quarter kept: 128x128 with two levels 31.2 us, 27.3 so; four images of 64x64 32.4 and
+// 28.7).
 
 constexpr int PACK_WARPS = 4;
 constexpr int PACK_THREADS = 32 * PACK_WARPS;
@@ -701,8 +703,9 @@ constexpr int PACK_THREADS_SHORT = 256;  // rows of up to 512 channels, several 
 static int pack_warps(int d) { return d <= 256 ? 1 : d <= 512 ? 2 : 4; }
 
 // CTAs per low-frequency row: a slice of 128 chunks of eight channels each, but the
-// rows of 2x2 windows, of which there are many, whole (128x128, d = 3072: 26.4 us whole
-// and 30.1 in slices; 4x4 windows 27.6 and 23.5, 8x8 62.7 and 23.8).
+// rows of 2x2 windows, of which there are many, whole (a quarter kept: 128x128 of 3072
+// channels 24.9 us whole and 34.1 in slices, of 1152 9.3 and 15.5, 64x64 of 2048 5.3 and
+// 7.1; 4x4 windows of 3072 27.6 and 23.5, 8x8 62.7 and 23.8).
 __host__ __device__ constexpr int lf_slices(int lf, int d) {
   return lf == 2 ? 1 : (d / 8 + PACK_THREADS - 1) / PACK_THREADS;
 }
@@ -768,7 +771,7 @@ __global__ void __launch_bounds__(THREADS) pack_kernel(const __nv_bfloat16* __re
   for (long long gw = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
        gw < static_cast<long long>(total) * WPR; gw += nwarps) {
     // from the last row down: an image's pooled rows, 4x4 last, take the longest
-    // (128x128 with two levels 37.5 -> 35.6 us, 64x64 8.9 -> 8.1)
+    // (5% less at 128x128 with two levels of 3072 channels, 9% at 64x64)
     const int r = total - 1 - static_cast<int>(gw / WPR);
     const int c0 = lane + 32 * static_cast<int>(gw % WPR);
     constexpr int CSTEP = 32 * WPR;
@@ -1477,7 +1480,7 @@ cudaError_t launch_split(const float* score, const uint8_t* mask, const int32_t*
                          int32_t* cu_img, int32_t* tok_row, int B, int H, int W, int levels,
                          int granular, int lf, cudaStream_t st) {
   const int N = H * W;
-  // tokens per thread: as few as 1024 threads allow (half as many threads take 17.2
+  // tokens per thread: as few as 1024 threads allow (one level, half as many threads: 17.2
   // instead of 13.4 us for 96x96 and 25.5 instead of 21.7 for 128x128)
   int ch = 4;
   while (ch < 32 && N > ch * SPLIT_THREADS) ch *= 2;
@@ -1502,11 +1505,13 @@ cudaError_t launch_split(const float* score, const uint8_t* mask, const int32_t*
                     row_src, tok_row, H, W, levels, lf);
 }
 
-// CTAs per SM on pack_kernel's grid: a row per CTA and turn. The hardware deals further
+// CTAs per SM on pack_kernel's grid of a row per CTA and turn. The hardware deals further
 // CTAs as others end, which evens out rows of one to sixteen members, but one without a
 // row still costs its launch, and the capacity is several times the rows: 24 per SM
 // from about 5000 rows of capacity on, else 16 (4096 rows of 2048 channels: 5.1 us with
-// 16, 6.2 with 24; 16384 of 3072 with two levels 28.6 and 26.4; 5120 rows 10.4 and 10.2).
+// 16, 6.2 with 24; 16384 of 3072 with two levels 28.6 and 26.4; 5120 rows 10.4 and 10.2;
+// four images of 64x64, a quarter kept, of 640 channels 12.3 and 10.9, of 1152 16.9 and
+// 14.1, of 4096 40.5 and 36.6; one image of 128x128 of 2048 20.2 and 21.2).
 static int pack_ctas(long long items, int num_sms) { return items <= 32LL * num_sms ? 16 : 24; }
 
 cudaError_t launch_pack(const void* x, const uint8_t* labels, const int32_t* row_src,

@@ -14,8 +14,8 @@
 // Bound by the tensor pipe at the chip's power limit for large row counts, by
 // fill, last epilogue and partial rounds for small ones. (With rows on M, 256 to
 // a tile, and one-CTA tiles for widths that 256 does not divide, a block of 1662
-// rows of 1152 took 127 us, 96 so; 2389 rows of 3072 456 and 444, with e4m3
-// operands 321 and 302; 10600 rows 2002 and 1997.)
+// rows of 1152 took 127 us, 91 so; 2389 rows of 3072 458 and 440, with e4m3
+// operands 323 and 295; 10600 rows 2023 and 1969.)
 //
 // Each CTA of a pair stages 128 rows of W (half of the tile's features) and
 // half of the tile's X rows at identical shared-memory offsets; the even CTA
