@@ -1533,8 +1533,11 @@ cudaError_t launch_pack(const void* x, const uint8_t* labels, const int32_t* row
                               : wpr == 1 ? pack_lf_kernel<2, 1, PACK_THREADS_SHORT>
                                          : pack_lf_kernel<2, 2, PACK_THREADS_SHORT>);
     const long long items = cap + (lf > 2 ? static_cast<long long>(B) * (H / lf) * (W / lf) * lf_slices(lf, d) : 0);
-    // (24 per SM at every size: 8x8 windows of 64x64 tokens of 3072 channels 12.3 us, 12.7 with 16)
-    const int ctas = few ? 8 : lf > 2 ? 24 : pack_ctas(cap, num_sms);
+    // 24 CTAs per SM, but 16 where that many hold most of the rows and the rows are short
+    // (64x64 tokens, 2x2 windows, a quarter kept: of 1152 channels 5.2 us with 24, 3.8 so, of
+    // 2048 5.3 and 4.2, none kept of 3072 4.7 and 6.1; 4x4 windows of 1024 4.3 and 3.3, of 2048
+    // 4.6 and 4.9; 8x8 of 3072, four images, 12.3 and 12.7)
+    const int ctas = few ? 8 : items <= 40LL * num_sms && d <= (lf == 2 ? 2048 : 1152) ? 16 : 24;
     return launch_pdl(kern, dim3(grid_for(items, few ? rows : 1, num_sms, ctas)),
                       dim3(few ? PACK_THREADS_SHORT : PACK_THREADS), 0, st, xs, row_src, counts, cu_img, ps, B, H, W, d,
                       cap);
